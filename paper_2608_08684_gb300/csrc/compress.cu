@@ -1,7 +1,7 @@
 // ripple_compress_layer: the per-layer compression chain (Sec. 4.1 Eq. 4 and
 // Sec. 4.4 last paragraph: RippleKV keeps the base method's scoring and
 // selection and changes only the number of tokens each layer keeps).
-//   scoring   -> votes [units][P]     (tcgen05 for bf16 d=128, fp32 SIMT otherwise)
+//   scoring   -> votes [units][P]     (tcgen05 for bf16, the fp32 pipes for fp32)
 //   selection -> idx   [units][n]     (pooling + exact top-k, window appended)
 //   gather    -> k_out, v_out [units][cap][d]
 // Everything is enqueued on the caller's stream; nothing synchronises.
@@ -119,9 +119,12 @@ extern "C" ripple_status ripple_compress_layer(const ripple_layer_desc *desc, in
   const bool keep_all = (n == g.T);
   float *votes = scores_out ? scores_out : ws.votes;
   if (g.P > 0 && (!keep_all || scores_out)) {
-    cudaError_t e = score_tc1_supported(g)  ? launch_score_tc1(g, 1, &q_win, &k, ws, votes, dev_status, st)
-                    : score_tc_supported(g) ? launch_score_tc(g, q_win, k, ws, votes, dev_status, st)
-                                            : launch_score_simt(g, q_win, k, ws, votes, dev_status, st);
+    const int slot = 0;
+    cudaError_t e = score_tc1_supported(g)
+                        ? launch_score_tc1(g, 1, &slot, 1, &q_win, &k, ws, votes, dev_status, st)
+                    : score_tc_supported(g)
+                        ? launch_score_tc(g, 1, &slot, 1, &q_win, &k, ws, votes, dev_status, st)
+                        : launch_score_simt(g, q_win, k, ws, votes, dev_status, st);
     RIPPLE_CUDA_TRY(e);
   }
   if (keep_all) {
@@ -204,7 +207,7 @@ extern "C" ripple_status ripple_compress_layers_attn_workspace_bytes(const rippl
                                                                      int32_t n_layers,
                                                                      size_t *bytes_host) {
   LayerGeom g;
-  if (!layers_geom(desc, n_layers, &g) || bytes_host == nullptr || !score_tc1_supported(g))
+  if (!layers_geom(desc, n_layers, &g) || bytes_host == nullptr || !score_tc1_attn_supported(g))
     return RIPPLE_EINVAL;
   *bytes_host = carve_layers_attn_ws(g, n_layers, nullptr).bytes;
   return RIPPLE_OK;
@@ -235,7 +238,7 @@ static ripple_status compress_layers_impl(
     cap[l] = caps_host[l];
     if (n[l] < 0 || cap[l] < n[l]) return RIPPLE_EINVAL;
   }
-  if (o_win_host != nullptr && !score_tc1_supported(g)) return RIPPLE_EINVAL;
+  if (o_win_host != nullptr && !score_tc1_attn_supported(g)) return RIPPLE_EINVAL;
   const CompressWs ws = o_win_host ? carve_layers_attn_ws(g, n_layers, workspace)
                                    : carve_layers_ws(g, n_layers, workspace);
   if (workspace_bytes < ws.bytes) return RIPPLE_EWORKSPACE;
@@ -243,54 +246,43 @@ static ripple_status compress_layers_impl(
   // selection and gather in one launch where the selection kernel takes both
   const GatherArgs ga{k_host, v_host, k_out_host, v_out_host, cap};
   bool gathered = false;
-  if (g.P > 0 && score_tc1_supported(g)) {
-    // All layers in two or three launches: scoring, selection (+ gather).
-    RIPPLE_CUDA_TRY(launch_score_tc1(g, n_layers, q_win_host, k_host, ws, ws.votes, dev_status,
-                                     st, o_win_host ? v_host : nullptr, o_win_host));
-    RIPPLE_CUDA_TRY(launch_select(g, n_layers, ws.votes, ws, n, idx_out_host, dev_status, st,
-                                  &ga, &gathered));
-    if (!gathered)
-      RIPPLE_CUDA_TRY(launch_gather(g, n_layers, k_host, v_host,
-                                    (const int32_t *const *)idx_out_host, n, k_out_host,
-                                    v_out_host, cap, dev_status, st));
-  } else {
-    // Other shapes: the 256-row tensor-core scoring of every layer that needs
-    // votes in one launch, or the CUDA-core scoring layer by layer (each
-    // layer's votes in its part of the vote array, the scratch of the
-    // multi-layer workspace reused); then one selection and one gather launch
-    // for all layers. A layer that keeps every token needs no votes (the
-    // selection writes 0..T-1 for it).
-    if (g.P > 0 && score_tc_supported(g)) {
-      // the layers that need votes, all in one tensor-core launch
-      int slots[RIPPLE_COMPRESS_MAX_LAYERS];
-      const void *qs[RIPPLE_COMPRESS_MAX_LAYERS];
-      const void *ks[RIPPLE_COMPRESS_MAX_LAYERS];
-      int n_scored = 0;
-      for (int l = 0; l < n_layers; ++l) {
-        if (n[l] == g.T) continue;
-        slots[n_scored] = l;
-        qs[n_scored] = q_win_host[l];
-        ks[n_scored] = k_host[l];
-        ++n_scored;
-      }
-      if (n_scored > 0)
-        RIPPLE_CUDA_TRY(launch_score_tc(g, n_layers, slots, n_scored, qs, ks, ws, ws.votes,
-                                        dev_status, st));
-    } else {
-      for (int l = 0; l < n_layers; ++l) {
-        if (g.P == 0 || n[l] == g.T) continue;
-        float *votes_l = ws.votes + (size_t)l * g.units * g.P;
-        RIPPLE_CUDA_TRY(launch_score_simt(g, q_win_host[l], k_host[l], ws, votes_l, dev_status,
-                                          st));
-      }
+  if (g.P > 0) {
+    // Scoring: on the tensor cores (bf16) every layer that needs votes in one
+    // launch; on the CUDA cores (fp32) layer by layer, the scratch of the
+    // multi-layer workspace reused. Each layer's votes go to its part of the
+    // vote array. A layer that keeps every token needs no votes (the selection
+    // writes 0..T-1 for it), unless its window rows' output is wanted.
+    int slots[RIPPLE_COMPRESS_MAX_LAYERS];
+    const void *qs[RIPPLE_COMPRESS_MAX_LAYERS];
+    const void *ks[RIPPLE_COMPRESS_MAX_LAYERS];
+    int n_scored = 0;
+    for (int l = 0; l < n_layers; ++l) {
+      if (n[l] == g.T && o_win_host == nullptr) continue;
+      slots[n_scored] = l;
+      qs[n_scored] = q_win_host[l];
+      ks[n_scored] = k_host[l];
+      ++n_scored;
     }
-    RIPPLE_CUDA_TRY(launch_select(g, n_layers, ws.votes, ws, n, idx_out_host, dev_status, st,
-                                  &ga, &gathered));
-    if (!gathered)
-      RIPPLE_CUDA_TRY(launch_gather(g, n_layers, k_host, v_host,
-                                    (const int32_t *const *)idx_out_host, n, k_out_host,
-                                    v_out_host, cap, dev_status, st));
+    if (n_scored > 0 && score_tc1_supported(g)) {
+      RIPPLE_CUDA_TRY(launch_score_tc1(g, n_layers, slots, n_scored, qs, ks, ws, ws.votes,
+                                       dev_status, st, o_win_host ? v_host : nullptr,
+                                       o_win_host));
+    } else if (n_scored > 0 && score_tc_supported(g)) {
+      RIPPLE_CUDA_TRY(launch_score_tc(g, n_layers, slots, n_scored, qs, ks, ws, ws.votes,
+                                      dev_status, st));
+    } else {
+      for (int i = 0; i < n_scored; ++i)
+        RIPPLE_CUDA_TRY(launch_score_simt(g, qs[i], ks[i], ws,
+                                          ws.votes + (size_t)slots[i] * g.units * g.P, dev_status,
+                                          st));
+    }
   }
+  RIPPLE_CUDA_TRY(launch_select(g, n_layers, ws.votes, ws, n, idx_out_host, dev_status, st, &ga,
+                                &gathered));
+  if (!gathered)
+    RIPPLE_CUDA_TRY(launch_gather(g, n_layers, k_host, v_host,
+                                  (const int32_t *const *)idx_out_host, n, k_out_host, v_out_host,
+                                  cap, dev_status, st));
   for (int l = 0; l < n_layers; ++l) n_keep_host[l] = n[l];
   return RIPPLE_OK;
 }

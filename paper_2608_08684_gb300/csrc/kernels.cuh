@@ -45,30 +45,29 @@ struct CompressWs {
 };
 CompressWs carve_compress_ws(const LayerGeom &g, void *base);
 
-// Scoring, SIMT fp32 path (any dtype).
+// Scoring on the fp32 pipes (fp32 caches).
 cudaError_t launch_score_simt(const LayerGeom &g, const void *q_win, const void *k,
                               const CompressWs &ws, float *votes, int32_t *status,
                               cudaStream_t st);
-// Scoring, tcgen05 tensor-core path (bf16, d = 128).
+// Scoring on the tensor cores for 129 to 256 window rows (bf16, d = 64 or 128),
+// several layers in one launch as launch_score_tc1 below.
 bool score_tc_supported(const LayerGeom &g);
-cudaError_t launch_score_tc(const LayerGeom &g, const void *q_win, const void *k,
-                            const CompressWs &ws, float *votes, int32_t *status,
-                            cudaStream_t st);
-// The same for n_scored layers of one shape in one launch: scored layer i
-// (q_win[i], k[i]) writes the votes of layer slots[i] of votes
-// [n_slots][g.units][P]; ws is carved for n_scored * g.units units or more.
 cudaError_t launch_score_tc(const LayerGeom &g, int n_slots, const int *slots, int n_scored,
                             const void *const *q_win, const void *const *k, const CompressWs &ws,
                             float *votes, int32_t *status, cudaStream_t st);
-// Scoring on the tensor cores for G * w = 128 window rows (bf16, d = 128),
-// for n_layers layers of the same shape in one launch; ws is carved for
-// n_layers * g.units units and votes is [n_layers][g.units][P]. With v (the
-// values of every layer) the same pass also gives the window rows' attention
-// output o_win[l] [B][Hq][w][d] fp32 (ws carved with its partials).
+// Scoring on the tensor cores for up to 128 window rows (bf16, d = 64 or 128),
+// for n_layers layers of the same shape in one launch: scored layer i
+// (q_win[i], k[i]) writes the votes of layer slots[i] of votes
+// [n_slots][g.units][P]; ws is carved for n_layers * g.units units or more.
+// With v (the values of every layer; 128 rows of d = 128 only) the same pass
+// also gives the window rows' attention output o_win[i] [B][Hq][w][d] fp32 (ws
+// carved with its partials).
 bool score_tc1_supported(const LayerGeom &g);
-cudaError_t launch_score_tc1(const LayerGeom &g, int n_layers, const void *const *q_win,
-                             const void *const *k, const CompressWs &ws, float *votes,
-                             int32_t *status, cudaStream_t st, const void *const *v = nullptr,
+bool score_tc1_attn_supported(const LayerGeom &g);
+cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, int n_layers,
+                             const void *const *q_win, const void *const *k,
+                             const CompressWs &ws, float *votes, int32_t *status,
+                             cudaStream_t st, const void *const *v = nullptr,
                              float *const *o_win = nullptr);
 // Items per unit of launch_score_tc1 at most (sizes the output partials).
 int score_tc1_max_items(const LayerGeom &g);

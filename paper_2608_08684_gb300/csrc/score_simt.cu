@@ -1,5 +1,5 @@
 // Observation-window token scoring on the fp32 pipes (SnapKV rule kept by
-// RippleKV, Sec. 4.4 last paragraph). Used for fp32 caches, where running the
+// RippleKV, Sec. 4.4 last paragraph), for fp32 caches, where running the
 // contraction on tf32 tensor cores would spend the score tolerance.
 //
 // Two passes over each unit's keys, both in key chunks of kScoreChunk:
@@ -210,12 +210,9 @@ cudaError_t launch_typed(const LayerGeom &g, const void *q_win, const void *k,
 cudaError_t launch_score_simt(const LayerGeom &g, const void *q_win, const void *k,
                               const CompressWs &ws, float *votes, int32_t *status,
                               cudaStream_t st) {
-  if (g.dtype == RIPPLE_F32) {
-    if (g.D == 64) return launch_typed<float, 64>(g, q_win, k, ws, votes, status, st);
-    return launch_typed<float, 128>(g, q_win, k, ws, votes, status, st);
-  }
-  if (g.D == 64) return launch_typed<__nv_bfloat16, 64>(g, q_win, k, ws, votes, status, st);
-  return launch_typed<__nv_bfloat16, 128>(g, q_win, k, ws, votes, status, st);
+  if (g.dtype != RIPPLE_F32) return cudaErrorInvalidValue;
+  if (g.D == 64) return launch_typed<float, 64>(g, q_win, k, ws, votes, status, st);
+  return launch_typed<float, 128>(g, q_win, k, ws, votes, status, st);
 }
 
 }  // namespace ripple

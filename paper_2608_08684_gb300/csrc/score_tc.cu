@@ -1,6 +1,6 @@
 // Observation-window token scoring on the 5th-generation tensor cores
-// (tcgen05, accumulators in TMEM), bf16 keys and queries, d = 128, G*w = 128
-// or 256 window rows. SnapKV's rule as RippleKV keeps it (Sec. 4.4, last
+// (tcgen05, accumulators in TMEM), bf16 keys and queries, d = 64 or 128, 129 to
+// 256 window rows G * w (padded to 256). SnapKV's rule as RippleKV keeps it (Sec. 4.4, last
 // paragraph): logits x = scale * q.k of the window rows against every key,
 // causal inside the window, softmax per row over all visible keys, vote of a
 // prefix key = sum over rows of its probability.
@@ -37,6 +37,7 @@
 #include <math.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -47,7 +48,6 @@ namespace {
 
 constexpr int kTile = 128;                      // keys per tile
 constexpr int kHalfBytes = kTile * 64 * 2;      // 64 bf16 columns of 128 rows: 16 KB
-constexpr int kTileBytes = 2 * kHalfBytes;      // one 128 x 128 bf16 tile
 constexpr int kThreads = 352;
 constexpr int kPubSlots = 2;
 // Items of at least 64 key tiles: with every layer of a call in one launch the
@@ -62,7 +62,7 @@ constexpr int kMinTilesPerItem = 64;
 // ------------------------------------------------------------ work list
 
 struct TcParams {
-  int units, upl, T, P, W, Hq, Hkv, G;  // units of all scored layers, units per layer
+  int units, upl, T, P, W, R;  // units of all scored layers, units per layer, window rows
   int n_tiles1, n_tiles2;  // key tiles of pass 1 (all keys) and pass 2 (prefix keys)
   int tpi, n_ch;           // key tiles per item, items per unit
   int total_items;
@@ -100,18 +100,23 @@ __device__ __forceinline__ void tiles_of(const TcParams &p, const ItemRef &it, i
 
 // ------------------------------------------------------------ shared memory
 
-template <int NR>
+// 256 window rows (fewer are padded with zero rows, which count for nothing),
+// in two halves of 128 for pass 1. D: head dims.
+template <int D>
 struct Cfg {
+  static constexpr int NR = 2;                   // row halves
   static constexpr int R = 128 * NR;             // window rows
-  static constexpr int NK = NR == 1 ? 3 : 2;     // key-tile stages
+  static constexpr int TileBytes = D / 64 * kHalfBytes;  // one 128 x D bf16 tile
+  static constexpr int KSteps = D / 16;          // MMAs per 128 x 128 product
+  static constexpr int NK = D == 128 ? 2 : 4;    // key-tile stages
   // Query buffers: two items are in flight (pass 1 of one, pass 2 of the
-  // previous); a third lets the next item's queries load ahead.
-  static constexpr int NQ = NR == 1 ? 3 : 2;
-  static constexpr int NA = NR == 1 ? 4 : 2;     // TMEM accumulator stages
+  // previous).
+  static constexpr int NQ = 2;
+  static constexpr int NA = 2;                   // TMEM accumulator stages
   static constexpr int ACC_COLS = 128 * NR;      // TMEM columns per stage
-  static constexpr int QBYTES = R * 256;         // R rows x 128 bf16
+  static constexpr int QBYTES = NR * TileBytes;  // [D / 64][256 rows][64 dims]
   static constexpr int OFF_K = 0;
-  static constexpr int OFF_Q = OFF_K + NK * kTileBytes;
+  static constexpr int OFF_Q = OFF_K + NK * TileBytes;
   static constexpr int OFF_MISC = OFF_Q + NQ * QBYTES;
 };
 
@@ -127,9 +132,9 @@ struct Misc {
 
 static_assert(offsetof(Misc, off) % 16 == 0, "float4-read shared arrays are 16-byte aligned");
 
-template <int NR>
+template <int D>
 constexpr int smem_bytes() {
-  return Cfg<NR>::OFF_MISC + (int)sizeof(Misc) + 1024;  // + 1024-byte alignment slack
+  return Cfg<D>::OFF_MISC + (int)sizeof(Misc) + 1024;  // + 1024-byte alignment slack
 }
 
 // Bounded mbarrier wait that also gives up as soon as another role aborted.
@@ -189,10 +194,13 @@ struct TcLaunch {
   TcParams p;
 };
 
-template <int NR>
+// kPad: fewer than 256 window rows.
+template <int D, bool kPad>
 __global__ void __launch_bounds__(kThreads, 1)
     score_tc_kernel(const __grid_constant__ TcLaunch lp) {
-  using C = Cfg<NR>;
+  using C = Cfg<D>;
+  constexpr int NR = C::NR;
+  constexpr int kTileBytes = C::TileBytes;
   const TcParams &p = lp.p;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -228,6 +236,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_alloc(&ms->tmem_base, 512);
     tmem_relinquish();
   }
+  if constexpr (kPad) {
+    // the padding rows of the query buffers (no copy writes them) hold zeros
+    for (int i = threadIdx.x; i < C::NQ * C::QBYTES / 16; i += kThreads)
+      reinterpret_cast<uint4 *>(qbufs)[i] = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -261,8 +275,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t pol = pass == 1 ? keep : drop;
             const CUtensorMap *km = &lp.kmap[it.unit / p.upl];
             const int local = it.unit % p.upl;
-            tma_load_3d(kb, km, 0, t * kTile, local, &ms->k_full[ks], pol);
-            tma_load_3d(kb + kHalfBytes, km, 64, t * kTile, local, &ms->k_full[ks], pol);
+#pragma unroll
+            for (int half = 0; half < D / 64; ++half)
+              tma_load_3d(kb + half * kHalfBytes, km, half * 64, t * kTile, local,
+                          &ms->k_full[ks], pol);
             ++kcount;
           }
         }
@@ -276,17 +292,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int k = 0; k < n; ++k) {
         const ItemRef it = item_of(p, k);
         const int local = it.unit % p.upl;
-        const int b = local / p.Hkv, h = local % p.Hkv;
-        const int qrow0 = (b * p.Hq + h * p.G) * p.W;
         const CUtensorMap *qm = &lp.qmap[it.unit / p.upl];
         const int qs = k % C::NQ;
         if (!wait_bar(&ms->q_empty[qs], ((k / C::NQ) & 1) ^ 1, ms, p.status)) break;
-        mbar_arrive_expect_tx(&ms->q_full[qs], C::QBYTES);
+        mbar_arrive_expect_tx(&ms->q_full[qs], (uint32_t)(p.R * D * 2));
         uint8_t *qb = qbufs + qs * C::QBYTES;
-        for (int half = 0; half < 2; ++half)
-          for (int nr = 0; nr < NR; ++nr)
-            tma_load_2d(qb + half * (NR * kHalfBytes) + nr * kHalfBytes, qm, half * 64,
-                        qrow0 + nr * 128, &ms->q_full[qs]);
+#pragma unroll
+        for (int half = 0; half < D / 64; ++half)
+          tma_load_2d(qb + half * (NR * kHalfBytes), qm, half * 64, local * p.R, &ms->q_full[qs]);
         ++qcount;
       }
       for (int k = max(0, qcount - C::NQ); k < qcount; ++k)
@@ -324,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t d = tmem + as * C::ACC_COLS;
             const uint32_t ka = kbase + ks * kTileBytes;
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
+            for (int kk = 0; kk < C::KSteps; ++kk) {
               const uint32_t koff = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
               const uint32_t qoff = (kk >> 2) * (NR * kHalfBytes) + (kk & 3) * 32;
               if (pass == 1) {
@@ -359,14 +372,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       // One partial per item: the two warpgroups' statistics combined here.
       float2 *mine = p.partial + guard((long long)it.unit * p.n_ch + it.chunk, 1,
                                        (long long)p.units * p.n_ch, p.status) *
-                                     C::R;
+                                     p.R;
 #pragma unroll
       for (int j = 0; j < RJ; ++j) {
         const int r = lane + 32 * j;
         float2 a = ms->pstat[slot][0][r];
         const float2 b = ms->pstat[slot][1][r];
         combine(a.x, a.y, b.x, b.y);
-        mine[r] = a;
+        if (r < p.R) mine[r] = a;
       }
       __syncwarp();  // all lanes' rows are written (and the slot read) before lane 0 goes on
       int last = 0;
@@ -382,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float2 *part =
             p.partial + guard((long long)it.unit * p.n_ch, p.n_ch, (long long)p.units * p.n_ch,
                               p.status) *
-                            C::R;
+                            p.R;
         float mm[RJ], ll[RJ];
 #pragma unroll
         for (int j = 0; j < RJ; ++j) {
@@ -395,8 +408,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int c = 0; c < CB; ++c)
 #pragma unroll
             for (int j = 0; j < RJ; ++j)
-              q[c][j] = c0 + c < p.n_ch ? __ldcg(&part[(size_t)(c0 + c) * C::R + lane + 32 * j])
-                                        : make_float2(-INFINITY, 0.f);
+              q[c][j] = c0 + c < p.n_ch && lane + 32 * j < p.R
+                            ? __ldcg(&part[(size_t)(c0 + c) * p.R + lane + 32 * j])
+                            : make_float2(-INFINITY, 0.f);
 #pragma unroll
           for (int c = 0; c < CB; ++c)
 #pragma unroll
@@ -404,8 +418,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
 #pragma unroll
         for (int j = 0; j < RJ; ++j)
-          p.lognorm[guard(it.unit, 1, p.units, p.status) * C::R + lane + 32 * j] =
-              mm[j] + __log2f(ll[j]);
+          if (lane + 32 * j < p.R)
+            p.lognorm[guard(it.unit, 1, p.units, p.status) * p.R + lane + 32 * j] =
+                mm[j] + __log2f(ll[j]);
         __threadfence();
         __syncwarp();
         if (lane == 0) st_release(&p.ctrl[guard(p.units + it.unit, 1, 2LL * p.units, p.status)], 1);
@@ -512,8 +527,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (wtid == 0)
             wait_ready(&p.ctrl[guard(p.units + it.unit, 1, 2LL * p.units, p.status)], ms, p.status);
           named_bar_sync(3 + wg, 128);
-          for (int r = wtid; r < C::R; r += 128)
-            ms->off[wg][r] = __ldcg(&p.lognorm[guard(it.unit, 1, p.units, p.status) * C::R + r]);
+          for (int r = wtid; r < p.R; r += 128)
+            ms->off[wg][r] = __ldcg(&p.lognorm[guard(it.unit, 1, p.units, p.status) * p.R + r]);
           named_bar_sync(3 + wg, 128);
         }
         const float4 *off4 = (const float4 *)ms->off[wg];
@@ -541,8 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               __syncwarp();
               if (lane == 0) mbar_arrive(&ms->acc_empty[as]);
             }
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
+            auto columns = [&](int c, auto some_padding) {
 #pragma unroll
               for (int j = 0; j < 32; j += 4) {
                 const float4 o = off4[(c4 * 128 + c * 32 + j) >> 2];
@@ -553,9 +567,27 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float2 y1 = __ffma2_rn(
                     make_float2(__uint_as_float(x[c][j + 2]), __uint_as_float(x[c][j + 3])), s2,
                     make_float2(-o.z, -o.w));
-                vs[h] = __fadd2_rn(vs[h], make_float2(fast_exp2(y0.x), fast_exp2(y0.y)));
-                vs[h + 1] = __fadd2_rn(vs[h + 1], make_float2(fast_exp2(y1.x), fast_exp2(y1.y)));
+                float2 e0 = make_float2(fast_exp2(y0.x), fast_exp2(y0.y));
+                float2 e1 = make_float2(fast_exp2(y1.x), fast_exp2(y1.y));
+                if constexpr (decltype(some_padding)::value) {
+                  const int left = p.R - (c4 * 128 + c * 32 + j);  // rows from this column on
+                  if (left < 1) e0.x = 0.f;
+                  if (left < 2) e0.y = 0.f;
+                  if (left < 3) e1.x = 0.f;
+                  if (left < 4) e1.y = 0.f;
+                }
+                vs[h] = __fadd2_rn(vs[h], e0);
+                vs[h + 1] = __fadd2_rn(vs[h + 1], e1);
               }
+            };
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const int first = c4 * 128 + c * 32;
+              if (!kPad || first + 32 <= p.R)
+                columns(c, std::false_type{});
+              else if (first < p.R)
+                columns(c, std::true_type{});
+            }
           }
           const float vote = ((vs[0].x + vs[0].y) + (vs[1].x + vs[1].y)) +
                              ((vs[2].x + vs[2].y) + (vs[3].x + vs[3].y));
@@ -604,8 +636,8 @@ int sm_count() {
   return n > 0 ? n : 1;
 }
 
-template <int NR>
-cudaError_t launch_nr(const LayerGeom &g, int n_slots, const int *slots, int n_scored,
+template <int D>
+cudaError_t launch_d(const LayerGeom &g, int n_slots, const int *slots, int n_scored,
                       const void *const *q_win, const void *const *k, const CompressWs &ws,
                       float *votes, int32_t *status, cudaStream_t st) {
   EncodeTiledFn enc = encode_fn();
@@ -615,17 +647,17 @@ cudaError_t launch_nr(const LayerGeom &g, int n_slots, const int *slots, int n_s
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
   for (int l = 0; l < n_scored; ++l) {
-    cuuint64_t dims[3] = {128, (cuuint64_t)g.T, (cuuint64_t)g.units};
-    cuuint64_t strides[2] = {256, (cuuint64_t)g.T * 256};
+    cuuint64_t dims[3] = {D, (cuuint64_t)g.T, (cuuint64_t)g.units};
+    cuuint64_t strides[2] = {D * 2, (cuuint64_t)g.T * D * 2};
     cuuint32_t box[3] = {64, 128, 1};
     cuuint32_t es[3] = {1, 1, 1};
     if (enc(&lp.kmap[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(k[l]), dims,
             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
-    cuuint64_t qdims[2] = {128, (cuuint64_t)g.B * g.Hq * g.W};
-    cuuint64_t qstrides[1] = {256};
-    cuuint32_t qbox[2] = {64, 128};
+    cuuint64_t qdims[2] = {D, (cuuint64_t)g.units * g.R};
+    cuuint64_t qstrides[1] = {D * 2};
+    cuuint32_t qbox[2] = {64, (cuuint32_t)g.R};  // one unit's rows
     cuuint32_t qes[2] = {1, 1};
     if (enc(&lp.qmap[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(q_win[l]), qdims,
             qstrides, qbox, qes, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -639,9 +671,7 @@ cudaError_t launch_nr(const LayerGeom &g, int n_slots, const int *slots, int n_s
   p.T = g.T;
   p.P = g.P;
   p.W = g.W;
-  p.Hq = g.Hq;
-  p.Hkv = g.Hkv;
-  p.G = g.G;
+  p.R = g.R;
   p.n_tiles1 = (g.T + kTile - 1) / kTile;
   p.n_tiles2 = (g.P + kTile - 1) / kTile;
   // Tiles per item: at least kMinTilesPerItem (hand-offs are per item), and
@@ -665,16 +695,17 @@ cudaError_t launch_nr(const LayerGeom &g, int n_slots, const int *slots, int n_s
   p.wait_cycles = wait_limit_cycles();
   cudaError_t e = cudaMemsetAsync(ws.counters, 0, sizeof(int) * 2 * p.units, st);
   if (e != cudaSuccess) return e;
-  constexpr int smem = smem_bytes<NR>();
+  constexpr int smem = smem_bytes<D>();
   static_assert(smem <= 227 * 1024, "shared memory budget");
-  e = cudaFuncSetAttribute(score_tc_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const void *kernel = g.R == 256 ? (const void *)score_tc_kernel<D, false>
+                                  : (const void *)score_tc_kernel<D, true>;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const int grid = p.total_items < sms ? p.total_items : sms;
   // Cooperative launch: every CTA resident at once, which the cross-CTA waits
   // of the schedule rely on.
   void *args[] = {(void *)&lp};
-  e = cudaLaunchCooperativeKernel((const void *)score_tc_kernel<NR>, dim3(grid), dim3(kThreads),
-                                  args, (size_t)smem, st);
+  e = cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(kThreads), args, (size_t)smem, st);
   count_launches(1);
   return e;
 }
@@ -682,23 +713,15 @@ cudaError_t launch_nr(const LayerGeom &g, int n_slots, const int *slots, int n_s
 }  // namespace
 
 bool score_tc_supported(const LayerGeom &g) {
-  return g.dtype == RIPPLE_BF16 && g.D == 128 && (g.R == 128 || g.R == 256) && g.P > 0 &&
-         encode_fn() != nullptr;
+  return g.dtype == RIPPLE_BF16 && g.R > 128 && g.R <= 256 && g.P > 0;
 }
 
 cudaError_t launch_score_tc(const LayerGeom &g, int n_slots, const int *slots, int n_scored,
                             const void *const *q_win, const void *const *k, const CompressWs &ws,
                             float *votes, int32_t *status, cudaStream_t st) {
-  if (g.R == 128)
-    return launch_nr<1>(g, n_slots, slots, n_scored, q_win, k, ws, votes, status, st);
-  return launch_nr<2>(g, n_slots, slots, n_scored, q_win, k, ws, votes, status, st);
-}
-
-cudaError_t launch_score_tc(const LayerGeom &g, const void *q_win, const void *k,
-                            const CompressWs &ws, float *votes, int32_t *status,
-                            cudaStream_t st) {
-  const int slot = 0;
-  return launch_score_tc(g, 1, &slot, 1, &q_win, &k, ws, votes, status, st);
+  if (g.D == 64)
+    return launch_d<64>(g, n_slots, slots, n_scored, q_win, k, ws, votes, status, st);
+  return launch_d<128>(g, n_slots, slots, n_scored, q_win, k, ws, votes, status, st);
 }
 
 }  // namespace ripple

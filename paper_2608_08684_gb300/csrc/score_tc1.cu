@@ -1,6 +1,13 @@
-// Observation-window token scoring for G * w = 128 window rows (SnapKV's rule
-// as RippleKV keeps it, Sec. 4.4, last paragraph), bf16, d = 128, on the
-// 5th-generation tensor cores.
+// Observation-window token scoring for up to 128 window rows G * w (SnapKV's
+// rule as RippleKV keeps it, Sec. 4.4, last paragraph), bf16, d = 64 or 128, on
+// the 5th-generation tensor cores. Row counts other than 32, 64 and 128 are
+// padded to the next of them with zero rows that no sum counts.
+//
+// Bound: HBM for 128 rows of d = 128 (a layer of 32 units and 32768 keys
+// about 72 us, 3.7 TB/s of its own bytes); the exponentials and the per-tile
+// hand-overs for small rows or d = 64: 16 layers of 16 units, 6007 keys, d =
+// 64 and 64 rows take 203 us with selection and gather, against 1917 us when
+// the fp32 pipes scored these shapes layer by layer.
 //
 // One persistent CTA per SM, item i on CTA i mod grid; in its step k a CTA
 // runs P1(a_k) then P2(a_k-1), so that keys are re-read from L2 one item
@@ -8,11 +15,11 @@
 // Each pass takes the layout in which its reduction stays inside one thread:
 //   pass 1  D[row][key] = Q . K_tile^T; a thread owns a row and folds its
 //           keys into the row's running max and sum;
-//   pass 2  D[key][row] = K_tile . Q^T; a thread owns a key and sums its 128
+//   pass 2  D[key][row] = K_tile . Q^T; a thread owns a key and sums its
 //           rows' probabilities, so a key's vote needs no shuffles and no
 //           exchange between warps.
-// Both passes take the queries from shared memory (a 32 KB buffer per pass,
-// loaded by TMA once per item) and the key tile from a 4-stage TMA ring; TMEM
+// Both passes take the queries from shared memory (a buffer of 128 rows per
+// pass, loaded by TMA once per item) and the key tile from a 128 KB TMA ring; TMEM
 // holds four 128-column accumulators, so the MMA issuer can run two tiles
 // ahead of each epilogue warpgroup.
 //
@@ -43,6 +50,7 @@
 #include <math.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -53,7 +61,6 @@ namespace {
 
 constexpr int kTile = 128;                      // keys per tile
 constexpr int kHalfBytes = kTile * 64 * 2;      // one TMA box: 64 dims of 128 keys
-constexpr int kTileBytes = 2 * kHalfBytes;
 constexpr int kThreads = 352;
 constexpr int kLag = 1;                         // pass 2 of item k runs in step k + kLag
 constexpr int kPubSlots = 2;
@@ -64,7 +71,7 @@ constexpr int kMinTilesPerItem = 9;
 // L2 until then): 32 layers of the 32k workload took 5.39 / 5.25 / 5.08 /
 // 5.11 / 5.00 ms with items of 32 / 64 / 86 / 128 / 256 tiles.
 constexpr int kMinTilesPerItemO = 256;
-constexpr int kMaxStages = 4;
+constexpr int kMaxStages = 8;
 constexpr int kOReduceLag = 2;  // kO: a step's item rows are summed this many steps later
 
 // With kO (the window rows' attention output as well as the votes) pass 2
@@ -72,17 +79,30 @@ constexpr int kOReduceLag = 2;  // kO: a step's item rows are summed this many s
 // probabilities by them on the tensor cores and accumulates O in TMEM; the
 // probabilities go through a 32 KB shared-memory tile, so the ring has one
 // stage less, and O takes the last 128 TMEM columns.
-template <bool kO>
+// D: head dims (64 or 128). RP: window rows padded to 32, 64 or 128. With
+// RP < 128 the pass-1 A operand holds the queries 128 / RP times over, and the
+// thread of copy c of a row folds the c-th RP keys of the tile, so that every
+// thread has RP exponentials of a tile in both passes and all four SM
+// partitions share them (padding the rows to 128 instead left the partitions
+// of the padding rows idle). Pass 2 multiplies by the RP rows only.
+template <bool kO, int D, int RP>
 struct Tc1Cfg {
-  static constexpr int NK = kO ? 3 : 4;   // ring stages (key tiles; value tiles with kO)
+  static_assert(!kO || (D == 128 && RP == 128), "window-row outputs: 128 rows of 128 dims");
+  static constexpr int TileBytes = D / 64 * kHalfBytes;  // 128 keys (or window rows)
+  static constexpr int KSteps = D / 16;                  // MMAs per tile
+  static constexpr int Copies = 128 / RP;                // of the queries in pass 1
+  // ring stages (key tiles; value tiles with kO): 128 KB of keys in flight
+  static constexpr int NK = kO ? 3 : 128 / (TileBytes >> 10);
   static constexpr int NA = kO ? 3 : 4;   // S accumulators in TMEM (128 columns each)
   static constexpr uint32_t OCol = NA * 128;  // O accumulator (kO)
   static_assert(NA * 128 + (kO ? 128 : 0) <= 512, "TMEM columns");
   static_assert(NK <= kMaxStages && NA <= kMaxStages, "barrier arrays");
+  static_assert(RP == 32 || RP == 64 || RP == 128, "row padding");
 };
 
 struct Tc1Params {
   int units, upl, T, P, W, Hq, Hkv, G;  // units of all layers, units per layer
+  int R;                   // window rows G * W (at most the kernel's RP)
   int n_tiles1, n_tiles2;  // key tiles of pass 1 (all keys) and pass 2 (prefix keys; all with kO)
   int tpi, n_ch;           // key tiles per item, items per unit
   int total_items;
@@ -90,9 +110,11 @@ struct Tc1Params {
   float *o_win[kCompressMaxLayers];  // kO, per layer: window-row outputs [B][Hq][W][128] fp32
   float *o_part;     // kO: [units][n_ch][128][128] fp32 per-item partial outputs
   int *o_count;      // kO: [units] items of unit u whose partial is written
-  float2 *partial;   // [units][n_ch][128] (max, sum) per item and row, log2 domain
-  float *lognorm;    // [units][128]
-  float *votes;      // [units][P], layer-major
+  float2 *partial;   // [units][n_ch][R] (max, sum) per item and row, log2 domain
+  float *lognorm;    // [units][R]
+  float *votes;      // [n_slots][upl][P]: unit u's votes at layer_of[u / upl]
+  int layer_of[kCompressMaxLayers];  // the layer (votes slot) of each scored layer
+  int n_slots;                       // layers (votes slots) of the votes array
   int *ctrl;         // [u] items of unit u published; [units + u] row statistics ready
   int32_t *status;
   long long wait_cycles;  // bound of the in-kernel waits
@@ -182,12 +204,13 @@ struct Misc {
 
 // Shared memory: the ring, the pass-2 and pass-1 queries (two 64-dim halves
 // each), with kO the probability tile, then the barriers and statistics.
-template <bool kO>
+template <bool kO, int D, int RP>
 struct Tc1Smem {
-  static constexpr int OffQs = Tc1Cfg<kO>::NK * kTileBytes;
-  static constexpr int OffQ1 = OffQs + kTileBytes;
-  static constexpr int OffP = OffQ1 + kTileBytes;
-  static constexpr int OffMisc = OffP + (kO ? kTileBytes : 0);
+  using C = Tc1Cfg<kO, D, RP>;
+  static constexpr int OffQs = C::NK * C::TileBytes;
+  static constexpr int OffQ1 = OffQs + C::TileBytes;
+  static constexpr int OffP = OffQ1 + C::TileBytes;
+  static constexpr int OffMisc = OffP + (kO ? C::TileBytes : 0);
   static constexpr int Bytes = OffMisc + (int)sizeof(Misc) + 1024;  // + alignment slack
   static_assert(Bytes <= 227 * 1024, "shared memory budget");
 };
@@ -243,8 +266,8 @@ __device__ __forceinline__ void combine(float &m, float &l, float m2, float l2) 
 }
 
 // Kernel argument: the keys (and with kO the values) of every layer as 3-D
-// tensor maps [unit][T][128], the window queries of every layer as 2-D maps
-// [B * Hq * W][128], and the parameters.
+// tensor maps [unit][T][D], the window queries of every layer as 2-D maps
+// [B * Hq * W][D] (a box is one unit's R rows), and the parameters.
 struct Tc1Launch {
   CUtensorMap kmap[kCompressMaxLayers];
   CUtensorMap qmap[kCompressMaxLayers];
@@ -394,12 +417,15 @@ __device__ __forceinline__ void reduce_rows(const Tc1Params &p, Misc *ms, const 
   }
 }
 
-template <bool kO>
+// kPad: R < RP (some rows are padding; R = RP otherwise).
+template <bool kO, int D, int RP, bool kPad>
 __global__ void __launch_bounds__(kThreads, 1)
     score_tc1_kernel(const __grid_constant__ Tc1Launch lp) {
-  using C = Tc1Cfg<kO>;
-  using SM = Tc1Smem<kO>;
+  using C = Tc1Cfg<kO, D, RP>;
+  using SM = Tc1Smem<kO, D, RP>;
+  constexpr int kTileBytes = C::TileBytes;
   const Tc1Params &p = lp.p;
+  const int R = kPad ? p.R : RP;  // window rows
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *ktiles = smem;
@@ -442,6 +468,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_alloc(&ms->tmem_base, 512);
     tmem_relinquish();
   }
+  if constexpr (kPad) {
+    // the padding rows of the query buffers (no copy writes them) hold zeros
+    for (int i = threadIdx.x; i < 2 * kTileBytes / 16; i += kThreads)
+      reinterpret_cast<uint4 *>(qsm)[i] = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -475,12 +507,13 @@ __global__ void __launch_bounds__(kThreads, 1)
               ok = false;
               break;
             }
-            const int layer = st.u1 / p.upl, local = st.u1 % p.upl;
-            const int b = local / p.Hkv, h = local % p.Hkv;
-            const int qrow0 = (b * p.Hq + h * p.G) * p.W;
-            mbar_arrive_expect_tx(&ms->q_full, kTileBytes);
-            tma_load_2d(q1m, &lp.qmap[layer], 0, qrow0, &ms->q_full);
-            tma_load_2d(q1m + kHalfBytes, &lp.qmap[layer], 64, qrow0, &ms->q_full);
+            mbar_arrive_expect_tx(&ms->q_full, (uint32_t)(C::Copies * R * D * 2));
+#pragma unroll
+            for (int i = 0; i < C::Copies * (D / 64); ++i) {
+              const int half = i % (D / 64), copy = i / (D / 64);
+              tma_load_2d(q1m + half * kHalfBytes + copy * RP * 128, &lp.qmap[l1], half * 64,
+                          loc1 * R, &ms->q_full);
+            }
           }
           if (kind == 2 && s == 0) {
             // the pass-2 item's queries (rows of its unit) into shared memory
@@ -488,12 +521,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               ok = false;
               break;
             }
-            const int layer = st.u2 / p.upl, local = st.u2 % p.upl;
-            const int b = local / p.Hkv, h = local % p.Hkv;
-            const int qrow0 = (b * p.Hq + h * p.G) * p.W;
-            mbar_arrive_expect_tx(&ms->qs_full, kTileBytes);
-            tma_load_2d(qsm, &lp.qmap[layer], 0, qrow0, &ms->qs_full);
-            tma_load_2d(qsm + kHalfBytes, &lp.qmap[layer], 64, qrow0, &ms->qs_full);
+            mbar_arrive_expect_tx(&ms->qs_full, (uint32_t)(R * D * 2));
+#pragma unroll
+            for (int half = 0; half < D / 64; ++half)
+              tma_load_2d(qsm + half * kHalfBytes, &lp.qmap[l2], half * 64, loc2 * R,
+                          &ms->qs_full);
             ++qcount;
           }
           const int tt = pass == 1 ? st.a0 + s : st.b0 + s;
@@ -509,8 +541,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           // out of the tile loop)
           const int layer = pass == 1 ? l1 : l2, local = pass == 1 ? loc1 : loc2;
           const CUtensorMap *km = kind == 3 ? &lp.vmap[layer] : &lp.kmap[layer];
-          tma_load_3d(kb, km, 0, tt * kTile, local, &ms->k_full[ks], pol);
-          tma_load_3d(kb + kHalfBytes, km, 64, tt * kTile, local, &ms->k_full[ks], pol);
+#pragma unroll
+          for (int half = 0; half < D / 64; ++half)
+            tma_load_3d(kb + half * kHalfBytes, km, half * 64, tt * kTile, local,
+                        &ms->k_full[ks], pol);
           ++kcount;
         }
       }
@@ -523,7 +557,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       int kcount = 0, acount = 0, qcount = 0, ocount = 0;
       int pv_count = 0;  // kO: probability tiles multiplied
-      constexpr uint32_t id = idesc_bf16(128, 128);
+      constexpr uint32_t id1 = idesc_bf16(128, 128);   // rows (all copies) x keys
+      constexpr uint32_t id2 = idesc_bf16(128, RP);    // keys x rows
       // O = P . V: P (rows x keys) and V (keys x dims) both MN-major
       constexpr uint32_t id_pv = idesc_bf16(128, 128) | (1u << 15) | (1u << 16);
       const uint32_t kbase = smem_u32(ktiles), qsbase = smem_u32(qsm), q1base = smem_u32(q1m);
@@ -596,9 +631,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t qd = pass == 1 ? q1d : qsd;
             const uint64_t ad = pass == 1 ? qd : kd, bd = pass == 1 ? kd : qd;
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
+            for (int kk = 0; kk < C::KSteps; ++kk) {
               const uint64_t off = (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
-              mma_bf16(d, ad + off, bd + off, id, kk > 0);
+              mma_bf16(d, ad + off, bd + off, pass == 1 ? id1 : id2, kk > 0);
             }
           }
           mma_commit(&ms->k_empty[ks]);
@@ -624,14 +659,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       const ItemRef it = item_of(p, k);
       float2 *mine = p.partial + guard((long long)it.unit * p.n_ch + it.chunk, 1,
                                        (long long)p.units * p.n_ch, p.status) *
-                                     128;
+                                     R;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < RP / 32; ++j) {
         const int r = lane + 32 * j;
         float2 a = ms->pstat[slot][0][r];
         const float2 b = ms->pstat[slot][1][r];
         combine(a.x, a.y, b.x, b.y);
-        mine[r] = a;
+#pragma unroll
+        for (int c = 1; c < C::Copies; ++c)
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            const float2 x = ms->pstat[slot][w][c * RP + r];
+            combine(a.x, a.y, x.x, x.y);
+          }
+        if (r < R) mine[r] = a;
       }
       __syncwarp();
       int last = 0;
@@ -646,30 +688,34 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float2 *part =
             p.partial + guard((long long)it.unit * p.n_ch, p.n_ch, (long long)p.units * p.n_ch,
                               p.status) *
-                            128;
-        float mm[4], ll[4];
+                            R;
+        constexpr int RJ = RP / 32;   // rows per lane
+        constexpr int CB = 32 / RJ;   // items per batch: 32 loads of a lane in flight
+        float mm[RJ], ll[RJ];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < RJ; ++j) {
           mm[j] = -INFINITY;
           ll[j] = 0.f;
         }
-        for (int c0 = 0; c0 < p.n_ch; c0 += 8) {
-          float2 q[8][4];
+        for (int c0 = 0; c0 < p.n_ch; c0 += CB) {
+          float2 q[CB][RJ];
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
+          for (int c = 0; c < CB; ++c)
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-              q[c][j] = c0 + c < p.n_ch ? __ldcg(&part[(size_t)(c0 + c) * 128 + lane + 32 * j])
-                                        : make_float2(-INFINITY, 0.f);
+            for (int j = 0; j < RJ; ++j)
+              q[c][j] = c0 + c < p.n_ch && lane + 32 * j < R
+                            ? __ldcg(&part[(size_t)(c0 + c) * R + lane + 32 * j])
+                            : make_float2(-INFINITY, 0.f);
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
+          for (int c = 0; c < CB; ++c)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) combine(mm[j], ll[j], q[c][j].x, q[c][j].y);
+            for (int j = 0; j < RJ; ++j) combine(mm[j], ll[j], q[c][j].x, q[c][j].y);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          p.lognorm[guard(it.unit, 1, p.units, p.status) * 128 + lane + 32 * j] =
-              mm[j] + __log2f(ll[j]);
+        for (int j = 0; j < RJ; ++j)
+          if (lane + 32 * j < R)
+            p.lognorm[guard(it.unit, 1, p.units, p.status) * R + lane + 32 * j] =
+                mm[j] + __log2f(ll[j]);
         __threadfence();
         __syncwarp();
         if (lane == 0) st_release(&p.ctrl[guard(p.units + it.unit, 1, 2LL * p.units, p.status)], 1);
@@ -679,7 +725,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------ epilogue warpgroups
     const int wg = (warp - 2) >> 2;
     const int quarter = warp & 3;              // TMEM lanes this warp may access
-    const int r = quarter * 32 + lane;         // window row of this thread
+    const int r = quarter * 32 + lane;         // TMEM lane of this thread
+    const int row = r % RP;                    // pass 1: its window row,
+    const int col0 = r / RP * RP;              //   and its first key column
+    const bool live1 = !kPad || quarter * 32 % RP < R;  // the warp has rows that are not padding
     const int wtid = threadIdx.x - 64 - wg * 128;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     int tcount = 0;  // tiles seen
@@ -692,7 +741,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int k = 0; k < n + kLag; ++k) {
       const Step st = step_of(p, k, n);
       float m = -INFINITY, l = 0.f;    // pass 1 of item k: this row's max and sum
-      const int last_vis = p.P + r % p.W;
+      const int last_vis = p.P + row % p.W;
+      // votes of the pass-2 unit: its layer's slot of the vote array
+      const long long vote0 =
+          (long long)(p.layer_of[st.u2 / p.upl] * p.upl + st.u2 % p.upl) * p.P;
       for (int j = 0; j < st.len; ++j) {
         int pass, s;
         seq_at(st, j, pass, s);
@@ -704,30 +756,32 @@ __global__ void __launch_bounds__(kThreads, 1)
           ++tcount;
           if (mine && warp_wait(&ms->acc_full[as], ph, ms, p.status)) {
             tc_fence_after();
-            uint32_t x[4][32];
+            uint32_t x[RP / 32][32];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) tmem_ld32(tmem + lane_addr + as * 128 + c * 32, x[c]);
+            for (int c = 0; c < RP / 32; ++c)
+              tmem_ld32(tmem + lane_addr + as * 128 + (C::Copies > 1 ? col0 : 0) + c * 32, x[c]);
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cnt(&ms->acc_empty[as], kO ? 2 : 1);
+            const int key0 = t * kTile + (C::Copies > 1 ? col0 : 0);  // this thread's first key
             if ((t + 1) * kTile - 1 >= p.P) {  // keys this row cannot see -> -inf
 #pragma unroll
-              for (int c = 0; c < 4; ++c)
+              for (int c = 0; c < RP / 32; ++c)
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
-                  if (t * kTile + c * 32 + j > last_vis) x[c][j] = 0xff800000u;
+                  if (key0 + c * 32 + j > last_vis) x[c][j] = 0xff800000u;
             }
             float mx[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) mx[i] = -INFINITY;
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
+            for (int c = 0; c < RP / 32; ++c)
 #pragma unroll
               for (int j = 0; j < 32; ++j) mx[j & 7] = fmaxf(mx[j & 7], __uint_as_float(x[c][j]));
             const float tmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
                                      fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
-            if (tmax != -INFINITY) {
+            if (live1 && tmax != -INFINITY) {
               const float mnew = fmaxf(m, tmax * p.scale2);
               // fp32x2: logits scaled and shifted two at a time, sums in pairs
               float2 sv[4];
@@ -735,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int i = 0; i < 4; ++i) sv[i] = make_float2(0.f, 0.f);
               const float2 s2 = make_float2(p.scale2, p.scale2), mn2 = make_float2(-mnew, -mnew);
 #pragma unroll
-              for (int c = 0; c < 4; ++c)
+              for (int c = 0; c < RP / 32; ++c)
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
                   const float2 y = __ffma2_rn(
@@ -767,8 +821,9 @@ __global__ void __launch_bounds__(kThreads, 1)
               wait_ready(&p.ctrl[guard(p.units + st.u2, 1, 2LL * p.units, p.status)], ms,
                          p.status);
             named_bar_sync(3 + wg, 128);
-            ms->offs[wg][wtid] =
-                __ldcg(&p.lognorm[guard(st.u2, 1, p.units, p.status) * 128 + wtid]);
+            if (wtid < R)
+              ms->offs[wg][wtid] =
+                  __ldcg(&p.lognorm[guard(st.u2, 1, p.units, p.status) * R + wtid]);
             named_bar_sync(3 + wg, 128);
           }
           const int t = st.b0 + s;
@@ -806,14 +861,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (wg == 1) ms->vhalf[ptc & 1][r] = half;
             named_bar_sync(6, 256);
             if (wg == 0 && got && key < p.P)
-              p.votes[guard((long long)st.u2 * p.P + key, 1, (long long)p.units * p.P, p.status)] =
+              p.votes[guard(vote0 + key, 1, (long long)p.n_slots * p.upl * p.P, p.status)] =
                   half + ms->vhalf[ptc & 1][r];
             ++ptc;
           } else if (wg_of(tcount) == wg && warp_wait(&ms->acc_full[as], ph, ms, p.status)) {
             tc_fence_after();
-            uint32_t x[4][32];
+            uint32_t x[RP / 32][32];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) tmem_ld32(tmem + lane_addr + as * 128 + c * 32, x[c]);
+            for (int c = 0; c < RP / 32; ++c)
+              tmem_ld32(tmem + lane_addr + as * 128 + c * 32, x[c]);
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
@@ -824,8 +880,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int i = 0; i < 8; ++i) sv[i >> 2][i & 3] = make_float2(0.f, 0.f);
             const float2 s2 = make_float2(p.scale2, p.scale2);
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
+            auto columns = [&](int c, auto some_padding) {
+              float2 *h = sv[c >> 1];
 #pragma unroll
               for (int j4 = 0; j4 < 8; ++j4) {
                 const float4 o = o4[c * 8 + j4];
@@ -835,19 +891,33 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float2 y1 = __ffma2_rn(make_float2(__uint_as_float(x[c][4 * j4 + 2]),
                                                          __uint_as_float(x[c][4 * j4 + 3])),
                                              s2, make_float2(-o.z, -o.w));
-                float2 *h = sv[c >> 1];
-                h[(2 * j4) & 3] =
-                    __fadd2_rn(h[(2 * j4) & 3], make_float2(fast_exp2(y0.x), fast_exp2(y0.y)));
-                h[(2 * j4 + 1) & 3] = __fadd2_rn(h[(2 * j4 + 1) & 3],
-                                                 make_float2(fast_exp2(y1.x), fast_exp2(y1.y)));
+                float2 e0 = make_float2(fast_exp2(y0.x), fast_exp2(y0.y));
+                float2 e1 = make_float2(fast_exp2(y1.x), fast_exp2(y1.y));
+                if constexpr (decltype(some_padding)::value) {
+                  const int left = R - (c * 32 + 4 * j4);  // rows from this column on
+                  if (left < 1) e0.x = 0.f;
+                  if (left < 2) e0.y = 0.f;
+                  if (left < 3) e1.x = 0.f;
+                  if (left < 4) e1.y = 0.f;
+                }
+                h[(2 * j4) & 3] = __fadd2_rn(h[(2 * j4) & 3], e0);
+                h[(2 * j4 + 1) & 3] = __fadd2_rn(h[(2 * j4 + 1) & 3], e1);
               }
+            };
+#pragma unroll
+            for (int c = 0; c < RP / 32; ++c) {
+              if (!kPad || (c + 1) * 32 <= R)
+                columns(c, std::false_type{});
+              else if (c * 32 < R)
+                columns(c, std::true_type{});
+            }
             const float h0 = ((sv[0][0].x + sv[0][0].y) + (sv[0][1].x + sv[0][1].y)) +
                              ((sv[0][2].x + sv[0][2].y) + (sv[0][3].x + sv[0][3].y));
             const float h1 = ((sv[1][0].x + sv[1][0].y) + (sv[1][1].x + sv[1][1].y)) +
                              ((sv[1][2].x + sv[1][2].y) + (sv[1][3].x + sv[1][3].y));
             const int key = t * kTile + r;
             if (key < p.P)
-              p.votes[guard((long long)st.u2 * p.P + key, 1, (long long)p.units * p.P, p.status)] =
+              p.votes[guard(vote0 + key, 1, (long long)p.n_slots * p.upl * p.P, p.status)] =
                   h0 + h1;
           }
           ++tcount;
@@ -927,19 +997,63 @@ EncodeTiledFn encode_fn() {
 
 }  // namespace
 
+bool score_tc1_supported(const LayerGeom &g) {
+  return g.dtype == RIPPLE_BF16 && g.R <= 128 && g.P > 0;
+}
+
+bool score_tc1_attn_supported(const LayerGeom &g) {
+  return score_tc1_supported(g) && g.D == 128 && g.R == 128;
+}
+
+namespace {
+
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 0 ? sms : 1;
+}
+
+// Key tiles per item of a unit of n_tiles: at least `least`, and no more items
+// than SMs (the deadlock-free schedule needs at most twice as many as CTAs).
+int tiles_per_item(int n_tiles, int least, int sms) {
+  const int tpi_min = (n_tiles + sms - 1) / sms;
+  return tpi_min > least ? tpi_min : least;
+}
+
+struct Tc1Kernel {
+  const void *fn;
+  int smem;
+};
+
+template <bool kO, int D, int RP, bool kPad>
+Tc1Kernel tc1_kernel() {
+  return {(const void *)score_tc1_kernel<kO, D, RP, kPad>, Tc1Smem<kO, D, RP>::Bytes};
+}
+
+// Rows are padded to 32, 64 or 128: a thread's share of a tile is then RP
+// exponentials, so a unit of 64 window rows costs half of one of 128.
+template <int D>
+Tc1Kernel tc1_kernel_for(int R) {
+  if (R == 128) return tc1_kernel<false, D, 128, false>();
+  if (R > 64) return tc1_kernel<false, D, 128, true>();
+  if (R == 64) return tc1_kernel<false, D, 64, false>();
+  if (R > 32) return tc1_kernel<false, D, 64, true>();
+  if (R == 32) return tc1_kernel<false, D, 32, false>();
+  return tc1_kernel<false, D, 32, true>();
+}
+
+}  // namespace
+
 int score_tc1_max_items(const LayerGeom &g) {
   const int n_tiles = (g.T + kTile - 1) / kTile;
   return (n_tiles + kMinTilesPerItemO - 1) / kMinTilesPerItemO;
 }
 
-bool score_tc1_supported(const LayerGeom &g) {
-  return g.dtype == RIPPLE_BF16 && g.D == 128 && g.R == 128 && g.P > 0 && encode_fn() != nullptr;
-}
-
-cudaError_t launch_score_tc1(const LayerGeom &g, int n_layers, const void *const *q_win,
-                             const void *const *k, const CompressWs &ws, float *votes,
-                             int32_t *status, cudaStream_t st, const void *const *v,
-                             float *const *o_win) {
+cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, int n_layers,
+                             const void *const *q_win, const void *const *k,
+                             const CompressWs &ws, float *votes, int32_t *status,
+                             cudaStream_t st, const void *const *v, float *const *o_win) {
   EncodeTiledFn enc = encode_fn();
   if (enc == nullptr || n_layers < 1 || n_layers > kCompressMaxLayers) return cudaErrorNotSupported;
   const bool with_o = v != nullptr;
@@ -949,8 +1063,9 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_layers, const void *const
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
   for (int l = 0; l < n_layers; ++l) {
-    cuuint64_t dims[3] = {128, (cuuint64_t)g.T, (cuuint64_t)g.units};
-    cuuint64_t strides[2] = {256, (cuuint64_t)g.T * 256};
+    const cuuint64_t row = (cuuint64_t)g.D * 2;
+    cuuint64_t dims[3] = {(cuuint64_t)g.D, (cuuint64_t)g.T, (cuuint64_t)g.units};
+    cuuint64_t strides[2] = {row, (cuuint64_t)g.T * row};
     cuuint32_t box[3] = {64, 128, 1};
     cuuint32_t es[3] = {1, 1, 1};
     if (enc(&lp.kmap[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(k[l]), dims,
@@ -962,22 +1077,20 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_layers, const void *const
             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
-    cuuint64_t qdims[2] = {128, (cuuint64_t)g.B * g.Hq * g.W};
-    cuuint64_t qstrides[1] = {256};
-    cuuint32_t qbox[2] = {64, 128};
+    cuuint64_t qdims[2] = {(cuuint64_t)g.D, (cuuint64_t)g.units * g.R};
+    cuuint64_t qstrides[1] = {row};
+    cuuint32_t qbox[2] = {64, (cuuint32_t)g.R};
     cuuint32_t qes[2] = {1, 1};
     if (enc(&lp.qmap[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(q_win[l]), qdims,
             qstrides, qbox, qes, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
   }
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (sms <= 0) sms = 1;
+  const int sms = sm_count();
   Tc1Params &p = lp.p;
   p.upl = g.units;
   p.units = g.units * n_layers;
+  p.R = g.R;
   p.T = g.T;
   p.P = g.P;
   p.W = g.W;
@@ -986,11 +1099,7 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_layers, const void *const
   p.G = g.G;
   p.n_tiles1 = (g.T + kTile - 1) / kTile;
   p.n_tiles2 = with_o ? p.n_tiles1 : (g.P + kTile - 1) / kTile;
-  // At least kMinTilesPerItem tiles per item, and no more items per unit than
-  // SMs (the deadlock-free schedule needs <= 2x as many as CTAs).
-  const int tpi_min = (p.n_tiles1 + sms - 1) / sms;
-  const int tpi_floor = with_o ? kMinTilesPerItemO : kMinTilesPerItem;
-  p.tpi = tpi_min > tpi_floor ? tpi_min : tpi_floor;
+  p.tpi = tiles_per_item(p.n_tiles1, with_o ? kMinTilesPerItemO : kMinTilesPerItem, sms);
   p.n_ch = (p.n_tiles1 + p.tpi - 1) / p.tpi;
   p.total_items = p.units * p.n_ch;
   p.scale2 = g.scale2;
@@ -1000,20 +1109,26 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_layers, const void *const
   p.partial = ws.row_partial;
   p.lognorm = ws.row_lognorm;
   p.votes = votes;
+  for (int l = 0; l < n_layers; ++l) {
+    if (slots[l] < 0 || slots[l] >= n_slots) return cudaErrorInvalidValue;
+    p.layer_of[l] = slots[l];
+  }
+  p.n_slots = n_slots;
   p.ctrl = ws.counters;
   p.status = status;
   p.wait_cycles = wait_limit_cycles();
   cudaError_t e = cudaMemsetAsync(ws.counters, 0, sizeof(int) * 2 * p.units, st);
   if (e == cudaSuccess && with_o) e = cudaMemsetAsync(ws.o_count, 0, sizeof(int) * p.units, st);
   if (e != cudaSuccess) return e;
-  const void *kernel = with_o ? (const void *)score_tc1_kernel<true>
-                              : (const void *)score_tc1_kernel<false>;
-  const int smem = with_o ? Tc1Smem<true>::Bytes : Tc1Smem<false>::Bytes;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const Tc1Kernel kernel = with_o         ? tc1_kernel<true, 128, 128, false>()
+                           : g.D == 64 ? tc1_kernel_for<64>(g.R)
+                                       : tc1_kernel_for<128>(g.R);
+  e = cudaFuncSetAttribute(kernel.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kernel.smem);
   if (e != cudaSuccess) return e;
   const int grid = p.total_items < sms ? p.total_items : sms;
   void *args[] = {(void *)&lp};
-  e = cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(kThreads), args, (size_t)smem, st);
+  e = cudaLaunchCooperativeKernel(kernel.fn, dim3(grid), dim3(kThreads), args,
+                                  (size_t)kernel.smem, st);
   count_launches(1);
   return e;
 }
