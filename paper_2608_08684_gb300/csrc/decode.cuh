@@ -35,17 +35,18 @@ struct DecParams {
 // than SMs (a single layer's step, short caches) smaller items, down to
 // kMinItemRows, as long as they fit in one wave.
 constexpr int kMaxItemRows = 4096;
-constexpr int kMinItemRows = 256;
+constexpr int kMinItemRows = 128;
+constexpr int kItemRowStep = 32;
 
 // Control block of a step in the workspace (int32 words). The init flag has a
 // 128-byte line to itself; CTA 0 zeroes the counters at the start of every
 // call and then sets the flag to the call's epoch, and the other CTAs use no
-// counter before they have seen it. The last CTA to leave sets the flag back
-// to 0, so that a replay of the same launch (same epoch) waits for CTA 0
-// again.
+// counter before they have seen it. The last block sets the flag back to 0
+// once all have, so that a replay of the same launch (same epoch) waits for
+// CTA 0 again.
 constexpr int kCtrlFlag = 0;    // init flag
 constexpr int kCtrlItem = 32;   // work-item counter
-constexpr int kCtrlExit = 33;   // CTAs that have left
+constexpr int kCtrlArrived = 33;  // CTAs that have read the lengths and seen the flag
 constexpr int kCtrlGroup = 34;  // + group: items of the group finished
 
 }  // namespace ripple
