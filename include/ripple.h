@@ -235,7 +235,7 @@ ripple_status ripple_compress_layers_attn_workspace_bytes(const ripple_layer_des
  *             256-byte aligned, no initialisation needed
  * Other arguments, outputs and errors as ripple_compress_layers, with the same
  * kept counts. The two calls split a unit's keys into different items (this
- * one takes up to 32768 keys a unit as one), so the row normalisers, merged
+ * one by the units of the whole call), so the row normalisers, merged
  * from the items' partial statistics, can differ in their last bits, and a
  * token whose pooled vote ties the selection threshold to within that
  * rounding can be kept by one call and not the other; units of at most 1152

@@ -69,8 +69,10 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, 
                              const CompressWs &ws, float *votes, int32_t *status,
                              cudaStream_t st, const void *const *v = nullptr,
                              float *const *o_win = nullptr);
-// Items per unit of launch_score_tc1 at most (sizes the output partials).
-int score_tc1_max_items(const LayerGeom &g);
+// Items per unit of a launch_score_tc1 with outputs (sizes the output partials):
+// the number with the least modelled time, the steps of the busiest CTA times
+// its item's tiles and the cost of a step, so that few units still fill the GPU.
+int score_tc1_attn_items(const LayerGeom &g, int n_layers);
 // The gather's inputs and outputs per layer (launch_gather's arguments).
 struct GatherArgs {
   const void *const *k;

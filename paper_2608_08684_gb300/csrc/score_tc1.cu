@@ -65,12 +65,12 @@ constexpr int kThreads = 352;
 constexpr int kLag = 1;                         // pass 2 of item k runs in step k + kLag
 constexpr int kPubSlots = 2;
 constexpr int kMinTilesPerItem = 9;
-// kO: a whole unit per item up to 32768 keys. An item's partial output, its
-// row-slice sum and pass 2's wait on the unit's other items cost more than
-// re-reading the keys from DRAM in pass 2 (an item's keys no longer stay in
-// L2 until then): 32 layers of the 32k workload took 5.39 / 5.25 / 5.08 /
-// 5.11 / 5.00 ms with items of 32 / 64 / 86 / 128 / 256 tiles.
-constexpr int kMinTilesPerItemO = 256;
+// kO: what a step costs on top of its item's tiles, in tiles: the item's
+// partial output, its row-slice sum, the hand-overs and the queries. Fitted to
+// 8 layers of 8 units and 256 tiles (items of 256 / 128 / 64 / 43 / 37 / 32 /
+// 19 tiles, 1 / 1 / 2 / 3 / 3 / 4 / 6 steps: 728 / 428 / 441 / 452 / 411 / 464
+// / 466 us, about 128 us and 2.34 us a tile) and to five other shapes.
+constexpr int kStepTilesO = 5;
 constexpr int kMaxStages = 8;
 constexpr int kOReduceLag = 2;  // kO: a step's item rows are summed this many steps later
 
@@ -1014,8 +1014,10 @@ int sm_count() {
   return sms > 0 ? sms : 1;
 }
 
-// Key tiles per item of a unit of n_tiles: at least `least`, and no more items
-// than SMs (the deadlock-free schedule needs at most twice as many as CTAs).
+// Votes only: key tiles per item of a unit of n_tiles: at least `least`, and no
+// more items than SMs (the deadlock-free schedule needs at most twice as many
+// as CTAs). A function of the prompt length alone, so that one layer's call
+// and a multi-layer call merge the same partial statistics.
 int tiles_per_item(int n_tiles, int least, int sms) {
   const int tpi_min = (n_tiles + sms - 1) / sms;
   return tpi_min > least ? tpi_min : least;
@@ -1045,9 +1047,23 @@ Tc1Kernel tc1_kernel_for(int R) {
 
 }  // namespace
 
-int score_tc1_max_items(const LayerGeom &g) {
-  const int n_tiles = (g.T + kTile - 1) / kTile;
-  return (n_tiles + kMinTilesPerItemO - 1) / kMinTilesPerItemO;
+int score_tc1_attn_items(const LayerGeom &g, int n_layers) {
+  const int n_tiles = (g.T + kTile - 1) / kTile, sms = sm_count();
+  // a unit of up to kMinTilesPerItem tiles is one item, as without outputs
+  const int most = n_tiles / kMinTilesPerItem < sms ? n_tiles / kMinTilesPerItem : sms;
+  const long long units = (long long)g.units * n_layers;
+  int best = 1;
+  long long best_cost = -1;
+  for (int n = 1; n <= most || n == 1; ++n) {
+    const int per = (n_tiles + n - 1) / n;
+    if ((n_tiles + per - 1) / per != n) continue;  // items would be left empty
+    const long long cost = (units * n + sms - 1) / sms * (per + kStepTilesO);
+    if (best_cost < 0 || cost * 50 < best_cost * 49) {  // more items by 2% or not
+      best = n;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, int n_layers,
@@ -1099,7 +1115,9 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, 
   p.G = g.G;
   p.n_tiles1 = (g.T + kTile - 1) / kTile;
   p.n_tiles2 = with_o ? p.n_tiles1 : (g.P + kTile - 1) / kTile;
-  p.tpi = tiles_per_item(p.n_tiles1, with_o ? kMinTilesPerItemO : kMinTilesPerItem, sms);
+  p.tpi = with_o ? (p.n_tiles1 + score_tc1_attn_items(g, n_layers) - 1) /
+                       score_tc1_attn_items(g, n_layers)
+                 : tiles_per_item(p.n_tiles1, kMinTilesPerItem, sms);
   p.n_ch = (p.n_tiles1 + p.tpi - 1) / p.tpi;
   p.total_items = p.units * p.n_ch;
   p.scale2 = g.scale2;
