@@ -108,20 +108,25 @@ struct Cfg {
   static constexpr int R = 128 * NR;             // window rows
   static constexpr int TileBytes = D / 64 * kHalfBytes;  // one 128 x D bf16 tile
   static constexpr int KSteps = D / 16;          // MMAs per 128 x 128 product
-  static constexpr int NK = D == 128 ? 2 : 4;    // key-tile stages
-  // Query buffers: two items are in flight (pass 1 of one, pass 2 of the
-  // previous).
-  static constexpr int NQ = 2;
-  static constexpr int NA = 2;                   // TMEM accumulator stages
-  static constexpr int ACC_COLS = 128 * NR;      // TMEM columns per stage
+  // Key-tile stages: 128 KB in flight hide the latency of HBM. The queries
+  // have one buffer, loaded anew for every pass of an item; with two buffers
+  // and half the stages the loads' latency bound the kernel.
+  static constexpr int NK = D == 128 ? 4 : 8;
+  // TMEM accumulators, one per row half of a tile, two tiles in flight. Each is
+  // filled and released by itself: with whole tiles (2 x 256 columns) the MMAs
+  // of a tile began only when its warpgroup had folded the first half of the
+  // tile before and loaded the second, and tensor cores and exponentials took
+  // turns (45% busy each).
+  static constexpr int NA = 2 * NR;
+  static constexpr int ACC_COLS = 128;
   static constexpr int QBYTES = NR * TileBytes;  // [D / 64][256 rows][64 dims]
   static constexpr int OFF_K = 0;
   static constexpr int OFF_Q = OFF_K + NK * TileBytes;
-  static constexpr int OFF_MISC = OFF_Q + NQ * QBYTES;
+  static constexpr int OFF_MISC = OFF_Q + QBYTES;
 };
 
 struct Misc {
-  uint64_t k_full[4], k_empty[4], q_full[3], q_empty[3], acc_full[4], acc_empty[4], mma_done;
+  uint64_t k_full[8], k_empty[8], q_full, q_empty, acc_full[4], acc_empty[4], mma_done;
   uint64_t pub_full[kPubSlots], pub_empty[kPubSlots];
   uint32_t tmem_base;
   int abort_flag;
@@ -215,10 +220,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&ms->k_full[i], 1);
       mbar_init(&ms->k_empty[i], 1);
     }
-    for (int i = 0; i < C::NQ; ++i) {
-      mbar_init(&ms->q_full[i], 1);
-      mbar_init(&ms->q_empty[i], 1);
-    }
+    mbar_init(&ms->q_full, 1);
+    mbar_init(&ms->q_empty, 1);
     for (int i = 0; i < C::NA; ++i) {
       mbar_init(&ms->acc_full[i], 1);
       mbar_init(&ms->acc_empty[i], 4);
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   if constexpr (kPad) {
     // the padding rows of the query buffers (no copy writes them) hold zeros
-    for (int i = threadIdx.x; i < C::NQ * C::QBYTES / 16; i += kThreads)
+    for (int i = threadIdx.x; i < C::QBYTES / 16; i += kThreads)
       reinterpret_cast<uint4 *>(qbufs)[i] = make_uint4(0, 0, 0, 0);
     fence_proxy_async_smem();
   }
@@ -288,73 +291,81 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = max(0, kcount - C::NK); j < kcount; ++j)
         mbar_wait(&ms->k_full[j % C::NK], (j / C::NK) & 1, nullptr);
     } else if (lane == 1) {
+      // in the order of the passes: P1(0) P1(1) P2(0) P1(2) P2(1) ..
       int qcount = 0;
-      for (int k = 0; k < n; ++k) {
-        const ItemRef it = item_of(p, k);
-        const int local = it.unit % p.upl;
-        const CUtensorMap *qm = &lp.qmap[it.unit / p.upl];
-        const int qs = k % C::NQ;
-        if (!wait_bar(&ms->q_empty[qs], ((k / C::NQ) & 1) ^ 1, ms, p.status)) break;
-        mbar_arrive_expect_tx(&ms->q_full[qs], (uint32_t)(p.R * D * 2));
-        uint8_t *qb = qbufs + qs * C::QBYTES;
+      bool ok = true;
+      for (int k = 0; k <= n && ok; ++k) {
+        for (int pass = 1; pass <= 2 && ok; ++pass) {
+          if ((pass == 1 && k >= n) || (pass == 2 && k < 1)) continue;
+          const ItemRef it = item_of(p, pass == 1 ? k : k - 1);
+          const int local = it.unit % p.upl;
+          const CUtensorMap *qm = &lp.qmap[it.unit / p.upl];
+          if (!wait_bar(&ms->q_empty, (qcount & 1) ^ 1, ms, p.status)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx(&ms->q_full, (uint32_t)(p.R * D * 2));
 #pragma unroll
-        for (int half = 0; half < D / 64; ++half)
-          tma_load_2d(qb + half * (NR * kHalfBytes), qm, half * 64, local * p.R, &ms->q_full[qs]);
-        ++qcount;
+          for (int half = 0; half < D / 64; ++half)
+            tma_load_2d(qbufs + half * (NR * kHalfBytes), qm, half * 64, local * p.R, &ms->q_full);
+          ++qcount;
+        }
       }
-      for (int k = max(0, qcount - C::NQ); k < qcount; ++k)
-        mbar_wait(&ms->q_full[k % C::NQ], (k / C::NQ) & 1, nullptr);
+      if (qcount > 0) mbar_wait(&ms->q_full, (qcount - 1) & 1, nullptr);
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     if (lane == 0) {
-      int kcount = 0, acount = 0;
-      constexpr uint32_t id1 = idesc_bf16(128, 128);
-      constexpr uint32_t id2 = idesc_bf16(128, 128 * NR);
+      int kcount = 0, acount = 0, qcount = 0;
+      constexpr uint32_t id = idesc_bf16(128, 128);
       const uint32_t kbase = smem_u32(ktiles), qbase = smem_u32(qbufs);
       bool ok = true;
       for (int k = 0; k <= n && ok; ++k) {
         for (int pass = 1; pass <= 2 && ok; ++pass) {
           if ((pass == 1 && k >= n) || (pass == 2 && k < 1)) continue;
-          const int item = pass == 1 ? k : k - 1;
-          const ItemRef it = item_of(p, item);
-          const int qs = item % C::NQ;
-          if (pass == 1 && !wait_bar(&ms->q_full[qs], (item / C::NQ) & 1, ms, p.status)) {
+          const ItemRef it = item_of(p, pass == 1 ? k : k - 1);
+          if (!wait_bar(&ms->q_full, qcount & 1, ms, p.status)) {
             ok = false;
             break;
           }
-          const uint32_t qa = qbase + qs * C::QBYTES;
+          ++qcount;
+          const uint32_t qa = qbase;
           int t0, t1;
           tiles_of(p, it, pass, t0, t1);
           for (int t = t0; t < t1; ++t) {
-            const int ks = kcount % C::NK, as = acount % C::NA;
-            if (!wait_bar(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status) ||
-                !wait_bar(&ms->acc_empty[as], ((acount / C::NA) & 1) ^ 1, ms, p.status)) {
+            const int ks = kcount % C::NK;
+            if (!wait_bar(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status)) {
               ok = false;
               break;
             }
-            tc_fence_after();
-            const uint32_t d = tmem + as * C::ACC_COLS;
-            const uint32_t ka = kbase + ks * kTileBytes;
+            const uint64_t kd = sw128_desc(kbase + ks * kTileBytes);
 #pragma unroll
-            for (int kk = 0; kk < C::KSteps; ++kk) {
-              const uint32_t koff = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
-              const uint32_t qoff = (kk >> 2) * (NR * kHalfBytes) + (kk & 3) * 32;
-              if (pass == 1) {
-#pragma unroll
-                for (int nr = 0; nr < NR; ++nr)
-                  mma_bf16(d + nr * 128, sw128_desc(qa + qoff + nr * kHalfBytes),
-                           sw128_desc(ka + koff), id1, kk > 0);
-              } else {
-                mma_bf16(d, sw128_desc(ka + koff), sw128_desc(qa + qoff), id2, kk > 0);
+            for (int nr = 0; nr < NR; ++nr) {
+              const int as = acount % C::NA;
+              if (!wait_bar(&ms->acc_empty[as], ((acount / C::NA) & 1) ^ 1, ms, p.status)) {
+                ok = false;
+                break;
               }
+              tc_fence_after();
+              const uint32_t d = tmem + as * C::ACC_COLS;
+              // the first K step's descriptors; the others differ only in their
+              // start-address field (16-byte units, no carry)
+              const uint64_t qd = sw128_desc(qa + nr * kHalfBytes);
+#pragma unroll
+              for (int kk = 0; kk < C::KSteps; ++kk) {
+                const uint64_t ko = kd + (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
+                const uint64_t qo =
+                    qd + (uint64_t)(((kk >> 2) * (NR * kHalfBytes) + (kk & 3) * 32) >> 4);
+                mma_bf16(d, pass == 1 ? qo : ko, pass == 1 ? ko : qo, id, kk > 0);
+              }
+              mma_commit(&ms->acc_full[as]);
+              ++acount;
             }
+            if (!ok) break;
             mma_commit(&ms->k_empty[ks]);
-            mma_commit(&ms->acc_full[as]);
             ++kcount;
-            ++acount;
           }
-          if (ok && pass == 2) mma_commit(&ms->q_empty[qs]);  // the item is done with its queries
+          if (ok) mma_commit(&ms->q_empty);  // the pass is done with its queries
         }
       }
       // All issued MMAs complete before TMEM is released.
@@ -453,22 +464,20 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int t = t0; t < t1; ++t, ++tcount) {
           if ((tcount & 1) != wg) continue;
-          const int as = tcount % C::NA;
-          if (!warp_wait(&ms->acc_full[as], (tcount / C::NA) & 1, ms, p.status)) continue;
-          tc_fence_after();
           const bool masked = (t + 1) * kTile - 1 >= p.P;
 #pragma unroll
           for (int nr = 0; nr < NR; ++nr) {
+            const int at = tcount * NR + nr, as = at % C::NA;
+            if (!warp_wait(&ms->acc_full[as], (at / C::NA) & 1, ms, p.status)) continue;
+            tc_fence_after();
             uint32_t x[4][32];
-            const uint32_t base = tmem + lane_addr + as * C::ACC_COLS + nr * 128;
+            const uint32_t base = tmem + lane_addr + as * C::ACC_COLS;
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld32(base + c * 32, x[c]);
             tmem_wait_ld();
-            if (nr == NR - 1) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(&ms->acc_empty[as]);
-            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ms->acc_empty[as]);
             if (masked) {  // keys this row cannot see (causal window, past T) -> -inf
 #pragma unroll
               for (int c = 0; c < 4; ++c)
@@ -536,26 +545,26 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int vunit = p.layer_of[it.unit / p.upl] * p.upl + it.unit % p.upl;
         for (int t = t0; t < t1; ++t, ++tcount) {
           if ((tcount & 1) != wg) continue;
-          const int as = tcount % C::NA;
-          if (!warp_wait(&ms->acc_full[as], (tcount / C::NA) & 1, ms, p.status)) continue;
-          tc_fence_after();
           // fp32x2: logits scaled and shifted two at a time, sums in pairs
           float2 vs[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) vs[i] = make_float2(0.f, 0.f);
           const float2 s2 = make_float2(p.scale2, p.scale2);
-          const uint32_t base = tmem + lane_addr + as * C::ACC_COLS;
+          bool got = true;
 #pragma unroll
           for (int c4 = 0; c4 < NR; ++c4) {
+            const int at = tcount * NR + c4, as = at % C::NA;
+            got = got && warp_wait(&ms->acc_full[as], (at / C::NA) & 1, ms, p.status);
+            if (!got) continue;
+            tc_fence_after();
             uint32_t x[4][32];
+            const uint32_t base = tmem + lane_addr + as * C::ACC_COLS;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) tmem_ld32(base + c4 * 128 + c * 32, x[c]);
+            for (int c = 0; c < 4; ++c) tmem_ld32(base + c * 32, x[c]);
             tmem_wait_ld();
-            if (c4 == NR - 1) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(&ms->acc_empty[as]);
-            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ms->acc_empty[as]);
             auto columns = [&](int c, auto some_padding) {
 #pragma unroll
               for (int j = 0; j < 32; j += 4) {
@@ -592,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float vote = ((vs[0].x + vs[0].y) + (vs[1].x + vs[1].y)) +
                              ((vs[2].x + vs[2].y) + (vs[3].x + vs[3].y));
           const int key = t * kTile + lrow;
-          if (key < p.P)
+          if (got && key < p.P)
             p.votes[guard((long long)vunit * p.P + key, 1, (long long)p.n_slots * p.upl * p.P,
                           p.status)] = vote;
         }
