@@ -36,7 +36,7 @@ CompressWs carve_compress_ws(const LayerGeom &g, void *base) {
   w.row_partial = (float2 *)take(sizeof(float2) * g.units * n_chunks * 2 * g.R);
   w.row_lognorm = (float *)take(sizeof(float) * g.units * g.R);
   w.votes = (float *)take(sizeof(float) * g.units * (size_t)g.P);
-  w.keys = (uint32_t *)take(g.P > kSelectSmemKeys ? sizeof(uint32_t) * g.units * (size_t)g.P : 0);
+  w.keys = (uint32_t *)take(g.P > kSelectClusterMaxP ? sizeof(uint32_t) * g.units * (size_t)g.P : 0);
   w.counters = (int32_t *)take(sizeof(int32_t) * (128 + 2 * (size_t)g.units));
   w.bytes = off;
   return w;
@@ -127,12 +127,8 @@ extern "C" ripple_status ripple_compress_layer(const ripple_layer_desc *desc, in
                         : launch_score_simt(g, q_win, k, ws, votes, dev_status, st);
     RIPPLE_CUDA_TRY(e);
   }
-  if (keep_all) {
-    RIPPLE_CUDA_TRY(launch_iota(g, idx_out, st));
-  } else {
-    RIPPLE_CUDA_TRY(launch_select(g, 1, votes, ws, &n, &idx_out, dev_status, st));
-  }
-  RIPPLE_CUDA_TRY(launch_gather(g, 1, &k, &v, &idx_out, &n, &k_out, &v_out, &cap, dev_status, st));
+  const GatherArgs ga{&k, &v, &k_out, &v_out, &cap};
+  RIPPLE_CUDA_TRY(launch_select(g, 1, votes, ws, &n, &idx_out, dev_status, st, ga));
   *n_keep_host = n;
   return RIPPLE_OK;
 }
@@ -157,12 +153,8 @@ extern "C" ripple_status ripple_select_layer(const ripple_layer_desc *desc, int6
   const CompressWs ws = carve_compress_ws(g, workspace);
   if (workspace_bytes < ws.bytes) return RIPPLE_EWORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
-  if (n == g.T) {
-    RIPPLE_CUDA_TRY(launch_iota(g, idx_out, st));
-  } else {
-    RIPPLE_CUDA_TRY(launch_select(g, 1, votes, ws, &n, &idx_out, dev_status, st));
-  }
-  RIPPLE_CUDA_TRY(launch_gather(g, 1, &k, &v, &idx_out, &n, &k_out, &v_out, &cap, dev_status, st));
+  const GatherArgs ga{&k, &v, &k_out, &v_out, &cap};
+  RIPPLE_CUDA_TRY(launch_select(g, 1, votes, ws, &n, &idx_out, dev_status, st, ga));
   *n_keep_host = n;
   return RIPPLE_OK;
 }
@@ -243,9 +235,7 @@ static ripple_status compress_layers_impl(
                                    : carve_layers_ws(g, n_layers, workspace);
   if (workspace_bytes < ws.bytes) return RIPPLE_EWORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
-  // selection and gather in one launch where the selection kernel takes both
   const GatherArgs ga{k_host, v_host, k_out_host, v_out_host, cap};
-  bool gathered = false;
   if (g.P > 0) {
     // Scoring: on the tensor cores (bf16) every layer that needs votes in one
     // launch; on the CUDA cores (fp32) layer by layer, the scratch of the
@@ -277,12 +267,7 @@ static ripple_status compress_layers_impl(
                                           st));
     }
   }
-  RIPPLE_CUDA_TRY(launch_select(g, n_layers, ws.votes, ws, n, idx_out_host, dev_status, st, &ga,
-                                &gathered));
-  if (!gathered)
-    RIPPLE_CUDA_TRY(launch_gather(g, n_layers, k_host, v_host,
-                                  (const int32_t *const *)idx_out_host, n, k_out_host, v_out_host,
-                                  cap, dev_status, st));
+  RIPPLE_CUDA_TRY(launch_select(g, n_layers, ws.votes, ws, n, idx_out_host, dev_status, st, ga));
   for (int l = 0; l < n_layers; ++l) n_keep_host[l] = n[l];
   return RIPPLE_OK;
 }

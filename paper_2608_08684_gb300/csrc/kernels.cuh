@@ -29,8 +29,8 @@ struct LayerGeom {
 constexpr int kCompressMaxLayers = RIPPLE_COMPRESS_MAX_LAYERS;
 
 constexpr int kScoreChunk = 128;      // keys per scoring work item
-constexpr int kSelectThreads = 1024;  // threads of the selection CTA
-constexpr int kSelectSmemKeys = 48 * 1024;  // prefix lengths up to this keep keys in smem
+// Longer prefixes keep their selection keys in the workspace.
+constexpr int kSelectClusterMaxP = 8 * 26 * 1024;  // 8 CTAs of 26K keys and votes in 227 KB
 
 // Workspace carve-up of one compression call.
 struct CompressWs {
@@ -81,16 +81,12 @@ struct GatherArgs {
   void *const *v_out;
   const int *cap;
 };
-// Pooling + exact top-k per unit of n_layers layers (votes [n_layers][units][P]);
-// writes idx[l] [units][n_keep[l]]. With gather and gathered given, the
-// kernel may also gather the kept rows (as launch_gather would); *gathered
-// says whether it did.
+// Pooling, exact top-k per unit of n_layers layers (votes [n_layers][units][P])
+// and the gather of the kept rows; writes idx[l] [units][n_keep[l]]. A layer
+// that keeps every token (or only the window) needs no votes.
 cudaError_t launch_select(const LayerGeom &g, int n_layers, const float *votes,
                           const CompressWs &ws, const int *n_keep, int32_t *const *idx,
-                          int32_t *status, cudaStream_t st, const GatherArgs *gather = nullptr,
-                          bool *gathered = nullptr);
-// idx = 0..T-1 for every unit (keep-all case).
-cudaError_t launch_iota(const LayerGeom &g, int32_t *idx, cudaStream_t st);
+                          int32_t *status, cudaStream_t st, const GatherArgs &gather);
 // Gather kept K and V rows of n_layers layers into [units][cap[l]][d].
 cudaError_t launch_gather(const LayerGeom &g, int n_layers, const void *const *k,
                           const void *const *v, const int32_t *const *idx, const int *n_keep,

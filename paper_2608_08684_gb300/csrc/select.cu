@@ -1,23 +1,20 @@
 // Pooling of the prefix votes and exact top-k selection per unit (SnapKV's
 // selection rule kept by RippleKV; retained set S_l of Eq. 4).
 //
-// Three kernels, one result (bit for bit): select_unit_kernel (one CTA per
-// unit, launches with many units), select_cluster_kernel (8-CTA clusters per
-// unit, few units) and select_kernel (very long prefixes). The steps, for
-// one unit (b, h):
+// Three kernels, one result (bit for bit): select_pool_kernel for prefixes of up
+// to 131072 tokens, which also gathers the unit's kept K and V rows, and for
+// longer ones select_cluster_kernel (keys in the shared memory of 8 CTAs) and
+// select_kernel (keys in global scratch). The steps, for one unit (b, h):
 //   1. pooled score of every prefix token (max or mean over the clipped
-//      window), mapped to an order-preserving uint32 key (in registers, in
-//      shared memory, or in global scratch for very long prefixes);
-//   2. radix select over the keys (4 x 8 bits, or 11 + 11 + 10 bits, from
-//      the top) finds the K-th largest key tau and how many keys equal to
-//      tau are kept;
+//      window), mapped to an order-preserving uint32 key;
+//   2. radix select over the keys from the top bits finds the K-th largest key
+//      tau and how many keys equal to tau are kept;
 //   3. an ordered compaction writes every token with key > tau and the first
 //      tokens with key == tau (lower index wins ties) in ascending order,
 //      followed by the w window positions P..T-1.
-// The result is bit-exact and deterministic for a given vote array. In a
-// multi-layer call select_unit_kernel also gathers its unit's kept K and V
-// rows (as gather_kernel would), so selection and gather are one launch.
+// The result is bit-exact and deterministic for a given vote array.
 #include <math.h>
+#include <stddef.h>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -25,7 +22,7 @@
 namespace ripple {
 namespace {
 
-constexpr int kThreads = kSelectThreads;
+constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 2048;
 // Shared words after the histogram: scan scratch [0, 33), control [40, 48),
@@ -69,13 +66,12 @@ __device__ __forceinline__ int block_exclusive_scan(int x, int *warp_tot, int *t
 
 __global__ void __launch_bounds__(kThreads) select_kernel(LayerGeom g, const float *votes,
                                                           uint32_t *keys_global, int n_keep,
-                                                          int in_smem, int32_t *idx,
-                                                          int32_t *status) {
+                                                          int32_t *idx, int32_t *status) {
   extern __shared__ uint32_t sm[];
   uint32_t *hist = sm;                              // [kBins]
   int *warp_tot = (int *)(sm + kBins);              // [33]
   int *ctrl = warp_tot + 40;                        // [8] control words
-  uint32_t *keys = in_smem ? sm + kBins + kCtrlWords : keys_global + (size_t)blockIdx.x * g.P;
+  uint32_t *keys = keys_global + (size_t)blockIdx.x * g.P;
 
   const int unit = blockIdx.x;
   const int P = g.P, K = n_keep - g.W;
@@ -229,7 +225,6 @@ __global__ void __launch_bounds__(kThreads) select_kernel(LayerGeom g, const flo
 constexpr int kCluster = 8;
 constexpr int kCThreads = 512;
 constexpr int kCWarps = kCThreads / 32;
-constexpr int kCMaxKeys = 40 * 1024;  // keys per CTA held in shared memory
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -254,6 +249,17 @@ __device__ __forceinline__ uint2 ld_cluster_v2(uint32_t addr) {
   uint2 v;
   asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
   return v;
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n"
@@ -296,8 +302,8 @@ struct SelTable {
   int n_keep[kCompressMaxLayers];
   int32_t *idx[kCompressMaxLayers];
   int32_t *status;
-  // select_unit_kernel with gather != 0 also copies each unit's kept rows
-  int gather, row_bytes;
+  // select_pool_kernel, which also copies each unit's kept rows:
+  int row_bytes;
   const uint8_t *k[kCompressMaxLayers];
   const uint8_t *v[kCompressMaxLayers];
   uint8_t *k_out[kCompressMaxLayers];
@@ -504,318 +510,380 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kCThreads)
   cluster_sync_all();  // no CTA leaves while others may still read its memory
 }
 
-// Prefixes up to kUMaxP tokens: one 1024-thread CTA per unit and no cluster
-// (a launch covers every unit of every layer, so the GPU is filled by units).
-// Thread t keeps the pooled keys of tokens 32t .. 32t + 31 in registers: the
-// votes are staged in shared memory with a pad word after every 32 (coalesced
-// stores, conflict-free reads of a thread's run), the 7-wide max pooling is
-// three maxima per key over the run and its halo, four radix rounds of 8 bits
-// count into per-warp histograms (no contention between warps), and the
-// ordered compaction is one block scan over the threads' counts followed by
-// each thread writing its kept tokens in order. Same result as select_kernel,
-// bit for bit.
-constexpr int kUThreads = 1024;
-constexpr int kUWarps = kUThreads / 32;
-constexpr int kUKeys = 32;                    // keys per thread
-constexpr int kUMaxP = kUThreads * kUKeys;
-constexpr int kUBins = 256;
-constexpr int kUMinUnits = 256;               // units per launch for this kernel
-constexpr int kUCand = 128;                   // bucket size that ends the radix rounds
-// shared words before the staged votes: per-warp histograms, bin totals,
-// scan scratch and control
-constexpr int kUHead = kUWarps * kUBins + kUBins + 64;
+// ---------------------------------------------------------------------------
+// Prefixes of up to kPoolMaxP tokens: pooling, selection and gather in one
+// launch, a cluster of C CTAs (1 to 8) per unit.
+//
+// CTA r of a unit takes kPoolThreads * KPT consecutive tokens, warp w of it KPT
+// rows of 32 consecutive tokens, one token of a row per lane, so that votes
+// are loaded coalesced straight into registers (a row more at either end is
+// the pooling halo) and a neighbour d tokens away is one select and one
+// shuffle. The K-th largest key is found by one radix round over all keys
+// (11 bits: exponent and three bits of the fraction; only the first of a
+// warp's run of equal digits, which pooling makes, adds to the histogram);
+// the keys of its bucket, if at most kPoolCand, are then copied to every CTA
+// of the unit, which finishes on them alone, without the cluster. Larger
+// buckets (many equal votes) take further rounds over all keys. Kept tokens go
+// to a list in shared memory, from which the positions are written and the
+// rows gathered.
+//
+// Bound: latency (barriers, votes from L2) for few units, HBM of the gather for
+// many. One layer of 32 units, 32736 tokens, 1024 kept, takes 20.5 us; three
+// 11-bit rounds over 8-CTA clusters, every CTA reading all the histograms, and
+// a gather kernel took 41 us, and 256 units of 5991 tokens 98 us against 35.
+constexpr int kPoolThreads = 512;
+constexpr int kPoolWarps = kPoolThreads / 32;
+constexpr int kPoolMaxCta = 8;                       // CTAs per unit, at most
+constexpr int kPoolMaxP = kPoolMaxCta * kPoolThreads * 32;
+constexpr int kPoolCand = 2048;
 
-// Shared-memory word of staged vote j: one pad word after every 32.
-__device__ __forceinline__ int upad(int j) { return j + (j >> 5); }
+struct PoolSmem {
+  alignas(16) uint32_t hist[2][kBins];  // one per round parity; read 16 bytes at a time
+  uint32_t cand[kPoolCand];     // this CTA's bucket keys
+  uint32_t all[kPoolCand];      // the unit's bucket keys
+  int n_cand;                   // this CTA's
+  alignas(8) int cnt[2];        // this CTA's kept keys: above tau, equal to tau; read as a pair
+  int wsum[2][kPoolWarps];
+  int wgt[kPoolWarps], weq[kPoolWarps];
+  int digit[2][3];              // per round parity: digit, remaining, bucket keys
+};
+static_assert(offsetof(PoolSmem, cnt) % 8 == 0 && offsetof(PoolSmem, hist) % 16 == 0 &&
+                  sizeof(PoolSmem) % 16 == 0,
+              "vector reads of shared memory");
 
-// Pooling, radix select and ordered compaction of one unit's prefix tokens
-// (0 < K < P): writes out[0 .. K).
-__device__ __forceinline__ void select_unit_keys(const LayerGeom &g, const float *v, int32_t *out,
-                                                 int K, uint32_t *sm, int32_t *status) {
-  uint32_t *hist = sm;                                   // [kUWarps][kUBins]
-  int *tot = (int *)(hist + kUWarps * kUBins);           // [kUBins]
-  int *warp_tot = tot + kUBins;                          // [33]
-  int *ctl = warp_tot + 40;                              // [6]
-  float *vs = reinterpret_cast<float *>(sm + kUHead);    // [P + P / 32], padded
-  const int P = g.P;
+// The digit of the K-th largest (`remaining`-th) key from 2048 bin counts, four
+// per thread in descending order (c[q]: bin 2047 - 4 tid - q). Two barriers.
+__device__ __forceinline__ void find_digit(const int (&c)[4], int &remaining, int par,
+                                           PoolSmem &s, int &digit, int &bucket) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-
-  // Votes into shared memory (coalesced, sixteen loads of a thread in flight),
-  // with one pad word after every 32: thread t then reads its run of keys
-  // 32t .. 32t + 31 (and the pooling halo) without bank conflicts.
+  const int sum = c[0] + c[1] + c[2] + c[3];
+  int incl = sum;
 #pragma unroll
-  for (int i0 = 0; i0 < kUKeys; i0 += 16) {
-    float x[16];
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s.wsum[par][wid] = incl;
+  __syncthreads();
+  int before = lane < wid ? s.wsum[par][lane] : 0;
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int j = (i0 + u) * kUThreads + tid;
-      x[u] = j < P ? __ldcg(v + j) : 0.f;
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  int above = before + incl - sum;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (above < remaining && remaining <= above + c[q]) {
+      s.digit[par][0] = kBins - 1 - 4 * tid - q;
+      s.digit[par][1] = remaining - above;
+      s.digit[par][2] = c[q];
     }
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int j = (i0 + u) * kUThreads + tid;
-      if (j < P) vs[upad(j)] = x[u];
-    }
+    above += c[q];
   }
   __syncthreads();
-
-  // Pooled keys of this thread's tokens j0 .. j0 + 31 (window clipped to the
-  // prefix).
-  const int half = g.pool_kernel / 2;
-  const int j0 = tid * kUKeys;
-  uint32_t key[kUKeys];
-  if (g.pool_type == RIPPLE_POOL_MAX && half == 3) {
-    // the 7-wide max from the votes w = v[j0 - 3 .. j0 + 34] (-inf outside
-    // the prefix): b[i] = max(w[i .. i + 3]) and pooled(j0 + i) = max(b[i], b[i + 3])
-    float w[kUKeys + 6];
-#pragma unroll
-    for (int i = 0; i < kUKeys + 6; ++i) {
-      const int j = j0 - 3 + i;
-      w[i] = j >= 0 && j < P ? vs[upad(j)] : -INFINITY;
-    }
-    float a[kUKeys + 5];
-#pragma unroll
-    for (int i = 0; i < kUKeys + 5; ++i) a[i] = fmaxf(w[i], w[i + 1]);
-    float b[kUKeys + 3];
-#pragma unroll
-    for (int i = 0; i < kUKeys + 3; ++i) b[i] = fmaxf(a[i], a[i + 2]);
-#pragma unroll
-    for (int i = 0; i < kUKeys; ++i) key[i] = order_key(fmaxf(b[i], b[i + 3]));
-  } else {
-#pragma unroll
-    for (int i = 0; i < kUKeys; ++i) {
-      const int j = j0 + i;
-      float r = 0.f;
-      if (j < P) {
-        if (g.pool_type == RIPPLE_POOL_MAX) {
-          r = vs[upad(j)];
-          for (int d = 1; d <= half; ++d) {
-            if (j - d >= 0) r = fmaxf(r, vs[upad(j - d)]);
-            if (j + d < P) r = fmaxf(r, vs[upad(j + d)]);
-          }
-        } else if (g.pool_type == RIPPLE_POOL_AVG) {
-          float sum = 0.f;
-          int c = 0;
-          for (int d = -half; d <= half; ++d) {
-            const int pos = j + d;
-            if (pos >= 0 && pos < P) {
-              sum = __fadd_rn(sum, vs[upad(pos)]);
-              ++c;
-            }
-          }
-          r = __fdiv_rn(sum, (float)c);
-        } else {
-          r = vs[upad(j)];
-        }
-      }
-      key[i] = order_key(r);
-    }
-  }
-
-  // Radix select of the K-th largest key: up to 4 rounds of 8 bits from the
-  // top; once the bucket that holds it has at most kUCand keys, the rest is
-  // found among that bucket's keys directly (tau is then the same key).
-  uint32_t prefix = 0, mask = 0;
-  int remaining = K;
-  uint32_t tau = 0;
-  int take_eq = -1;
-  uint32_t *hw = hist + wid * kUBins;
-  for (int round = 0; round < 4; ++round) {
-    const int shift = 24 - 8 * round;
-#pragma unroll
-    for (int b = lane; b < kUBins; b += 32) hw[b] = 0;
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < kUKeys; ++i)
-      if (j0 + i < P && (key[i] & mask) == prefix) atomicAdd(&hw[(key[i] >> shift) & 255u], 1u);
-    __syncthreads();
-    if (tid < kUBins) {
-      int sum = 0;
-#pragma unroll 8
-      for (int w = 0; w < kUWarps; ++w) sum += (int)hist[w * kUBins + tid];
-      tot[tid] = sum;
-    }
-    __syncthreads();
-    if (wid == 0) {
-      // lane l holds digits 255 - 8l down to 248 - 8l
-      int c[8], sum = 0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        c[q] = tot[kUBins - 1 - 8 * lane - q];
-        sum += c[q];
-      }
-      int incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      int above = incl - sum;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (above < remaining && remaining <= above + c[q]) {
-          ctl[0] = kUBins - 1 - 8 * lane - q;
-          ctl[1] = remaining - above;
-          ctl[2] = c[q];
-        }
-        above += c[q];
-      }
-      if (lane == 0) ctl[3] = 0;
-    }
-    __syncthreads();
-    prefix |= (uint32_t)ctl[0] << shift;
-    mask |= 255u << shift;
-    remaining = ctl[1];
-    if (round < 3 && ctl[2] <= kUCand) {
-      // the bucket's keys into a list (any order); each of them counts the
-      // keys above and equal to it, and the one with remaining - 1 above
-      // and at least remaining above or equal is tau
-      uint32_t *cand = hist;  // the histograms are not needed any more
-#pragma unroll
-      for (int i = 0; i < kUKeys; ++i)
-        if (j0 + i < P && (key[i] & mask) == prefix) cand[atomicAdd(&ctl[3], 1)] = key[i];
-      __syncthreads();
-      const int nc = ctl[2];
-      if (tid < nc) {
-        const uint32_t x = cand[tid];
-        int above = 0, same = 0;
-        for (int c = 0; c < nc; ++c) {
-          const uint32_t y = cand[c];
-          above += y > x;
-          same += y == x;
-        }
-        if (above < remaining && remaining <= above + same) {
-          ctl[4] = (int)x;
-          ctl[5] = remaining - above;
-        }
-      }
-      __syncthreads();
-      tau = (uint32_t)ctl[4];
-      take_eq = ctl[5];
-      break;
-    }
-  }
-  if (take_eq < 0) {
-    tau = prefix;
-    take_eq = remaining;
-  }
-
-  // Ordered compaction: this thread's counts of keys above and equal to tau,
-  // one block scan over the threads (token order), then its kept tokens in
-  // order: every key above tau and the first take_eq keys equal to it.
-  int gt = 0, eq = 0;
-#pragma unroll
-  for (int i = 0; i < kUKeys; ++i) {
-    gt += j0 + i < P && key[i] > tau;
-    eq += j0 + i < P && key[i] == tau;
-  }
-  int total;
-  const int off = block_exclusive_scan((gt << 16) | eq, warp_tot, &total);
-  int g_rank = off >> 16, e_rank = off & 0xffff;
-#pragma unroll
-  for (int i = 0; i < kUKeys; ++i) {
-    const bool is_gt = j0 + i < P && key[i] > tau, is_eq = j0 + i < P && key[i] == tau;
-    if (is_gt || (is_eq && e_rank < take_eq))
-      out[guard(g_rank + min(e_rank, take_eq), 1, K, status)] = j0 + i;
-    g_rank += is_gt;
-    e_rank += is_eq;
-  }
+  digit = s.digit[par][0];
+  remaining = s.digit[par][1];
+  bucket = s.digit[par][2];
 }
 
-__global__ void __launch_bounds__(kUThreads, 1)
-    select_unit_kernel(LayerGeom g, const float *votes, const __grid_constant__ SelTable tab) {
-  extern __shared__ uint32_t sm[];
-  const int unit = blockIdx.x;  // over all layers of the launch
+// The value d tokens further on (d > 0) or back (d < 0) of a row `cur` between
+// its neighbour rows; |d| <= 31.
+__device__ __forceinline__ float ahead(float cur, float next, int d, int lane) {
+  return __shfl_sync(0xffffffffu, lane < d ? next : cur, lane + d);
+}
+__device__ __forceinline__ float behind(float prev, float cur, int d, int lane) {
+  return __shfl_sync(0xffffffffu, lane >= 32 - d ? prev : cur, lane - d);
+}
+
+template <int KPT>
+__global__ void __launch_bounds__(kPoolThreads, 2)
+    select_pool_kernel(LayerGeom g, const float *votes, const __grid_constant__ SelTable tab,
+                       int n_cta) {
+  extern __shared__ __align__(16) uint8_t pool_sm[];
+  PoolSmem &s = *reinterpret_cast<PoolSmem *>(pool_sm);
+  int *list = reinterpret_cast<int *>(pool_sm + sizeof(PoolSmem));  // kept tokens of this CTA
+  constexpr int kCtaTokens = kPoolThreads * KPT;
+  const int rank = n_cta > 1 ? (int)cluster_rank() : 0;
+  const int unit = blockIdx.x / n_cta;  // over all layers of the launch
   const int layer = unit / tab.upl;
   const int n_keep = tab.n_keep[layer];
   const int P = g.P, K = n_keep - g.W;
-  int32_t *out = tab.idx[layer] + (size_t)(unit % tab.upl) * n_keep;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int t0 = rank * kCtaTokens;                 // this CTA's first token
+  int first = 0, kept = 0;                          // its rows of the compact cache
 
-  for (int j = tid; j < g.W; j += kUThreads) out[K + j] = P + j;
-  if (K >= P) {
-    for (int t = tid; t < P; t += kUThreads) out[t] = t;
-  } else if (K > 0) {
-    select_unit_keys(g, votes + (size_t)unit * P, out, K, sm, tab.status);
-  }
-  if (tab.gather) {
-    // the unit's kept K and V rows into its compact cache rows 0 .. n_keep - 1:
-    // row_bytes / 16 consecutive threads copy one row 16 bytes each, four rows
-    // a thread in flight
-    __syncthreads();  // out[] of this CTA written
-    const int rb = tab.row_bytes, lpr = rb >> 4, rpp = kUThreads / lpr;
-    const int r_in = tid / lpr, c16 = (tid % lpr) * 16;
-    const size_t local = (size_t)(unit % tab.upl);
-    const uint8_t *kin = tab.k[layer] + local * g.T * rb;
-    const uint8_t *vin = tab.v[layer] + local * g.T * rb;
-    uint8_t *kout = tab.k_out[layer] + local * tab.cap[layer] * rb;
-    uint8_t *vout = tab.v_out[layer] + local * tab.cap[layer] * rb;
-    for (int r0 = 0; r0 < n_keep; r0 += 4 * rpp) {
-      uint4 xk[4], xv[4];
+  if (K <= 0 || K >= P) {
+    // window only, or every token: this CTA's share of the tokens in order
+    if (K > 0) {
+      first = min(t0, P);
+      kept = min(P, t0 + kCtaTokens) - first;
+      for (int i = tid; i < kept; i += kPoolThreads) list[i] = first + i;
+    }
+  } else {
+    // ---------------- pooled keys
+    const int w0 = t0 + wid * (KPT * 32);           // this warp's first token
+    const float *v = votes + (size_t)unit * P;
+    const float fill = g.pool_type == RIPPLE_POOL_MAX ? -INFINITY : 0.f;
+    float x[KPT + 2];  // rows -1 .. KPT
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = r0 + u * rpp + r_in;
-        if (r < n_keep) {
-          const long long t = guard(__ldcg(&out[r]), 1, g.T, tab.status);
-          xk[u] = __ldcs(reinterpret_cast<const uint4 *>(kin + t * rb + c16));
-          xv[u] = __ldcs(reinterpret_cast<const uint4 *>(vin + t * rb + c16));
+    for (int i = 0; i < KPT + 2; ++i) {
+      const int j = w0 + (i - 1) * 32 + lane;
+      x[i] = j >= 0 && j < P ? __ldcg(v + j) : fill;
+    }
+    for (int i = tid; i < kBins; i += kPoolThreads) s.hist[0][i] = 0;
+    const int half = g.pool_kernel / 2;
+    if (g.pool_type == RIPPLE_POOL_MAX && half > 0) {
+      // x[j] = max of the width tokens from j on, width the largest power of
+      // two within the window; the window is two of those runs
+      int width = 1;
+      for (; 2 * width <= g.pool_kernel; width *= 2) {
+#pragma unroll
+        for (int i = 0; i < KPT + 2; ++i)
+          x[i] = fmaxf(x[i], ahead(x[i], i < KPT + 1 ? x[i + 1] : fill, width, lane));
+      }
+      const int b = width - 1 - half;
+#pragma unroll
+      for (int i = KPT; i >= 1; --i)
+        x[i] = fmaxf(behind(x[i - 1], x[i], half, lane), behind(x[i - 1], x[i], b, lane));
+    } else if (g.pool_type == RIPPLE_POOL_AVG) {
+      // ascending positions from zero, like the definition's sum (positions
+      // outside the prefix add nothing)
+      float prev = x[0];
+#pragma unroll
+      for (int i = 1; i <= KPT; ++i) {
+        const float cur = x[i];
+        float sum = 0.f;
+        for (int d = half; d > 0; --d) sum = __fadd_rn(sum, behind(prev, cur, d, lane));
+        sum = __fadd_rn(sum, cur);
+        for (int d = 1; d <= half; ++d) sum = __fadd_rn(sum, ahead(cur, x[i + 1], d, lane));
+        const int j = w0 + (i - 1) * 32 + lane;
+        const int n = max(1, min(P - 1, j + half) - max(0, j - half) + 1);
+        x[i] = __fdiv_rn(sum, (float)n);
+        prev = cur;
+      }
+    }
+    uint32_t key[KPT];
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) key[i] = order_key(x[i + 1]);
+    const int live = P - w0 - lane;  // key[i] is a token's if 32 i < live
+
+    // ---------------- the K-th largest key
+    // Rounds over the 31 bits below the sign bit, for the keys that have it
+    // (votes >= 0; the others, and zeros, count in the lowest bin of the first
+    // round); if the threshold falls into that bin, the search starts over on
+    // all 32 bits.
+    uint32_t prefix = 0, mask = 0;
+    int remaining = K;
+    bool full = false;
+    auto shift_of = [&](int level) { return level == 2 ? 0 : (level == 1 ? 9 : 20) + (full ? 1 : 0); };
+    auto dmask_of = [&](int level) { return level < 2 ? 2047u : full ? 1023u : 511u; };
+    __syncthreads();  // the first histogram is clear
+    for (int it = 0, level = 0; level < 3; ++it, ++level) {
+      uint32_t *hist = s.hist[it & 1];
+      const int shift = shift_of(level);
+      const uint32_t dmask = dmask_of(level);
+#pragma unroll
+      for (int i = 0; i < KPT; ++i) {
+        const bool in = 32 * i < live && (key[i] & mask) == prefix;
+        uint32_t d = key[i] >> shift & dmask;
+        if (level == 0 && !full && !(key[i] >> 31)) d = 0;
+        // the first lane of a run of equal digits adds the run's length
+        if (!in) d = 0xffffffffu;
+        const uint32_t up = __shfl_up_sync(0xffffffffu, d, 1);
+        const bool head = lane == 0 || up != d;
+        const uint32_t heads = __ballot_sync(0xffffffffu, head);
+        if (head && in) {
+          const uint32_t later = lane == 31 ? 0u : heads >> (lane + 1);
+          atomicAdd(&hist[d], (uint32_t)(later ? __ffs(later) : 32 - lane));
         }
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = r0 + u * rpp + r_in;
-        if (r < n_keep) {
-          *reinterpret_cast<uint4 *>(kout + (size_t)r * rb + c16) = xk[u];
-          *reinterpret_cast<uint4 *>(vout + (size_t)r * rb + c16) = xv[u];
+      const int d0 = kBins - 1 - 4 * tid;  // this thread's bins d0 .. d0 - 3
+      int c[4] = {0, 0, 0, 0};
+      if (n_cta > 1)
+        cluster_sync_all();  // every CTA's histogram of this round is complete
+      else
+        __syncthreads();
+      for (int r = 0; r < n_cta; ++r) {
+        const uint4 h = n_cta > 1 ? ld_cluster_v4(cluster_addr(hist + d0 - 3, r))
+                                  : *reinterpret_cast<const uint4 *>(hist + d0 - 3);
+        c[0] += (int)h.w;
+        c[1] += (int)h.z;
+        c[2] += (int)h.y;
+        c[3] += (int)h.x;
+      }
+      // the other histogram, for the next round (its readers have passed this
+      // round's barrier)
+      for (int i = tid; i < kBins; i += kPoolThreads) s.hist[(it & 1) ^ 1][i] = 0;
+      if (tid == 0) s.n_cand = 0;
+      int digit, bucket;
+      find_digit(c, remaining, it & 1, s, digit, bucket);
+      if (level == 0 && !full) {
+        if (digit == 0) {
+          full = true;
+          remaining = K;
+          level = -1;
+          continue;
         }
+        prefix = mask = 0x80000000u;
+      }
+      prefix |= (uint32_t)digit << shift;
+      mask |= dmask << shift;
+      if (level == 2 || bucket > kPoolCand) continue;
+      // ---------------- the bucket's keys, to every CTA of the unit
+#pragma unroll
+      for (int i = 0; i < KPT; ++i) {
+        const bool in = 32 * i < live && (key[i] & mask) == prefix;
+        const uint32_t m = __ballot_sync(0xffffffffu, in);
+        if (m == 0) continue;
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&s.n_cand, __popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+        if (in) s.cand[at] = key[i];
+      }
+      const uint32_t *all = s.cand;
+      if (n_cta > 1) {
+        cluster_sync_all();
+        int off = 0;
+        for (int r = 0; r < n_cta; ++r) {
+          const int n = (int)ld_cluster_u32(cluster_addr(&s.n_cand, r));
+          for (int i = tid; i < n; i += kPoolThreads)
+            s.all[off + i] = ld_cluster_u32(cluster_addr(&s.cand[i], r));
+          off += n;
+        }
+        all = s.all;
+      }
+      __syncthreads();
+      // the remaining rounds on those keys alone
+      for (++it, ++level; level < 3; ++it, ++level) {
+        uint32_t *h2 = s.hist[it & 1];
+        const int sh = shift_of(level);
+        const uint32_t dm = dmask_of(level);
+        for (int i = tid; i < bucket; i += kPoolThreads) {
+          const uint32_t u = all[i];
+          if ((u & mask) == prefix) atomicAdd(&h2[u >> sh & dm], 1u);
+        }
+        __syncthreads();
+        const uint4 h = *reinterpret_cast<const uint4 *>(h2 + d0 - 3);
+        const int cc[4] = {(int)h.w, (int)h.z, (int)h.y, (int)h.x};
+        for (int i = tid; i < kBins; i += kPoolThreads) s.hist[(it & 1) ^ 1][i] = 0;
+        int n_eq;
+        find_digit(cc, remaining, it & 1, s, digit, n_eq);
+        prefix |= (uint32_t)digit << sh;
+        mask |= dm << sh;
+      }
+    }
+    const uint32_t tau = prefix;
+    const int take_eq = remaining;  // keys equal to tau that are kept (>= 1)
+
+    // ---------------- ordered compaction into the list
+    int cgt = 0, ceq = 0;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+      cgt += __popc(__ballot_sync(0xffffffffu, 32 * i < live && key[i] > tau));
+      ceq += __popc(__ballot_sync(0xffffffffu, 32 * i < live && key[i] == tau));
+    }
+    if (lane == 0) {
+      s.wgt[wid] = cgt;
+      s.weq[wid] = ceq;
+    }
+    __syncthreads();
+    int gt = lane < kPoolWarps ? s.wgt[lane] : 0, eq = lane < kPoolWarps ? s.weq[lane] : 0;
+    int gt_w = lane < wid ? gt : 0, eq_w = lane < wid ? eq : 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      gt += __shfl_xor_sync(0xffffffffu, gt, o);
+      eq += __shfl_xor_sync(0xffffffffu, eq, o);
+      gt_w += __shfl_xor_sync(0xffffffffu, gt_w, o);
+      eq_w += __shfl_xor_sync(0xffffffffu, eq_w, o);
+    }
+    int gt_c = 0, eq_c = 0;  // of the lower-ranked CTAs
+    if (n_cta > 1) {
+      if (tid == 0) {
+        s.cnt[0] = gt;
+        s.cnt[1] = eq;
+      }
+      cluster_sync_all();  // every CTA's counts are published
+      for (int r = 0; r < rank; ++r) {
+        const uint2 c = ld_cluster_v2(cluster_addr(s.cnt, r));
+        gt_c += (int)c.x;
+        eq_c += (int)c.y;
+      }
+      cluster_arrive();  // this CTA reads no other's shared memory any more
+    }
+    first = gt_c + min(eq_c, take_eq);
+    kept = gt_c + gt + min(eq_c + eq, take_eq) - first;
+    int gt_before = gt_c + gt_w, eq_before = eq_c + eq_w;
+    const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+      const bool is_gt = 32 * i < live && key[i] > tau, is_eq = 32 * i < live && key[i] == tau;
+      const uint32_t bg = __ballot_sync(0xffffffffu, is_gt);
+      const uint32_t be = __ballot_sync(0xffffffffu, is_eq);
+      if ((bg | be) == 0) continue;
+      const int g_rank = gt_before + __popc(bg & below), e_rank = eq_before + __popc(be & below);
+      if (is_gt || (is_eq && e_rank < take_eq))
+        list[guard(g_rank + min(e_rank, take_eq) - first, 1, kCtaTokens, tab.status)] =
+            w0 + i * 32 + lane;
+      gt_before += __popc(bg);
+      eq_before += __popc(be);
+    }
+  }
+
+  // ---------------- positions and rows; the last CTA has the window as well
+  const int window = rank == n_cta - 1 ? g.W : 0;
+  if (window > 0) {
+    if (kept == 0) first = max(K, 0);
+    for (int i = tid; i < window; i += kPoolThreads) list[kept + i] = P + i;
+  }
+  const int rows = kept + window;
+  __syncthreads();
+  const int local = unit % tab.upl;
+  int32_t *out = tab.idx[layer] + (size_t)local * n_keep + first;
+  for (int i = tid; i < rows; i += kPoolThreads) out[i] = list[i];
+  // row_bytes / 16 consecutive threads copy one row 16 bytes each, four rows a
+  // thread in flight
+  const int rb = tab.row_bytes, lpr = rb >> 4, rpp = kPoolThreads / lpr;
+  const int r_in = tid / lpr, c16 = (tid % lpr) * 16;
+  const uint8_t *kin = tab.k[layer] + (size_t)local * g.T * rb;
+  const uint8_t *vin = tab.v[layer] + (size_t)local * g.T * rb;
+  uint8_t *kout = tab.k_out[layer] + ((size_t)local * tab.cap[layer] + first) * rb;
+  uint8_t *vout = tab.v_out[layer] + ((size_t)local * tab.cap[layer] + first) * rb;
+  for (int r0 = 0; r0 < rows; r0 += 4 * rpp) {
+    uint4 xk[4], xv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + u * rpp + r_in;
+      if (r < rows) {
+        const long long t = guard(list[r], 1, g.T, tab.status);
+        xk[u] = __ldcs(reinterpret_cast<const uint4 *>(kin + t * rb + c16));
+        xv[u] = __ldcs(reinterpret_cast<const uint4 *>(vin + t * rb + c16));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + u * rpp + r_in;
+      if (r < rows) {
+        *reinterpret_cast<uint4 *>(kout + (size_t)r * rb + c16) = xk[u];
+        *reinterpret_cast<uint4 *>(vout + (size_t)r * rb + c16) = xv[u];
       }
     }
   }
+  // no CTA leaves while others may still read its shared memory
+  if (n_cta > 1 && K > 0 && K < P) cluster_wait();
 }
 
 }  // namespace
 
-cudaError_t launch_select(const LayerGeom &g, int n_layers, const float *votes,
-                          const CompressWs &ws, const int *n_keep, int32_t *const *idx,
-                          int32_t *status, cudaStream_t st, const GatherArgs *gather,
-                          bool *gathered) {
-  if (n_layers < 1 || n_layers > kCompressMaxLayers) return cudaErrorInvalidValue;
-  if (gathered != nullptr) *gathered = false;
-  // One CTA per unit once the launch has enough units to fill the GPU;
-  // fewer units (a single layer) are spread over 8-CTA clusters instead.
-  if (g.P <= kUMaxP && (long long)g.units * n_layers >= kUMinUnits) {
-    SelTable tab;
-    tab.upl = g.units;
-    tab.status = status;
-    tab.gather = gather != nullptr && gathered != nullptr;
-    tab.row_bytes = g.D * (g.dtype == RIPPLE_F32 ? 4 : 2);
-    for (int l = 0; l < n_layers; ++l) {
-      tab.n_keep[l] = n_keep[l];
-      tab.idx[l] = idx[l];
-      if (tab.gather) {
-        tab.k[l] = (const uint8_t *)gather->k[l];
-        tab.v[l] = (const uint8_t *)gather->v[l];
-        tab.k_out[l] = (uint8_t *)gather->k_out[l];
-        tab.v_out[l] = (uint8_t *)gather->v_out[l];
-        tab.cap[l] = gather->cap[l];
-      }
-    }
-    const size_t smem = sizeof(uint32_t) * ((size_t)kUHead + g.P + g.P / 32 + 1);
-    cudaError_t e = cudaFuncSetAttribute(select_unit_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    select_unit_kernel<<<g.units * n_layers, kUThreads, smem, st>>>(g, votes, tab);
-    count_launches(1);
-    e = cudaGetLastError();
-    if (e == cudaSuccess && gathered != nullptr) *gathered = tab.gather != 0;
-    return e;
-  }
+namespace {
+
+// Prefixes beyond kPoolMaxP: 8-CTA clusters with their keys in shared memory, or
+// one CTA per unit with its keys in global scratch.
+cudaError_t select_long(const LayerGeom &g, int n_layers, const float *votes, const CompressWs &ws,
+                        const int *n_keep, int32_t *const *idx, int32_t *status,
+                        cudaStream_t st) {
   const int per_cta = ((g.P + kCluster - 1) / kCluster + 31) & ~31;
-  if (per_cta <= kCMaxKeys && (long long)g.units * n_layers * kCluster <= 0x7fffffff) {
+  if (g.P <= kSelectClusterMaxP) {
     SelTable tab;
     tab.upl = g.units;
     tab.status = status;
-    tab.gather = 0;
     for (int l = 0; l < n_layers; ++l) {
       tab.n_keep[l] = n_keep[l];
       tab.idx[l] = idx[l];
@@ -830,30 +898,96 @@ cudaError_t launch_select(const LayerGeom &g, int n_layers, const float *votes,
     return cudaGetLastError();
   }
   // Very long prefixes: one CTA per unit, layer by layer.
-  const int in_smem = g.P <= kSelectSmemKeys;
-  const size_t smem = sizeof(uint32_t) * (kBins + kCtrlWords + (in_smem ? g.P : 0));
-  cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = sizeof(uint32_t) * (kBins + kCtrlWords);
   for (int l = 0; l < n_layers; ++l) {
     select_kernel<<<g.units, kThreads, smem, st>>>(g, votes + (size_t)l * g.units * g.P, ws.keys,
-                                                   n_keep[l], in_smem, idx[l], status);
+                                                   n_keep[l], idx[l], status);
     count_launches(1);
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-__global__ void iota_kernel(int T, int32_t *idx) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x)
-    idx[(size_t)blockIdx.y * T + t] = t;
+// Keys per thread (8, 16 or 32; 512 threads a CTA) and CTAs per unit: 16, or
+// 8 where they fill the CTA (P <= 4096) or where 16 leave three quarters of
+// the SMs idle, or 32 where there are CTAs for many waves, which saves cluster
+// barriers. Measured with 8 / 16 / 32 keys: one layer of 32 units and 32736
+// tokens 26.6 / 20.5 / 27.1 us, 8 units of 8160 tokens (with scoring) 39.9 /
+// 43.5 / 52.3 us, 256 units of 5991 tokens (with scoring) 143 / 136 / 166 us,
+// 1024 units of 32736 tokens (with scoring) 2872 / 2663 / 2630 us.
+void pool_shape(int P, int n_units, int *kpt, int *n_cta) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  auto ctas = [&](int keys) {
+    int n = 1;
+    while (n * kPoolThreads * keys < P) n *= 2;
+    return n;
+  };
+  const long long at16 = (long long)n_units * ctas(16);
+  if (P <= kPoolThreads * 8 || (ctas(8) <= kPoolMaxCta && at16 * 4 <= sms))
+    *kpt = 8;
+  else
+    *kpt = ctas(16) > kPoolMaxCta || (P > kPoolThreads * 16 && at16 >= 8LL * sms) ? 32 : 16;
+  *n_cta = ctas(*kpt);
 }
 
-cudaError_t launch_iota(const LayerGeom &g, int32_t *idx, cudaStream_t st) {
-  iota_kernel<<<dim3((g.T + 255) / 256, g.units), 256, 0, st>>>(g.T, idx);
+template <int KPT>
+cudaError_t launch_pool(const LayerGeom &g, int n_units, const float *votes, const SelTable &tab,
+                        int n_cta, cudaStream_t st) {
+  const size_t smem = sizeof(PoolSmem) + sizeof(int) * (kPoolThreads * KPT + 64);
+  cudaError_t e = cudaFuncSetAttribute(select_pool_kernel<KPT>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_units * n_cta);
+  cfg.blockDim = dim3(kPoolThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = n_cta;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, select_pool_kernel<KPT>, g, votes, tab, n_cta);
   count_launches(1);
-  return cudaGetLastError();
+  return e;
+}
+
+}  // namespace
+
+cudaError_t launch_select(const LayerGeom &g, int n_layers, const float *votes,
+                          const CompressWs &ws, const int *n_keep, int32_t *const *idx,
+                          int32_t *status, cudaStream_t st, const GatherArgs &gather) {
+  if (n_layers < 1 || n_layers > kCompressMaxLayers) return cudaErrorInvalidValue;
+  const int n_units = g.units * n_layers;
+  if (g.P <= kPoolMaxP) {
+    SelTable tab;
+    tab.upl = g.units;
+    tab.status = status;
+    tab.row_bytes = g.D * (g.dtype == RIPPLE_F32 ? 4 : 2);
+    for (int l = 0; l < n_layers; ++l) {
+      tab.n_keep[l] = n_keep[l];
+      tab.idx[l] = idx[l];
+      tab.k[l] = (const uint8_t *)gather.k[l];
+      tab.v[l] = (const uint8_t *)gather.v[l];
+      tab.k_out[l] = (uint8_t *)gather.k_out[l];
+      tab.v_out[l] = (uint8_t *)gather.v_out[l];
+      tab.cap[l] = gather.cap[l];
+    }
+    int kpt, n_cta;
+    pool_shape(g.P, n_units, &kpt, &n_cta);
+    return kpt == 8    ? launch_pool<8>(g, n_units, votes, tab, n_cta, st)
+           : kpt == 16 ? launch_pool<16>(g, n_units, votes, tab, n_cta, st)
+                       : launch_pool<32>(g, n_units, votes, tab, n_cta, st);
+  }
+  // Longer prefixes: selection, then the gather of all layers.
+  cudaError_t e = select_long(g, n_layers, votes, ws, n_keep, idx, status, st);
+  if (e != cudaSuccess) return e;
+  return launch_gather(g, n_layers, gather.k, gather.v, (const int32_t *const *)idx, n_keep,
+                       gather.k_out, gather.v_out, gather.cap, status, st);
 }
 
 }  // namespace ripple

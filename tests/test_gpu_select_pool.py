@@ -1,0 +1,78 @@
+"""Selection with the gather over prefixes of up to 131072 tokens (and just
+beyond, where another kernel takes over): bit-exact against the oracle on shared
+votes, at prefix lengths around the edges of a warp's rows, of a CTA and of a
+cluster, few and many units, every pooling; ties, equal votes (the radix bucket
+does not fit the candidate list), zeros at the threshold (the search starts over
+on all bits), and every budget edge."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import ripple_oracle as O
+from paper_2608_08684_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _run(lib, votes, budget, w, pool, kernel, check):
+    units, P = votes.shape
+    g = torch.Generator(device=DEV).manual_seed(P + units)
+    k = torch.randn(1, units, P + w, 64, dtype=torch.bfloat16, device=DEV, generator=g)
+    v = torch.randn(1, units, P + w, 64, dtype=torch.bfloat16, device=DEV, generator=g)
+    desc = lib.layer_desc(1, units, units, 64, P + w, w, kernel, pool, torch.bfloat16)
+    n = lib.ripple_keep_count(budget, P + w, w)
+    k_out = torch.zeros(1, units, n + 1, 64, dtype=torch.bfloat16, device=DEV)
+    v_out = torch.zeros_like(k_out)
+    idx = torch.full((units * n,), -1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(lib.ripple_compress_workspace_bytes(desc), dtype=torch.uint8, device=DEV)
+    assert lib.ripple_select_layer(desc, budget, votes.to(DEV), k, v, k_out, v_out, idx, ws) == n
+    torch.cuda.synchronize()
+    got = idx.view(units, n).cpu().numpy()
+    for u in check:
+        want = O.select_tokens(O.pool_scores(votes[u].numpy(), kernel, pool), n, P + w, w)
+        np.testing.assert_array_equal(got[u], want)
+        at = torch.from_numpy(want).long().to(DEV)
+        assert torch.equal(k_out[0, u, :n], k[0, u][at])
+        assert torch.equal(v_out[0, u, :n], v[0, u][at])
+    assert not k_out[0, :, n].any()  # rows past the kept ones are left alone
+
+
+@pytest.mark.parametrize("P", [1, 31, 33, 255, 257, 4095, 4096, 4097, 8191, 8193, 16385, 32768,
+                               32769, 65537, 131071, 131072, 131073, 212992, 212993])
+def test_prefix_lengths(lib, P):
+    votes = synth.synthetic_votes(900 + P, 2, P, 0)
+    _run(lib, votes, 8 + max(1, P // 7), 8, "max", 7, range(2))
+
+
+@pytest.mark.parametrize("units,P", [(600, 700), (1300, 300), (160, 9000), (620, 8200)])
+def test_many_units(lib, units, P):
+    votes = synth.synthetic_votes(950 + P, units, P, 200)
+    _run(lib, votes, 8 + P // 5, 8, "max", 7, [0, units // 2, units - 1])
+
+
+@pytest.mark.parametrize("pool,kernel", [("max", 1), ("max", 3), ("max", 5), ("max", 13),
+                                         ("max", 31), ("avg", 3), ("avg", 5), ("avg", 31),
+                                         ("none", 7)])
+@pytest.mark.parametrize("P", [20, 1000, 9001])
+def test_pooling(lib, pool, kernel, P):
+    votes = synth.synthetic_votes(970 + P, 2, P, 50 if kernel == 5 else 0)
+    _run(lib, votes, 8 + P // 3, 8, pool, kernel, range(2))
+
+
+@pytest.mark.parametrize("P", [500, 9001, 40000])
+@pytest.mark.parametrize("kind", ["equal", "zeros", "mostly_zero", "two_values", "spread"])
+def test_vote_distributions(lib, kind, P):
+    r = np.random.default_rng(P)
+    x = {"equal": np.full((2, P), 0.25), "zeros": np.zeros((2, P)),
+         "mostly_zero": np.where(r.random((2, P)) < 0.01, r.random((2, P)), 0.0),
+         "two_values": np.where(r.random((2, P)) < 0.5, 1.0, 1.0 + 2.0 ** -20),
+         "spread": np.exp(30 * (r.random((2, P)) - 0.9))}[kind]
+    votes = torch.from_numpy(x.astype(np.float32))
+    _run(lib, votes, 8 + P // 3, 8, "max", 3, range(2))
+
+
+@pytest.mark.parametrize("budget", [0, 8, 9, 8999, 9007, 9008, 9009, 10**7])
+def test_budget_edges(lib, budget):
+    votes = synth.synthetic_votes(990, 2, 9000, 0)
+    _run(lib, votes, budget, 8, "max", 7, range(2))
