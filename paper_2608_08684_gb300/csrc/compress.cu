@@ -75,6 +75,20 @@ static bool make_geom(const ripple_layer_desc *d, LayerGeom *g) {
   return true;
 }
 
+// Scoring of n_scored layers by the kernel for their shape (launch_score_tc1's
+// arguments).
+static cudaError_t launch_score(const LayerGeom &g, int n_slots, const int *slots, int n_scored,
+                                const void *const *q_win, const void *const *k,
+                                const CompressWs &ws, float *votes, int32_t *status,
+                                cudaStream_t st, const void *const *v = nullptr,
+                                float *const *o_win = nullptr) {
+  if (score_tc1_supported(g))
+    return launch_score_tc1(g, n_slots, slots, n_scored, q_win, k, ws, votes, status, st, v, o_win);
+  if (score_tc_supported(g))
+    return launch_score_tc(g, n_slots, slots, n_scored, q_win, k, ws, votes, status, st);
+  return launch_score_simt(g, n_slots, slots, n_scored, q_win, k, ws, votes, status, st);
+}
+
 }  // namespace ripple
 
 using namespace ripple;
@@ -120,12 +134,7 @@ extern "C" ripple_status ripple_compress_layer(const ripple_layer_desc *desc, in
   float *votes = scores_out ? scores_out : ws.votes;
   if (g.P > 0 && (!keep_all || scores_out)) {
     const int slot = 0;
-    cudaError_t e = score_tc1_supported(g)
-                        ? launch_score_tc1(g, 1, &slot, 1, &q_win, &k, ws, votes, dev_status, st)
-                    : score_tc_supported(g)
-                        ? launch_score_tc(g, 1, &slot, 1, &q_win, &k, ws, votes, dev_status, st)
-                        : launch_score_simt(g, q_win, k, ws, votes, dev_status, st);
-    RIPPLE_CUDA_TRY(e);
+    RIPPLE_CUDA_TRY(launch_score(g, 1, &slot, 1, &q_win, &k, ws, votes, dev_status, st));
   }
   const GatherArgs ga{&k, &v, &k_out, &v_out, &cap};
   RIPPLE_CUDA_TRY(launch_select(g, 1, votes, ws, &n, &idx_out, dev_status, st, ga));
@@ -237,11 +246,10 @@ static ripple_status compress_layers_impl(
   cudaStream_t st = (cudaStream_t)stream;
   const GatherArgs ga{k_host, v_host, k_out_host, v_out_host, cap};
   if (g.P > 0) {
-    // Scoring: on the tensor cores (bf16) every layer that needs votes in one
-    // launch; on the CUDA cores (fp32) layer by layer, the scratch of the
-    // multi-layer workspace reused. Each layer's votes go to its part of the
-    // vote array. A layer that keeps every token needs no votes (the selection
-    // writes 0..T-1 for it), unless its window rows' output is wanted.
+    // Scoring: every layer that needs votes in one go, each layer's votes in
+    // its part of the vote array. A layer that keeps every token needs none
+    // (the selection writes 0..T-1 for it), unless its window rows' output is
+    // wanted.
     int slots[RIPPLE_COMPRESS_MAX_LAYERS];
     const void *qs[RIPPLE_COMPRESS_MAX_LAYERS];
     const void *ks[RIPPLE_COMPRESS_MAX_LAYERS];
@@ -253,19 +261,9 @@ static ripple_status compress_layers_impl(
       ks[n_scored] = k_host[l];
       ++n_scored;
     }
-    if (n_scored > 0 && score_tc1_supported(g)) {
-      RIPPLE_CUDA_TRY(launch_score_tc1(g, n_layers, slots, n_scored, qs, ks, ws, ws.votes,
-                                       dev_status, st, o_win_host ? v_host : nullptr,
-                                       o_win_host));
-    } else if (n_scored > 0 && score_tc_supported(g)) {
-      RIPPLE_CUDA_TRY(launch_score_tc(g, n_layers, slots, n_scored, qs, ks, ws, ws.votes,
-                                      dev_status, st));
-    } else {
-      for (int i = 0; i < n_scored; ++i)
-        RIPPLE_CUDA_TRY(launch_score_simt(g, qs[i], ks[i], ws,
-                                          ws.votes + (size_t)slots[i] * g.units * g.P, dev_status,
-                                          st));
-    }
+    if (n_scored > 0)
+      RIPPLE_CUDA_TRY(launch_score(g, n_layers, slots, n_scored, qs, ks, ws, ws.votes, dev_status,
+                                   st, o_win_host ? v_host : nullptr, o_win_host));
   }
   RIPPLE_CUDA_TRY(launch_select(g, n_layers, ws.votes, ws, n, idx_out_host, dev_status, st, ga));
   for (int l = 0; l < n_layers; ++l) n_keep_host[l] = n[l];

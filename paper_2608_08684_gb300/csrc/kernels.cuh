@@ -45,8 +45,10 @@ struct CompressWs {
 };
 CompressWs carve_compress_ws(const LayerGeom &g, void *base);
 
-// Scoring on the fp32 pipes (fp32 caches).
-cudaError_t launch_score_simt(const LayerGeom &g, const void *q_win, const void *k,
+// Scoring on the fp32 pipes (fp32 caches), several layers in one launch as
+// launch_score_tc1 below.
+cudaError_t launch_score_simt(const LayerGeom &g, int n_slots, const int *slots, int n_scored,
+                              const void *const *q_win, const void *const *k,
                               const CompressWs &ws, float *votes, int32_t *status,
                               cudaStream_t st);
 // Scoring on the tensor cores for 129 to 256 window rows (bf16, d = 64 or 128),
