@@ -215,6 +215,16 @@ __device__ __forceinline__ void bulk_wait_read_all() {
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
+// Programmatic dependent launches. A kernel that may be followed by a dependent
+// lets it take its place as early as SMs are free; a dependent reads and
+// writes nothing of the stream's earlier kernels before the wait returns, which
+// it does once they have completed and their writes are visible (at once when
+// it was launched as an ordinary kernel).
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 }  // namespace ripple
 
 // Host-side launch check used by the entry points.

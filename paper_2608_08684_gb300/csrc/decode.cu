@@ -1101,7 +1101,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
   // step's CTAs take SMs as this grid's CTAs leave, and wait here until the
   // previous grid has completed and its writes (lengths, appended rows,
   // counters) are visible.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_launch_dependents();
   if (warp == 0) prefetch_first_item<Tin, D, G>(p, lane);
   if (tid == 32) {
     for (int i = 0; i < C::STAGES; ++i) {
@@ -1116,7 +1116,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
     s.init_seen = 0;
     fence_mbar_init();
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   // CTA 0 zeroes this call's counters (the workspace may hold anything),
   // then raises the init flag; the other CTAs use no counter before they see
   // it (wait_init).

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kThreads) score_pass1_simt(LayerGeom g,
                                                              const __grid_constant__ SimtTable t) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   SimtSmem<D> &s = *reinterpret_cast<SimtSmem<D> *>(smem_raw);
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_launch_dependents();
   const int unit = blockIdx.y, chunk = blockIdx.x;
   const int layer = unit / g.units, local = unit % g.units;
   const int key0 = chunk * kScoreChunk;
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kThreads) score_pass2_simt(LayerGeom g,
   const float *q_unit = t.q[layer] + (size_t)local * g.R * D;
   load_transposed<D, kRows>(q_unit, g.R, s.q);
   // the inputs were there before pass 1 began; its results from here on
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   for (int r = threadIdx.x; r < 256; r += kThreads)
     ln[r] = r >= g.R ? INFINITY  // rows past the last count for nothing
             : fused_merge ? merged_row(t, g.R, unit, r)

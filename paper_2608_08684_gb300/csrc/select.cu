@@ -609,6 +609,7 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int t0 = rank * kCtaTokens;                 // this CTA's first token
   int first = 0, kept = 0;                          // its rows of the compact cache
+  pdl_wait();  // the votes
 
   if (K <= 0 || K >= P) {
     // window only, or every token: this CTA's share of the tokens in order
@@ -945,12 +946,14 @@ cudaError_t launch_pool(const LayerGeom &g, int n_units, const float *votes, con
   cfg.blockDim = dim3(kPoolThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = n_cta;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   e = cudaLaunchKernelEx(&cfg, select_pool_kernel<KPT>, g, votes, tab, n_cta);
   count_launches(1);
   return e;

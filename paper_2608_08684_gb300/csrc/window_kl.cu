@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(kKlThreads, 1)
 template <bool kCached>
 __global__ void __launch_bounds__(kKlMergeWarps * 32)
     kl_merge_kernel(const __grid_constant__ KlParams P) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * kKlMergeWarps + (threadIdx.x >> 5);
   if (row >= P.n_sets * P.n_pos) return;
