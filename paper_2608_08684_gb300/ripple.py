@@ -142,9 +142,21 @@ def _ptr(t):
     return t.data_ptr()
 
 
+# The current device's current stream without a torch.cuda.Stream object, which
+# took a third of a call's time in this module (3.0 of 9.2 us, ripple_decode_attn).
+try:
+    from torch._C import _cuda_getCurrentRawStream, _cuda_getDevice
+except ImportError:
+    def _current_stream():
+        return torch.cuda.current_stream().cuda_stream
+else:
+    def _current_stream():
+        return _cuda_getCurrentRawStream(_cuda_getDevice())
+
+
 def _stream(stream):
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     return getattr(stream, "cuda_stream", stream)
 
 
