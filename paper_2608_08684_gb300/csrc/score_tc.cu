@@ -50,13 +50,15 @@ constexpr int kTile = 128;                      // keys per tile
 constexpr int kHalfBytes = kTile * 64 * 2;      // 64 bf16 columns of 128 rows: 16 KB
 constexpr int kThreads = 352;
 constexpr int kPubSlots = 2;
-// Items of at least 64 key tiles: with every layer of a call in one launch the
-// pipeline's fill and drain no longer favour small items, and fewer items
-// mean fewer partial statistics to publish and merge (80 layers of the 70B
-// shape: 12.36 / 12.07 / 11.76 / 11.59 / 11.58 / 11.53 / 13.11 ms with items
-// of 14 / 18 / 32 / 64 / 128 / 256 / 1024 tiles; one item per unit leaves the
-// last wave of units short).
-constexpr int kMinTilesPerItem = 64;
+// A unit is cut into items of 8 tiles (up to 64 tiles) or 16, but at most 16
+// items: more partial statistics take the one publisher that merges them too
+// long, and fewer items leave small calls on few SMs. One 8k-token layer of 8
+// units took 161 / 63 / 54 / 49 us with items of 64 / 16 / 12 / 8 tiles, 16
+// layers of 256 tiles 628 / 600 / 641 us with 64 / 16 / 15, 16 layers of 1024
+// tiles 2181 / 2207 / 2267 us with 64 / 57 / 86 (16 / 18 / 12 items).
+constexpr int kTilesPerItem = 16, kTilesPerItemShort = 8;
+constexpr int kShortTiles = 64;
+constexpr int kMaxItems = 16;
 
 
 // ------------------------------------------------------------ work list
@@ -683,11 +685,12 @@ cudaError_t launch_d(const LayerGeom &g, int n_slots, const int *slots, int n_sc
   p.R = g.R;
   p.n_tiles1 = (g.T + kTile - 1) / kTile;
   p.n_tiles2 = (g.P + kTile - 1) / kTile;
-  // Tiles per item: at least kMinTilesPerItem (hand-offs are per item), and
-  // enough that a unit has no more items than there are SMs (deadlock-free
-  // schedule, see the header comment).
-  const int tpi_min = (p.n_tiles1 + sms - 1) / sms;
-  p.tpi = tpi_min > kMinTilesPerItem ? tpi_min : kMinTilesPerItem;
+  // (and no more items than SMs: deadlock-free schedule, see the header comment)
+  const int per = p.n_tiles1 <= kShortTiles ? kTilesPerItemShort : kTilesPerItem;
+  const int items = (p.n_tiles1 + per - 1) / per;
+  p.n_ch = items < kMaxItems ? items : kMaxItems;
+  p.n_ch = p.n_ch < sms ? p.n_ch : sms;
+  p.tpi = (p.n_tiles1 + p.n_ch - 1) / p.n_ch;
   p.n_ch = (p.n_tiles1 + p.tpi - 1) / p.tpi;
   p.total_items = p.units * p.n_ch;
   p.scale2 = g.scale2;

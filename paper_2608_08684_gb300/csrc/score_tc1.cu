@@ -64,7 +64,13 @@ constexpr int kHalfBytes = kTile * 64 * 2;      // one TMA box: 64 dims of 128 k
 constexpr int kThreads = 352;
 constexpr int kLag = 1;                         // pass 2 of item k runs in step k + kLag
 constexpr int kPubSlots = 2;
-constexpr int kMinTilesPerItem = 9;
+// Key tiles of an item, at most. Two items a CTA stay in L2 between the passes,
+// and a smaller item pays its queries, hand-overs and merge more often: 32
+// layers of 8 units and 64 tiles took 273 / 235 / 207 / 201 / 222 / 221 us with
+// items of 3 / 4 / 6 / 8 / 12 / 18 tiles; with d = 64 (half the bytes a tile) 16
+// layers of 16 units and 47 tiles 149 / 135 / 120 / 117 / 115 / 122 us.
+constexpr int kTilesPerItem = 9;
+constexpr int kTilesPerItem64 = 12;
 // kO: what a step costs on top of its item's tiles, in tiles: the item's
 // partial output, its row-slice sum, the hand-overs and the queries. Fitted to
 // 8 layers of 8 units and 256 tiles (items of 256 / 128 / 64 / 43 / 37 / 32 /
@@ -1014,13 +1020,17 @@ int sm_count() {
   return sms > 0 ? sms : 1;
 }
 
-// Votes only: key tiles per item of a unit of n_tiles: at least `least`, and no
-// more items than SMs (the deadlock-free schedule needs at most twice as many
-// as CTAs). A function of the prompt length alone, so that one layer's call
-// and a multi-layer call merge the same partial statistics.
-int tiles_per_item(int n_tiles, int least, int sms) {
-  const int tpi_min = (n_tiles + sms - 1) / sms;
-  return tpi_min > least ? tpi_min : least;
+// Votes only: key tiles per item of a unit of n_tiles: the unit is cut into the
+// fewest items of at most `most` tiles, all of the same size but the last (64
+// tiles as 8 items of 8 instead of 7 of 9 and one of 1: 32 layers of 8 units
+// 214 -> 201 us), and into no more items than SMs (the deadlock-free schedule
+// needs at most twice as many as CTAs). A function of the prompt length alone,
+// so that one layer's call and a multi-layer call merge the same partial
+// statistics.
+int tiles_per_item(int n_tiles, int most, int sms) {
+  const int tpi_min = (n_tiles + sms - 1) / sms, tpi = tpi_min > most ? tpi_min : most;
+  const int items = (n_tiles + tpi - 1) / tpi;
+  return (n_tiles + items - 1) / items;
 }
 
 struct Tc1Kernel {
@@ -1049,8 +1059,8 @@ Tc1Kernel tc1_kernel_for(int R) {
 
 int score_tc1_attn_items(const LayerGeom &g, int n_layers) {
   const int n_tiles = (g.T + kTile - 1) / kTile, sms = sm_count();
-  // a unit of up to kMinTilesPerItem tiles is one item, as without outputs
-  const int most = n_tiles / kMinTilesPerItem < sms ? n_tiles / kMinTilesPerItem : sms;
+  // a unit of up to kTilesPerItem tiles is one item, as without outputs
+  const int most = n_tiles / kTilesPerItem < sms ? n_tiles / kTilesPerItem : sms;
   const long long units = (long long)g.units * n_layers;
   int best = 1;
   long long best_cost = -1;
@@ -1117,7 +1127,7 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, 
   p.n_tiles2 = with_o ? p.n_tiles1 : (g.P + kTile - 1) / kTile;
   p.tpi = with_o ? (p.n_tiles1 + score_tc1_attn_items(g, n_layers) - 1) /
                        score_tc1_attn_items(g, n_layers)
-                 : tiles_per_item(p.n_tiles1, kMinTilesPerItem, sms);
+                 : tiles_per_item(p.n_tiles1, g.D == 64 ? kTilesPerItem64 : kTilesPerItem, sms);
   p.n_ch = (p.n_tiles1 + p.tpi - 1) / p.tpi;
   p.total_items = p.units * p.n_ch;
   p.scale2 = g.scale2;
