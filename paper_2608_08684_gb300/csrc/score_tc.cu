@@ -316,8 +316,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (qcount > 0) mbar_wait(&ms->q_full, (qcount - 1) & 1, nullptr);
     }
   } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // ------------------------------------------------ MMA issuer (the whole warp
+    // runs the loop and waits; one elected lane issues)
+    {
       int kcount = 0, acount = 0, qcount = 0;
       constexpr uint32_t id = idesc_bf16(128, 128);
       const uint32_t kbase = smem_u32(ktiles), qbase = smem_u32(qbufs);
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int pass = 1; pass <= 2 && ok; ++pass) {
           if ((pass == 1 && k >= n) || (pass == 2 && k < 1)) continue;
           const ItemRef it = item_of(p, pass == 1 ? k : k - 1);
-          if (!wait_bar(&ms->q_full, qcount & 1, ms, p.status)) {
+          if (!warp_wait(&ms->q_full, qcount & 1, ms, p.status)) {
             ok = false;
             break;
           }
@@ -336,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           tiles_of(p, it, pass, t0, t1);
           for (int t = t0; t < t1; ++t) {
             const int ks = kcount % C::NK;
-            if (!wait_bar(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status)) {
+            if (!warp_wait(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status)) {
               ok = false;
               break;
             }
@@ -344,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int nr = 0; nr < NR; ++nr) {
               const int as = acount % C::NA;
-              if (!wait_bar(&ms->acc_empty[as], ((acount / C::NA) & 1) ^ 1, ms, p.status)) {
+              if (!warp_wait(&ms->acc_empty[as], ((acount / C::NA) & 1) ^ 1, ms, p.status)) {
                 ok = false;
                 break;
               }
@@ -353,6 +354,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               // the first K step's descriptors; the others differ only in their
               // start-address field (16-byte units, no carry)
               const uint64_t qd = sw128_desc(qa + nr * kHalfBytes);
+              if (elect_one()) {
 #pragma unroll
               for (int kk = 0; kk < C::KSteps; ++kk) {
                 const uint64_t ko = kd + (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
@@ -361,17 +363,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                 mma_bf16(d, pass == 1 ? qo : ko, pass == 1 ? ko : qo, id, kk > 0);
               }
               mma_commit(&ms->acc_full[as]);
+              if (nr == NR - 1) mma_commit(&ms->k_empty[ks]);
+              }
+              __syncwarp();
               ++acount;
             }
             if (!ok) break;
-            mma_commit(&ms->k_empty[ks]);
             ++kcount;
           }
-          if (ok) mma_commit(&ms->q_empty);  // the pass is done with its queries
+          if (ok && elect_one()) mma_commit(&ms->q_empty);  // the pass is done with its queries
+          __syncwarp();
         }
       }
       // All issued MMAs complete before TMEM is released.
-      mma_commit(&ms->mma_done);
+      if (elect_one()) mma_commit(&ms->mma_done);
+      __syncwarp();
       mbar_wait(&ms->mma_done, 0, nullptr);
     }
   } else if (warp == 10) {

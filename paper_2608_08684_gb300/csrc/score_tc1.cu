@@ -61,7 +61,7 @@ namespace {
 
 constexpr int kTile = 128;                      // keys per tile
 constexpr int kHalfBytes = kTile * 64 * 2;      // one TMA box: 64 dims of 128 keys
-constexpr int kThreads = 352;
+constexpr int kThreads = 384;
 constexpr int kLag = 1;                         // pass 2 of item k runs in step k + kLag
 constexpr int kPubSlots = 2;
 // Key tiles of an item, at most. Two items a CTA stay in L2 between the passes,
@@ -112,6 +112,9 @@ struct Tc1Params {
   int n_tiles1, n_tiles2;  // key tiles of pass 1 (all keys) and pass 2 (prefix keys; all with kO)
   int tpi, n_ch;           // key tiles per item, items per unit
   int total_items;
+  // a CTA's next item, gridDim items further on: units, items of a unit, layers
+  // and units of a layer
+  int d_unit, d_chunk, d_layer, d_local;
   float scale2;
   float *o_win[kCompressMaxLayers];  // kO, per layer: window-row outputs [B][Hq][W][128] fp32
   float *o_part;     // kO: [units][n_ch][128][128] fp32 per-item partial outputs
@@ -140,12 +143,6 @@ __device__ __forceinline__ int items_of_cta(const Tc1Params &p) {
   return b < p.total_items ? (p.total_items - 1 - b) / (int)gridDim.x + 1 : 0;
 }
 
-__device__ __forceinline__ void tiles_of(const Tc1Params &p, const ItemRef &it, int pass, int &t0,
-                                         int &t1) {
-  t0 = it.chunk * p.tpi;
-  t1 = min(pass == 1 ? p.n_tiles1 : p.n_tiles2, t0 + p.tpi);
-}
-
 // Step k of a CTA's schedule: pass 1 of its item k (if k < n), then pass 2
 // of its item k - kLag (if k >= kLag). With a lag of one item, an item's keys
 // are re-read one item later, so about two items of keys per CTA (78 MB over
@@ -156,40 +153,64 @@ __device__ __forceinline__ void tiles_of(const Tc1Params &p, const ItemRef &it, 
 // with a lag of two and each step's pass-1 and pass-2 tiles alternating,
 // 2.90 / 2.95 / 3.13 / 3.84 ms with items of 9 / 7 / 6 / 5 tiles.
 
-struct Step {
-  int u1, a0, n1;  // pass 1: unit, first tile, tiles
-  int u2, b0, n2;  // pass 2
-  int len;         // max(n1, n2)
+// One item of the CTA's sequence with its layer and its unit's number in the
+// layer. Every role steps it along by additions: four divisions a step took
+// 900 cycles in each of them.
+struct ItemAt {
+  int unit, chunk, layer, local;
 };
 
-__device__ __forceinline__ Step step_of(const Tc1Params &p, int k, int n) {
-  Step s{0, 0, 0, 0, 0, 0, 0};
-  int e;
-  if (k < n) {
-    const ItemRef it = item_of(p, k);
-    tiles_of(p, it, 1, s.a0, e);
-    s.u1 = it.unit;
-    s.n1 = max(0, e - s.a0);
+__device__ __forceinline__ ItemAt first_item(const Tc1Params &p) {
+  const ItemRef it = item_of(p, 0);
+  return {it.unit, it.chunk, it.unit / p.upl, it.unit % p.upl};
+}
+
+__device__ __forceinline__ void advance(const Tc1Params &p, ItemAt &it) {
+  it.unit += p.d_unit;
+  it.layer += p.d_layer;
+  it.local += p.d_local;
+  it.chunk += p.d_chunk;
+  if (it.chunk >= p.n_ch) {
+    it.chunk -= p.n_ch;
+    ++it.unit;
+    ++it.local;
   }
-  if (k >= kLag) {
-    const ItemRef it = item_of(p, k - kLag);
-    tiles_of(p, it, 2, s.b0, e);
-    s.u2 = it.unit;
-    s.n2 = max(0, e - s.b0);
+  if (it.local >= p.upl) {  // d_local < upl: once, or once more by the carry
+    it.local -= p.upl;
+    ++it.layer;
+    if (it.local >= p.upl) {
+      it.local -= p.upl;
+      ++it.layer;
+    }
   }
-  s.len = s.n1 + s.n2;
+}
+
+// Step k: pass 1 of item i1 (tiles a0 .. a0 + n1 - 1) and pass 2 of item i2,
+// the one before.
+struct Step {
+  ItemAt i1, i2;
+  int a0, n1;
+  int b0, n2;
+};
+
+// The steps of a CTA in order: start() gives step 0, next() the one after.
+__device__ __forceinline__ Step start(const Tc1Params &p, int n) {
+  Step s;
+  s.i1 = first_item(p);
+  s.i2 = s.i1;
+  s.a0 = s.i1.chunk * p.tpi;
+  s.n1 = n > 0 ? min(p.tpi, p.n_tiles1 - s.a0) : 0;
+  s.b0 = s.n2 = 0;
   return s;
 }
 
-// The epilogue warpgroup that takes the CTA's tile number `tc`: alternate
-// tiles, so that each warpgroup meets every phase of its accumulator slot.
-__device__ __forceinline__ int wg_of(int tc) { return tc & 1; }
-
-// Position j of step s's tile sequence: its pass-1 tiles, then its pass-2
-// tiles.
-__device__ __forceinline__ void seq_at(const Step &s, int j, int &pass, int &idx) {
-  pass = j < s.n1 ? 1 : 2;
-  idx = j < s.n1 ? j : j - s.n1;
+__device__ __forceinline__ void next(const Tc1Params &p, Step &s, int k, int n) {
+  s.i2 = s.i1;
+  s.b0 = s.a0;
+  s.n2 = max(0, min(p.tpi, p.n_tiles2 - s.b0));
+  advance(p, s.i1);
+  s.a0 = s.i1.chunk * p.tpi;
+  s.n1 = k + 1 < n ? min(p.tpi, p.n_tiles1 - s.a0) : 0;
 }
 
 struct Misc {
@@ -205,7 +226,8 @@ struct Misc {
   int abort_flag;
   long long wait_cycles;  // bound of the waits of this launch
   float2 pstat[kPubSlots][2][128];      // pass-1 row statistics per slot and warpgroup
-  alignas(16) float offs[2][128];       // per warpgroup: the pass-2 item's row log-normalisers
+  alignas(16) float offs[2][128];       // pass-2 items' row log-normalisers, per step parity
+  uint64_t offs_full[2], offs_empty[2];
 };
 
 // Shared memory: the ring, the pass-2 and pass-1 queries (two 64-dim halves
@@ -281,34 +303,28 @@ struct Tc1Launch {
   Tc1Params p;
 };
 
-// With kO the producer and the MMA warp walk a step as: the pass-1 key tiles,
-// then the pass-2 item's key tiles with value tile s - kPvLag after key tile
-// s (the order the MMA warp consumes them in: it multiplies a tile's
-// probabilities by its values after issuing the logits kPvLag tiles on, so
-// that the warpgroup that has just written a tile's probabilities finds its
-// next tile's logits done), then the last value tiles.
-// kind 1: pass-1 key tile, 2: pass-2 key tile, 3: pass-2 value tile.
+// With kO the producer and the MMA warp walk a step's pass 2 as: the item's key
+// tiles with value tile s - kPvLag after key tile s (the order the MMA warp
+// consumes them in: it multiplies a tile's probabilities by its values after
+// issuing the logits kPvLag tiles on, so that the warpgroup that has just
+// written a tile's probabilities finds its next tile's logits done), then the
+// last value tiles. Position q of the 2 * n2: whether it is a value tile, and
+// which tile s.
 constexpr int kPvLag = 2;
-__device__ __forceinline__ void oseq_at(const Step &s, int j, int &kind, int &idx) {
-  if (j < s.n1) {
-    kind = 1;
-    idx = j;
-    return;
-  }
-  const int q = j - s.n1;
-  const int a = min(s.n2, kPvLag);           // leading key tiles
-  const int pairs = max(0, s.n2 - kPvLag);   // (key s, value s - kPvLag)
+__device__ __forceinline__ bool ovalue_at(int n2, int q, int &s) {
+  const int a = min(n2, kPvLag);           // leading key tiles
+  const int pairs = max(0, n2 - kPvLag);   // (key s, value s - kPvLag)
   if (q < a) {
-    kind = 2;
-    idx = q;
-  } else if (q - a < 2 * pairs) {
-    const int t = (q - a) >> 1;
-    kind = (q - a) & 1 ? 3 : 2;
-    idx = (q - a) & 1 ? t : kPvLag + t;
-  } else {
-    kind = 3;
-    idx = pairs + (q - a - 2 * pairs);
+    s = q;
+    return false;
   }
+  if (q - a < 2 * pairs) {
+    const int t = (q - a) >> 1;
+    s = (q - a) & 1 ? t : kPvLag + t;
+    return (q - a) & 1;
+  }
+  s = pairs + (q - a - 2 * pairs);
+  return true;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
@@ -461,6 +477,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&ms->pub_full[i], 8);
       mbar_init(&ms->pub_empty[i], 1);
     }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&ms->offs_full[i], 1);
+      mbar_init(&ms->offs_empty[i], 8);
+    }
     mbar_init(&ms->mma_done, 1);
     mbar_init(&ms->p_full, 8);
     mbar_init(&ms->p_empty, 1);
@@ -489,78 +509,65 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     // ------------------------------------------------ key-tile producer
     if (lane == 0) {
-      int kcount = 0, qcount = 0;
+      int kcount = 0, qcount = 0, q1count = 0;
       const uint64_t keep = policy_evict_last(), drop = policy_evict_first();
       bool ok = true;
-      for (int k = 0; k < n + kLag && ok; ++k) {
-        const Step st = step_of(p, k, n);
-        const int l1 = st.u1 / p.upl, loc1 = st.u1 - l1 * p.upl;
-        const int l2 = st.u2 / p.upl, loc2 = st.u2 - l2 * p.upl;
-        const int len = kO ? st.n1 + 2 * st.n2 : st.len;
-        for (int j = 0; j < len && ok; ++j) {
-          int pass, s, kind;
-          if (kO) {
-            oseq_at(st, j, kind, s);
-            pass = kind == 1 ? 1 : 2;
-          } else {
-            seq_at(st, j, pass, s);
-            kind = pass;
-          }
-          if (kind == 1 && s == 0) {
-            // item k's queries into the pass-1 buffer, once the previous
-            // item's pass-1 MMAs have read it
-            if (!wait_bar(&ms->q_empty, (k & 1) ^ 1, ms, p.status)) {
-              ok = false;
-              break;
-            }
-            mbar_arrive_expect_tx(&ms->q_full, (uint32_t)(C::Copies * R * D * 2));
+      // one tile of keys (or values) into the ring
+      auto load_tile = [&](const CUtensorMap *map, int tile, int local, uint64_t pol) {
+        const int ks = kcount % C::NK;
+        if (!wait_bar(&ms->k_empty[ks], ((kcount / C::NK) & 1) ^ 1, ms, p.status)) return false;
+        mbar_arrive_expect_tx(&ms->k_full[ks], kTileBytes);
+        uint8_t *kb = ktiles + ks * kTileBytes;
 #pragma unroll
-            for (int i = 0; i < C::Copies * (D / 64); ++i) {
-              const int half = i % (D / 64), copy = i / (D / 64);
-              tma_load_2d(q1m + half * kHalfBytes + copy * RP * 128, &lp.qmap[l1], half * 64,
-                          loc1 * R, &ms->q_full);
-            }
-          }
-          if (kind == 2 && s == 0) {
-            // the pass-2 item's queries (rows of its unit) into shared memory
-            if (!wait_bar(&ms->qs_empty, (qcount & 1) ^ 1, ms, p.status)) {
-              ok = false;
-              break;
-            }
-            mbar_arrive_expect_tx(&ms->qs_full, (uint32_t)(R * D * 2));
+        for (int half = 0; half < D / 64; ++half)
+          tma_load_3d(kb + half * kHalfBytes, map, half * 64, tile * kTile, local,
+                      &ms->k_full[ks], pol);
+        ++kcount;
+        return true;
+      };
+      Step st = start(p, n);
+      for (int k = 0; k < n + kLag && ok; next(p, st, k, n), ++k) {
+        if (st.n1 > 0) {
+          // item k's queries into the pass-1 buffer, once the previous item's
+          // pass-1 MMAs have read it
+          if (!wait_bar(&ms->q_empty, (k & 1) ^ 1, ms, p.status)) break;
+          mbar_arrive_expect_tx(&ms->q_full, (uint32_t)(C::Copies * R * D * 2));
 #pragma unroll
-            for (int half = 0; half < D / 64; ++half)
-              tma_load_2d(qsm + half * kHalfBytes, &lp.qmap[l2], half * 64, loc2 * R,
-                          &ms->qs_full);
-            ++qcount;
+          for (int i = 0; i < C::Copies * (D / 64); ++i) {
+            const int half = i % (D / 64), copy = i / (D / 64);
+            tma_load_2d(q1m + half * kHalfBytes + copy * RP * 128, &lp.qmap[st.i1.layer],
+                        half * 64, st.i1.local * R, &ms->q_full);
           }
-          const int tt = pass == 1 ? st.a0 + s : st.b0 + s;
-          const int ks = kcount % C::NK;
-          if (!wait_bar(&ms->k_empty[ks], ((kcount / C::NK) & 1) ^ 1, ms, p.status)) {
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(&ms->k_full[ks], kTileBytes);
-          uint8_t *kb = ktiles + ks * kTileBytes;
-          const uint64_t pol = pass == 1 ? keep : drop;
-          // the step's two units' layers and local indices (divisions hoisted
-          // out of the tile loop)
-          const int layer = pass == 1 ? l1 : l2, local = pass == 1 ? loc1 : loc2;
-          const CUtensorMap *km = kind == 3 ? &lp.vmap[layer] : &lp.kmap[layer];
+          ++q1count;
+          for (int s = 0; s < st.n1 && ok; ++s)
+            ok = load_tile(&lp.kmap[st.i1.layer], st.a0 + s, st.i1.local, keep);
+        }
+        if (ok && st.n2 > 0) {
+          // the pass-2 item's queries (rows of its unit) into shared memory
+          if (!wait_bar(&ms->qs_empty, (qcount & 1) ^ 1, ms, p.status)) break;
+          mbar_arrive_expect_tx(&ms->qs_full, (uint32_t)(R * D * 2));
 #pragma unroll
           for (int half = 0; half < D / 64; ++half)
-            tma_load_3d(kb + half * kHalfBytes, km, half * 64, tt * kTile, local,
-                        &ms->k_full[ks], pol);
-          ++kcount;
+            tma_load_2d(qsm + half * kHalfBytes, &lp.qmap[st.i2.layer], half * 64,
+                        st.i2.local * R, &ms->qs_full);
+          ++qcount;
+          for (int j = 0; j < (kO ? 2 : 1) * st.n2 && ok; ++j) {
+            int s = j;
+            const bool value = kO && ovalue_at(st.n2, j, s);
+            const CUtensorMap *map = value ? &lp.vmap[st.i2.layer] : &lp.kmap[st.i2.layer];
+            ok = load_tile(map, st.b0 + s, st.i2.local, drop);
+          }
         }
       }
       for (int j = max(0, kcount - C::NK); j < kcount; ++j)
         mbar_wait(&ms->k_full[j % C::NK], (j / C::NK) & 1, nullptr);
       if (qcount > 0) mbar_wait(&ms->qs_full, (qcount - 1) & 1, nullptr);
+      if (q1count > 0) mbar_wait(&ms->q_full, (q1count - 1) & 1, nullptr);
     }
   } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // ------------------------------------------------ MMA issuer (the whole warp
+    // runs the loop and waits; one elected lane issues)
+    {
       int kcount = 0, acount = 0, qcount = 0, ocount = 0;
       int pv_count = 0;  // kO: probability tiles multiplied
       constexpr uint32_t id1 = idesc_bf16(128, 128);   // rows (all copies) x keys
@@ -571,98 +578,90 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t pbase = smem_u32(ptile);
       const uint64_t q1d = sw128_desc(q1base), qsd = sw128_desc(qsbase);
       bool ok = true;
-      for (int k = 0; k < n + kLag && ok; ++k) {
-        const Step st = step_of(p, k, n);
-        if (k < n && !wait_bar(&ms->q_full, k & 1, ms, p.status)) break;
-        const int len = kO ? st.n1 + 2 * st.n2 : st.len;
-        for (int j = 0; j < len && ok; ++j) {
-          int pass, s, kind;
-          if (kO) {
-            oseq_at(st, j, kind, s);
-            pass = kind == 1 ? 1 : 2;
-          } else {
-            seq_at(st, j, pass, s);
-            kind = pass;
+      // logits of one key tile: D = A . B^T, A and B the first K step's
+      // descriptors (the others differ only in their start-address field, in
+      // 16-byte units, without carry)
+      auto logits = [&](bool pass1, bool last) {
+        const int ks = kcount % C::NK, as = acount % C::NA;
+        if (!warp_wait(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status) ||
+            !warp_wait(&ms->acc_empty[as], ((acount / C::NA) & 1) ^ 1, ms, p.status))
+          return false;
+        tc_fence_after();
+        const uint32_t d = tmem + as * 128;
+        const uint64_t kd = sw128_desc(kbase + ks * kTileBytes);
+        const uint64_t ad = pass1 ? q1d : kd, bd = pass1 ? kd : qsd;
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < C::KSteps; ++kk) {
+            const uint64_t off = (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
+            mma_bf16(d, ad + off, bd + off, pass1 ? id1 : id2, kk > 0);
           }
-          const int ks = kcount % C::NK;
-          const uint32_t ka = kbase + ks * kTileBytes;
-          if (kO && kind == 3) {
+          mma_commit(&ms->k_empty[ks]);
+          mma_commit(&ms->acc_full[as]);
+          if (last) mma_commit(pass1 ? &ms->q_empty : &ms->qs_empty);  // its queries are free
+        }
+        __syncwarp();
+        ++kcount;
+        ++acount;
+        return true;
+      };
+      Step st = start(p, n);
+      for (int k = 0; k < n + kLag && ok; next(p, st, k, n), ++k) {
+        if (st.n1 > 0 && !warp_wait(&ms->q_full, k & 1, ms, p.status)) break;
+        for (int s = 0; s < st.n1 && ok; ++s) ok = logits(true, s == st.n1 - 1);
+        if (!ok || st.n2 == 0) continue;
+        if (!warp_wait(&ms->qs_full, qcount & 1, ms, p.status)) break;
+        if constexpr (!kO) {
+          for (int s = 0; s < st.n2 && ok; ++s) ok = logits(false, s == st.n2 - 1);
+        } else {
+          for (int j = 0; j < 2 * st.n2 && ok; ++j) {
+            int s;
+            if (!ovalue_at(st.n2, j, s)) {
+              ok = logits(false, s == st.n2 - 1);
+              continue;
+            }
             // O (+)= P . V for pass-2 tile s, once the epilogue has written
             // its probabilities (and, for the item's first tile, has read
             // out the previous item's O)
-            if ((s == 0 && !wait_bar(&ms->o_empty, (ocount & 1) ^ 1, ms, p.status)) ||
-                !wait_bar(&ms->p_full, pv_count & 1, ms, p.status) ||
-                !wait_bar(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status)) {
+            const int ks = kcount % C::NK;
+            if ((s == 0 && !warp_wait(&ms->o_empty, (ocount & 1) ^ 1, ms, p.status)) ||
+                !warp_wait(&ms->p_full, pv_count & 1, ms, p.status) ||
+                !warp_wait(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            // K step kk: 16 keys further along both MN-major operands
-            const uint64_t pd = sw128_desc_mn(pbase, kHalfBytes, 1024);
-            const uint64_t vd = sw128_desc_mn(ka, kHalfBytes, 1024);
+            if (elect_one()) {
+              // K step kk: 16 keys further along both MN-major operands
+              const uint64_t pd = sw128_desc_mn(pbase, kHalfBytes, 1024);
+              const uint64_t vd = sw128_desc_mn(kbase + ks * kTileBytes, kHalfBytes, 1024);
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const uint64_t step = (uint64_t)(kk * 2048 >> 4);
-              mma_bf16(tmem + C::OCol, pd + step, vd + step, id_pv, kk > 0 || s > 0);
+              for (int kk = 0; kk < 8; ++kk) {
+                const uint64_t step = (uint64_t)(kk * 2048 >> 4);
+                mma_bf16(tmem + C::OCol, pd + step, vd + step, id_pv, kk > 0 || s > 0);
+              }
+              mma_commit(&ms->k_empty[ks]);
+              mma_commit(&ms->p_empty);
+              if (s == st.n2 - 1) mma_commit(&ms->o_full);
             }
-            mma_commit(&ms->k_empty[ks]);
-            mma_commit(&ms->p_empty);
+            __syncwarp();
             ++kcount;
             ++pv_count;
-            if (s == st.n2 - 1) {
-              mma_commit(&ms->o_full);
-              ++ocount;
-            }
-            continue;
+            if (s == st.n2 - 1) ++ocount;
           }
-          if (pass == 2 && s == 0) {
-            if (st.n1 > 0) mma_commit(&ms->q_empty);  // item k's pass-1 queries are free
-            if (!wait_bar(&ms->qs_full, qcount & 1, ms, p.status)) {
-              ok = false;
-              break;
-            }
-          }
-          const int as = acount % C::NA;
-          if (!wait_bar(&ms->k_full[ks], (kcount / C::NK) & 1, ms, p.status) ||
-              !wait_bar(&ms->acc_empty[as], ((acount / C::NA) & 1) ^ 1, ms, p.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t d = tmem + as * 128;
-          {
-            // descriptors of the tile's first K step; the others differ only
-            // in their start-address field (16-byte units, no carry)
-            const uint64_t kd = sw128_desc(ka);
-            const uint64_t qd = pass == 1 ? q1d : qsd;
-            const uint64_t ad = pass == 1 ? qd : kd, bd = pass == 1 ? kd : qd;
-#pragma unroll
-            for (int kk = 0; kk < C::KSteps; ++kk) {
-              const uint64_t off = (uint64_t)(((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4);
-              mma_bf16(d, ad + off, bd + off, pass == 1 ? id1 : id2, kk > 0);
-            }
-          }
-          mma_commit(&ms->k_empty[ks]);
-          mma_commit(&ms->acc_full[as]);
-          ++kcount;
-          ++acount;
         }
-        if (ok && st.n2 > 0) {
-          mma_commit(&ms->qs_empty);  // the pass-2 queries are free
-          ++qcount;
-        } else if (ok && st.n1 > 0) {
-          mma_commit(&ms->q_empty);  // no pass-2 tiles: item k's pass-1 queries are free
-        }
+        ++qcount;
       }
-      mma_commit(&ms->mma_done);
+      if (elect_one()) mma_commit(&ms->mma_done);
+      __syncwarp();
       mbar_wait(&ms->mma_done, 0, nullptr);
     }
   } else if (warp == 10) {
     // ------------------------------------------------ publisher of pass-1 results
-    for (int k = 0; k < n; ++k) {
+    ItemAt it = first_item(p);
+    for (int k = 0; k < n; advance(p, it), ++k) {
       const int slot = k % kPubSlots;
       if (!warp_wait(&ms->pub_full[slot], (k / kPubSlots) & 1, ms, p.status)) break;
-      const ItemRef it = item_of(p, k);
       float2 *mine = p.partial + guard((long long)it.unit * p.n_ch + it.chunk, 1,
                                        (long long)p.units * p.n_ch, p.status) *
                                      R;
@@ -727,6 +726,31 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) st_release(&p.ctrl[guard(p.units + it.unit, 1, 2LL * p.units, p.status)], 1);
       }
     }
+  } else if (warp == 11) {
+    // ------------------------------------------------ normalisers of pass-2 items:
+    // waits for the unit's row statistics and brings them in, so that the
+    // epilogue meets neither the flag's latency nor the loads' (3000 cycles
+    // an item)
+    Step st = start(p, n);
+    int count = 0;
+    for (int k = 0; k < n + kLag; next(p, st, k, n), ++k) {
+      if (st.n2 == 0) continue;
+      const int b = count & 1;
+      if (!warp_wait(&ms->offs_empty[b], ((count >> 1) & 1) ^ 1, ms, p.status)) break;
+      int ok = 1;
+      if (lane == 0)
+        ok = wait_ready(&p.ctrl[guard(p.units + st.i2.unit, 1, 2LL * p.units, p.status)], ms,
+                        p.status);
+      if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+      __syncwarp();  // lane 0's acquire orders every lane's loads
+      const float *ln = p.lognorm + guard(st.i2.unit, 1, p.units, p.status) * R;
+#pragma unroll
+      for (int r = 0; r < RP / 32; ++r)
+        if (!kPad || lane + 32 * r < R) ms->offs[b][lane + 32 * r] = __ldcg(ln + lane + 32 * r);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ms->offs_full[b]);
+      ++count;
+    }
   } else {
     // ------------------------------------------------ epilogue warpgroups
     const int wg = (warp - 2) >> 2;
@@ -740,102 +764,92 @@ __global__ void __launch_bounds__(kThreads, 1)
     int tcount = 0;  // tiles seen
     int oc = 0;            // kO: pass-2 items seen
     int ptc = 0;           // kO: probability tiles written
+    int ocount = 0;        // pass-2 items seen
 
     // Inside an item every warp follows the same control flow even if a wait
     // gives up (the tile is then skipped), so that the named barriers below
     // are always reached by all of their threads.
-    for (int k = 0; k < n + kLag; ++k) {
-      const Step st = step_of(p, k, n);
+    Step st = start(p, n);
+    for (int k = 0; k < n + kLag; next(p, st, k, n), ++k) {
       float m = -INFINITY, l = 0.f;    // pass 1 of item k: this row's max and sum
       const int last_vis = p.P + row % p.W;
-      // votes of the pass-2 unit: its layer's slot of the vote array
-      const long long vote0 =
-          (long long)(p.layer_of[st.u2 / p.upl] * p.upl + st.u2 % p.upl) * p.P;
-      for (int j = 0; j < st.len; ++j) {
-        int pass, s;
-        seq_at(st, j, pass, s);
-        if (pass == 1) {
-          // ---------------- a pass-1 tile of item k
+      // ---------------- this warpgroup's pass-1 tiles of item k: every other one
+      // of the CTA's tiles, so that it meets every phase of its accumulators
+      for (int s = (tcount ^ wg) & 1; s < st.n1; s += 2) {
+        const int as = (tcount + s) % C::NA, ph = ((tcount + s) / C::NA) & 1;
+        if (warp_wait(&ms->acc_full[as], ph, ms, p.status)) {
+          tc_fence_after();
           const int t = st.a0 + s;
-          const int mine = wg_of(tcount) == wg;
-          const int as = tcount % C::NA, ph = (tcount / C::NA) & 1;
-          ++tcount;
-          if (mine && warp_wait(&ms->acc_full[as], ph, ms, p.status)) {
-            tc_fence_after();
-            uint32_t x[RP / 32][32];
+          uint32_t x[RP / 32][32];
 #pragma unroll
-            for (int c = 0; c < RP / 32; ++c)
-              tmem_ld32(tmem + lane_addr + as * 128 + (C::Copies > 1 ? col0 : 0) + c * 32, x[c]);
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cnt(&ms->acc_empty[as], kO ? 2 : 1);
-            const int key0 = t * kTile + (C::Copies > 1 ? col0 : 0);  // this thread's first key
-            if ((t + 1) * kTile - 1 >= p.P) {  // keys this row cannot see -> -inf
-#pragma unroll
-              for (int c = 0; c < RP / 32; ++c)
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                  if (key0 + c * 32 + j > last_vis) x[c][j] = 0xff800000u;
-            }
-            float mx[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) mx[i] = -INFINITY;
+          for (int c = 0; c < RP / 32; ++c)
+            tmem_ld32(tmem + lane_addr + as * 128 + (C::Copies > 1 ? col0 : 0) + c * 32, x[c]);
+          tmem_wait_ld();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cnt(&ms->acc_empty[as], kO ? 2 : 1);
+          const int key0 = t * kTile + (C::Copies > 1 ? col0 : 0);  // this thread's first key
+          if ((t + 1) * kTile - 1 >= p.P) {  // keys this row cannot see -> -inf
 #pragma unroll
             for (int c = 0; c < RP / 32; ++c)
 #pragma unroll
-              for (int j = 0; j < 32; ++j) mx[j & 7] = fmaxf(mx[j & 7], __uint_as_float(x[c][j]));
-            const float tmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
-                                     fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
-            if (live1 && tmax != -INFINITY) {
-              const float mnew = fmaxf(m, tmax * p.scale2);
-              // fp32x2: logits scaled and shifted two at a time, sums in pairs
-              float2 sv[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) sv[i] = make_float2(0.f, 0.f);
-              const float2 s2 = make_float2(p.scale2, p.scale2), mn2 = make_float2(-mnew, -mnew);
-#pragma unroll
-              for (int c = 0; c < RP / 32; ++c)
-#pragma unroll
-                for (int j = 0; j < 32; j += 2) {
-                  const float2 y = __ffma2_rn(
-                      make_float2(__uint_as_float(x[c][j]), __uint_as_float(x[c][j + 1])), s2, mn2);
-                  sv[(j >> 1) & 3] =
-                      __fadd2_rn(sv[(j >> 1) & 3], make_float2(fast_exp2(y.x), fast_exp2(y.y)));
-                }
-              const float sum = ((sv[0].x + sv[0].y) + (sv[1].x + sv[1].y)) +
-                                ((sv[2].x + sv[2].y) + (sv[3].x + sv[3].y));
-              l = l * fast_exp2(m - mnew) + sum;
-              m = mnew;
-            }
+              for (int j = 0; j < 32; ++j)
+                if (key0 + c * 32 + j > last_vis) x[c][j] = 0xff800000u;
           }
-          if (s == st.n1 - 1) {
-            // Item k's last pass-1 tile: this warpgroup's row statistics go to
-            // the publisher now, ahead of the step's pass-2 tiles.
-            const int slot = k % kPubSlots;
-            warp_wait(&ms->pub_empty[slot], ((k / kPubSlots) & 1) ^ 1, ms, p.status);
-            ms->pstat[slot][wg][r] = make_float2(m, l);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&ms->pub_full[slot]);
+          float mx[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mx[i] = -INFINITY;
+#pragma unroll
+          for (int c = 0; c < RP / 32; ++c)
+#pragma unroll
+            for (int j = 0; j < 32; ++j) mx[j & 7] = fmaxf(mx[j & 7], __uint_as_float(x[c][j]));
+          const float tmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
+                                   fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
+          if (live1 && tmax != -INFINITY) {
+            const float mnew = fmaxf(m, tmax * p.scale2);
+            // fp32x2: logits scaled and shifted two at a time, sums in pairs
+            float2 sv[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sv[i] = make_float2(0.f, 0.f);
+            const float2 s2 = make_float2(p.scale2, p.scale2), mn2 = make_float2(-mnew, -mnew);
+#pragma unroll
+            for (int c = 0; c < RP / 32; ++c)
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) {
+                const float2 y = __ffma2_rn(
+                    make_float2(__uint_as_float(x[c][j]), __uint_as_float(x[c][j + 1])), s2, mn2);
+                sv[(j >> 1) & 3] =
+                    __fadd2_rn(sv[(j >> 1) & 3], make_float2(fast_exp2(y.x), fast_exp2(y.y)));
+              }
+            const float sum = ((sv[0].x + sv[0].y) + (sv[1].x + sv[1].y)) +
+                              ((sv[2].x + sv[2].y) + (sv[3].x + sv[3].y));
+            l = l * fast_exp2(m - mnew) + sum;
+            m = mnew;
           }
         }
-        if (pass == 2) {
-          // ---------------- a pass-2 tile of item k - kLag: votes of its keys
-          // (D[key][row]: this thread's TMEM lane is key t * 128 + r)
-          if (s == 0) {
-            if (wtid == 0)
-              wait_ready(&p.ctrl[guard(p.units + st.u2, 1, 2LL * p.units, p.status)], ms,
-                         p.status);
-            named_bar_sync(3 + wg, 128);
-            if (wtid < R)
-              ms->offs[wg][wtid] =
-                  __ldcg(&p.lognorm[guard(st.u2, 1, p.units, p.status) * R + wtid]);
-            named_bar_sync(3 + wg, 128);
-          }
-          const int t = st.b0 + s;
-          const int as = tcount % C::NA, ph = (tcount / C::NA) & 1;
-          if constexpr (kO) {
-            const int key = t * kTile + r;
+      }
+      tcount += st.n1;
+      if (st.n1 > 0) {
+        // This warpgroup's row statistics go to the publisher now, ahead of
+        // the step's pass-2 tiles.
+        const int slot = k % kPubSlots;
+        warp_wait(&ms->pub_empty[slot], ((k / kPubSlots) & 1) ^ 1, ms, p.status);
+        ms->pstat[slot][wg][r] = make_float2(m, l);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ms->pub_full[slot]);
+      }
+      // ---------------- pass 2 of item k - kLag: votes of its keys
+      // (D[key][row]: this thread's TMEM lane is key (b0 + s) * 128 + r)
+      if (st.n2 > 0) {
+        const int ob = ocount & 1;
+        warp_wait(&ms->offs_full[ob], (ocount >> 1) & 1, ms, p.status);
+        // votes of the unit: its layer's slot of the vote array
+        const long long vote0 =
+            (long long)(p.layer_of[st.i2.layer] * p.upl + st.i2.local) * p.P;
+        if constexpr (kO) {
+          for (int s = 0; s < st.n2; ++s) {
+            const int key = (st.b0 + s) * kTile + r;
+            const int as = (tcount + s) % C::NA, ph = ((tcount + s) / C::NA) & 1;
             // both warpgroups take every pass-2 tile, each for 64 of its 128
             // window rows (logit columns 64 wg ..): its half of the key's
             // probabilities, half of the vote (summed over the warpgroups
@@ -854,7 +868,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               // a window key (or a key past the end) is seen only by the rows
               // at or after it (causal inside the window)
               uint32_t pk[32];
-              half = half_probs<true>(x, reinterpret_cast<const float4 *>(ms->offs[wg]), 2 * wg,
+              half = half_probs<true>(x, reinterpret_cast<const float4 *>(ms->offs[ob]), 2 * wg,
                                       p.scale2, key >= p.P ? key - p.P : -1, p.W, pk);
               // into the tile once the previous tile's probabilities have
               // been multiplied
@@ -870,7 +884,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               p.votes[guard(vote0 + key, 1, (long long)p.n_slots * p.upl * p.P, p.status)] =
                   half + ms->vhalf[ptc & 1][r];
             ++ptc;
-          } else if (wg_of(tcount) == wg && warp_wait(&ms->acc_full[as], ph, ms, p.status)) {
+          }
+        } else {
+          for (int s = (tcount ^ wg) & 1; s < st.n2; s += 2) {
+            const int as = (tcount + s) % C::NA, ph = ((tcount + s) / C::NA) & 1;
+            if (!warp_wait(&ms->acc_full[as], ph, ms, p.status)) continue;
             tc_fence_after();
             uint32_t x[RP / 32][32];
 #pragma unroll
@@ -880,7 +898,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&ms->acc_empty[as]);
-            const float4 *o4 = reinterpret_cast<const float4 *>(ms->offs[wg]);
+            const float4 *o4 = reinterpret_cast<const float4 *>(ms->offs[ob]);
             // the two halves' sums as half_probs forms them, in one pass
             float2 sv[2][4];
 #pragma unroll
@@ -921,20 +939,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                              ((sv[0][2].x + sv[0][2].y) + (sv[0][3].x + sv[0][3].y));
             const float h1 = ((sv[1][0].x + sv[1][0].y) + (sv[1][1].x + sv[1][1].y)) +
                              ((sv[1][2].x + sv[1][2].y) + (sv[1][3].x + sv[1][3].y));
-            const int key = t * kTile + r;
+            const int key = (st.b0 + s) * kTile + r;
             if (key < p.P)
               p.votes[guard(vote0 + key, 1, (long long)p.n_slots * p.upl * p.P, p.status)] =
                   h0 + h1;
           }
-          ++tcount;
         }
+        tcount += st.n2;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ms->offs_empty[ob]);
+        ++ocount;
       }
       if (kO && st.n2 > 0) {
         // ---------------- kO: item k - kLag's partial O (both warpgroups:
         // this thread's row, warpgroup wg's 64 dims), and the unit's output
         // from its items' partials, summed in item order by the item that
         // completes the unit
-        const ItemRef it = item_of(p, k - kLag);
+        const ItemAt &it = st.i2;
         const size_t prow = ((size_t)it.unit * p.n_ch + it.chunk) * 128 + r;
         if (warp_wait(&ms->o_full, oc & 1, ms, p.status)) {
           tc_fence_after();
@@ -1154,6 +1175,10 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, 
   e = cudaFuncSetAttribute(kernel.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kernel.smem);
   if (e != cudaSuccess) return e;
   const int grid = p.total_items < sms ? p.total_items : sms;
+  p.d_unit = grid / p.n_ch;
+  p.d_chunk = grid % p.n_ch;
+  p.d_layer = p.d_unit / p.upl;
+  p.d_local = p.d_unit % p.upl;
   void *args[] = {(void *)&lp};
   e = cudaLaunchCooperativeKernel(kernel.fn, dim3(grid), dim3(kThreads), args,
                                   (size_t)kernel.smem, st);
