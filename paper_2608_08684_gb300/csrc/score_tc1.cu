@@ -3,11 +3,14 @@
 // the 5th-generation tensor cores. Row counts other than 32, 64 and 128 are
 // padded to the next of them with zero rows that no sum counts.
 //
-// Bound: HBM for 128 rows of d = 128 (a layer of 32 units and 32768 keys
-// about 72 us, 3.7 TB/s of its own bytes); the exponentials and the per-tile
-// hand-overs for small rows or d = 64: 16 layers of 16 units, 6007 keys, d =
-// 64 and 64 rows take 203 us with selection and gather, against 1917 us when
-// the fp32 pipes scored these shapes layer by layer.
+// Bound: board power for 128 rows of d = 128 in large calls (32 layers of 32
+// units, 32768 keys: 1370 W, the SM clock down to 1970 MHz, 70 us a layer), so
+// that schedules with the same reads, MMAs and exponentials take the same
+// time; else the epilogue's arithmetic (about 1350 cycles for 128 logits a
+// thread, two warps to an SM partition, the exponential unit 75% busy) and, for
+// few rows or d = 64, the MMA warp's issue of about 900 cycles a tile. Before
+// these kernels took every bf16 shape, 16 layers of 16 units, 6007 keys, d = 64
+// and 64 rows took 1917 us on the fp32 pipes; 105 us now, with selection.
 //
 // One persistent CTA per SM, item i on CTA i mod grid; in its step k a CTA
 // runs P1(a_k) then P2(a_k-1), so that keys are re-read from L2 one item
@@ -23,9 +26,11 @@
 // holds four 128-column accumulators, so the MMA issuer can run two tiles
 // ahead of each epilogue warpgroup.
 //
-// Warp roles (352 threads): warp 0 = key-tile and query producer, warp 1 =
-// MMA issuer and TMEM owner, warps 2-9 = two epilogue warpgroups taking
-// alternate tiles, warp 10 = publisher of pass-1 results. Every wait is
+// Warp roles (384 threads): warp 0 = key-tile and query producer, warp 1 =
+// MMA issuer and TMEM owner, warps 2-9 = two epilogue warpgroups, which take
+// alternate tiles (with 128 rows both take every pass-2 tile, half of its rows
+// each), warp 10 = publisher of pass-1 results, warp 11 brings in the row
+// normalisers of pass-2 items. Every wait is
 // bounded; on timeout the CTA raises RIPPLE_ETIMEOUT, every role leaves its
 // loop and TMEM is released.
 //
@@ -222,6 +227,10 @@ struct Misc {
   // P . V MMA releases it) and the O accumulator
   uint64_t p_full, p_empty, o_full, o_empty;
   float vhalf[2][128];  // kO: warpgroup 1's half of each key's vote, per tile parity
+  // votes only: the same in a ring with more entries than accumulators, so that
+  // warpgroup 1 (at most an accumulator ring ahead) overwrites none unread
+  float vring[kMaxStages][128];
+  uint64_t vr_full[kMaxStages];
   uint32_t tmem_base;
   int abort_flag;
   long long wait_cycles;  // bound of the waits of this launch
@@ -446,6 +455,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   using C = Tc1Cfg<kO, D, RP>;
   using SM = Tc1Smem<kO, D, RP>;
   constexpr int kTileBytes = C::TileBytes;
+  // 128 rows: both epilogue warpgroups take every pass-2 tile, each for 64 of
+  // its rows, whose normalisers a thread keeps in registers for the item. With a
+  // tile to a warpgroup every tile reads all of them from shared memory; at the
+  // power limit, where the 32k workload runs, those reads cost 2% (2624 -> 2570
+  // us). Not with padding rows, which would leave one warpgroup short of work
+  // (96 rows: 112 -> 115 us).
+  constexpr bool kSplit = RP == 128 && !kPad;
   const Tc1Params &p = lp.p;
   const int R = kPad ? p.R : RP;  // window rows
   extern __shared__ uint8_t smem_raw[];
@@ -469,7 +485,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&ms->acc_full[i], 1);
       // kO: pass-2 tiles are released by all eight epilogue warps, pass-1
       // tiles by the four of their warpgroup with two arrivals each
-      mbar_init(&ms->acc_empty[i], kO ? 8 : 4);
+      mbar_init(&ms->acc_empty[i], kSplit ? 8 : 4);
     }
     mbar_init(&ms->qs_full, 1);
     mbar_init(&ms->qs_empty, 1);
@@ -477,6 +493,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&ms->pub_full[i], 8);
       mbar_init(&ms->pub_empty[i], 1);
     }
+    for (int i = 0; i < kMaxStages; ++i) mbar_init(&ms->vr_full[i], 4);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&ms->offs_full[i], 1);
       mbar_init(&ms->offs_empty[i], 8);
@@ -787,7 +804,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_wait_ld();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cnt(&ms->acc_empty[as], kO ? 2 : 1);
+          if (lane == 0) mbar_arrive_cnt(&ms->acc_empty[as], kSplit ? 2 : 1);
           const int key0 = t * kTile + (C::Copies > 1 ? col0 : 0);  // this thread's first key
           if ((t + 1) * kTile - 1 >= p.P) {  // keys this row cannot see -> -inf
 #pragma unroll
@@ -883,6 +900,62 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (wg == 0 && got && key < p.P)
               p.votes[guard(vote0 + key, 1, (long long)p.n_slots * p.upl * p.P, p.status)] =
                   half + ms->vhalf[ptc & 1][r];
+            ++ptc;
+          }
+        } else if constexpr (kSplit) {
+          float o[64];
+          const float4 *o4 = reinterpret_cast<const float4 *>(ms->offs[ob]) + wg * 16;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float4 v4 = o4[i];
+            o[4 * i] = v4.x;
+            o[4 * i + 1] = v4.y;
+            o[4 * i + 2] = v4.z;
+            o[4 * i + 3] = v4.w;
+          }
+          for (int s = 0; s < st.n2; ++s) {
+            const int as = (tcount + s) % C::NA, ph = ((tcount + s) / C::NA) & 1;
+            const bool got = warp_wait(&ms->acc_full[as], ph, ms, p.status);
+            float half = 0.f;
+            if (got) {
+              tc_fence_after();
+              uint32_t x[2][32];
+              tmem_ld32(tmem + lane_addr + as * 128 + wg * 64, x[0]);
+              tmem_ld32(tmem + lane_addr + as * 128 + wg * 64 + 32, x[1]);
+              tmem_wait_ld();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&ms->acc_empty[as]);
+              // this half's sum as half_probs forms it
+              float2 sv[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) sv[i] = make_float2(0.f, 0.f);
+              const float2 s2 = make_float2(p.scale2, p.scale2);
+#pragma unroll
+              for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int j = 0; j < 32; j += 2) {
+                  const float2 y = __ffma2_rn(
+                      make_float2(__uint_as_float(x[c][j]), __uint_as_float(x[c][j + 1])), s2,
+                      make_float2(-o[c * 32 + j], -o[c * 32 + j + 1]));
+                  sv[(j >> 1) & 3] =
+                      __fadd2_rn(sv[(j >> 1) & 3], make_float2(fast_exp2(y.x), fast_exp2(y.y)));
+                }
+              half = ((sv[0].x + sv[0].y) + (sv[1].x + sv[1].y)) +
+                     ((sv[2].x + sv[2].y) + (sv[3].x + sv[3].y));
+            }
+            const int vs = ptc % kMaxStages;
+            if (wg == 1) {
+              ms->vring[vs][r] = half;
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&ms->vr_full[vs]);
+            } else {
+              warp_wait(&ms->vr_full[vs], (ptc / kMaxStages) & 1, ms, p.status);
+              const int key = (st.b0 + s) * kTile + r;
+              if (got && key < p.P)
+                p.votes[guard(vote0 + key, 1, (long long)p.n_slots * p.upl * p.P, p.status)] =
+                    half + ms->vring[vs][r];
+            }
             ++ptc;
           }
         } else {
