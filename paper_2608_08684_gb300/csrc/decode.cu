@@ -60,6 +60,7 @@
 #include <atomic>
 #include <chrono>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "decode.cuh"
@@ -81,7 +82,7 @@ constexpr float kRescaleLog2 = 8.f;
 constexpr int kSmemBudget = 226 * 1024;
 constexpr int kMiscBytes = 4096;              // barriers, work list, merge statistics
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kComb = 8;                      // partials of a group combined at a time
+constexpr int kMaxComb = 16;                  // partials of a group combined at a time, at most
 constexpr int kPlanPerLane = RIPPLE_MAX_LAYERS / 32;  // layers per lane of the work list
 constexpr long long kSuspendCycles = 1000000;  // wait bounds from here on suspend
 
@@ -504,36 +505,46 @@ __device__ __forceinline__ void finish_item(const DecParams &p, DecSmem<Tin, D, 
     if (s.last) {
       __threadfence();
       const long long ib = guard(item_base, f.nch, p.ws_items, p.status);
-      for (int e = tid; e < G * D; e += kWarps * 32) {
-        const int g = e / D;
-        // partials in item order, kComb at a time so that their loads overlap
-        float M = -INFINITY, num = 0.f, den = 0.f;
-        for (int c0 = 0; c0 < f.nch; c0 += kComb) {
-          float2 ml[kComb];
-          float o[kComb];
+      // partials in item order, kComb at a time so that their loads overlap (as
+      // few more than there are: 16 loads for 3 partials cost 0.6 us a step)
+      auto combine = [&](auto comb) {
+        constexpr int kComb = decltype(comb)::value;
+        for (int e = tid; e < G * D; e += kWarps * 32) {
+          const int g = e / D;
+          float M = -INFINITY, num = 0.f, den = 0.f;
+          for (int c0 = 0; c0 < f.nch; c0 += kComb) {
+            float2 ml[kComb];
+            float o[kComb];
 #pragma unroll
-          for (int c = 0; c < kComb; ++c) {
-            const size_t i = ib + min(c0 + c, f.nch - 1);
-            ml[c] = __ldcg(&p.ws_ml[i * G + g]);
-            o[c] = __ldcg(&p.ws_o[i * G * D + e]);
-            if (c0 + c >= f.nch) ml[c] = make_float2(-INFINITY, 0.f);
+            for (int c = 0; c < kComb; ++c) {
+              const size_t i = ib + min(c0 + c, f.nch - 1);
+              ml[c] = __ldcg(&p.ws_ml[i * G + g]);
+              o[c] = __ldcg(&p.ws_o[i * G * D + e]);
+              if (c0 + c >= f.nch) ml[c] = make_float2(-INFINITY, 0.f);
+            }
+            float Mn = M;
+#pragma unroll
+            for (int c = 0; c < kComb; ++c) Mn = fmaxf(Mn, ml[c].x);
+            const float a = fast_exp2(M - Mn);  // Mn is finite: every item has rows
+            num *= a;
+            den *= a;
+            M = Mn;
+#pragma unroll
+            for (int c = 0; c < kComb; ++c) {
+              const float wgt = fast_exp2(ml[c].x - M);
+              den += wgt * ml[c].y;
+              num += wgt * o[c];
+            }
           }
-          float Mn = M;
-#pragma unroll
-          for (int c = 0; c < kComb; ++c) Mn = fmaxf(Mn, ml[c].x);
-          const float a = fast_exp2(M - Mn);  // Mn is finite: every item has rows
-          num *= a;
-          den *= a;
-          M = Mn;
-#pragma unroll
-          for (int c = 0; c < kComb; ++c) {
-            const float wgt = fast_exp2(ml[c].x - M);
-            den += wgt * ml[c].y;
-            num += wgt * o[c];
-          }
+          p.out[guard(qrow * D + e, 1, (long long)p.L * p.B * p.Hq * D, p.status)] = num / den;
         }
-        p.out[guard(qrow * D + e, 1, (long long)p.L * p.B * p.Hq * D, p.status)] = num / den;
-      }
+      };
+      if (f.nch <= 4)
+        combine(std::integral_constant<int, 4>{});
+      else if (f.nch <= 8)
+        combine(std::integral_constant<int, 8>{});
+      else
+        combine(std::integral_constant<int, kMaxComb>{});
     }
   }
 }
@@ -1257,13 +1268,15 @@ int next_epoch() {
 
 // Cache rows per work item for these capacities (the workspace holds one
 // partial per item): kMaxItemRows when that already gives at least one item
-// per SM; otherwise (a single layer's step, short caches) the fewest rows, in
-// steps of kItemRowStep from kMinItemRows, whose items still fit in one wave of
-// one CTA per SM, so that no CTA takes two items one after the other and the
-// longest item is short (a graph of 32 single-layer steps over 470 to 3763
-// rows a group took 382 us, against 413 us with powers of two from 256). A step's
-// lengths are at most its capacities, so the plan's item count bounds the
-// kernel's.
+// per SM; otherwise (a single layer's step, short caches) items that fit one
+// wave of one CTA per SM, so that no CTA takes two one after the other, cut so
+// that the longest group takes the least modelled time: its item's bytes at
+// kItemBytesPerNs, plus, when the group has several items, their hand-over and
+// combination. Measured on graphs of 32 single-layer steps, 8 groups, 4 heads
+// of 128 dims, per step: one item 4.75 us + 6.6 ns a row; items of 128 rows
+// 7.5 us for 3 to 7 of them (320 rows: 210 us for the 32 layers as one item, 240
+// as three; 576 rows 264 as one, 239 as five). A step's lengths are at most
+// its capacities, so the plan's item count bounds the kernel's.
 int item_rows(const ripple_decode_desc *d, const int32_t *caps) {
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1275,13 +1288,35 @@ int item_rows(const ripple_decode_desc *d, const int32_t *caps) {
     return n;
   };
   if (items(kMaxItemRows) >= sms) return kMaxItemRows;
-  // items() only falls as the rows grow: bisect the steps
+  // the fewest rows whose items fit one wave: items() only falls as they grow,
+  // so bisect the steps
   int lo = 0, hi = (kMaxItemRows - kMinItemRows) / kItemRowStep;
   while (lo < hi) {
     const int mid = (lo + hi) / 2;
     if (items(kMinItemRows + mid * kItemRowStep) <= sms) hi = mid; else lo = mid + 1;
   }
-  return kMinItemRows + lo * kItemRowStep;
+  const int least = kMinItemRows + lo * kItemRowStep;
+  int longest = 0;
+  for (int l = 0; l < d->n_layers; ++l) longest = caps[l] > longest ? caps[l] : longest;
+  const int row_bytes = 2 * d->head_dim * (d->dtype == RIPPLE_F32 ? 4 : 2);  // K and V
+  int best = kMaxItemRows;
+  long long best_ns = -1;
+  for (int n = (longest + kMaxItemRows - 1) / kMaxItemRows; ; ++n) {
+    int rows = (longest + n - 1) / n;
+    rows = (rows + kItemRowStep - 1) / kItemRowStep * kItemRowStep;
+    if (rows > kMaxItemRows) rows = kMaxItemRows;
+    const bool end = rows <= least;
+    if (end) rows = least;
+    const int parts = (longest + rows - 1) / rows;
+    const long long ns = (long long)rows * row_bytes / kItemBytesPerNs +
+                         (parts > 1 ? 2000 + 50 * parts + (parts - 1) / kMaxComb * 900 : 0);
+    if (best_ns < 0 || ns < best_ns) {
+      best = rows;
+      best_ns = ns;
+    }
+    if (end) break;
+  }
+  return best;
 }
 
 static size_t round_up(size_t x) { return (x + 255) & ~(size_t)255; }

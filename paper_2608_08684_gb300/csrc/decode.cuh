@@ -37,6 +37,7 @@ struct DecParams {
 constexpr int kMaxItemRows = 4096;
 constexpr int kMinItemRows = 128;
 constexpr int kItemRowStep = 32;
+constexpr int kItemBytesPerNs = 77;  // an item's K and V bytes, one CTA of few
 
 // Control block of a step in the workspace (int32 words). The init flag has a
 // 128-byte line to itself; CTA 0 zeroes the counters at the start of every
