@@ -519,23 +519,27 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kCThreads)
 // are loaded coalesced straight into registers (a row more at either end is
 // the pooling halo) and a neighbour d tokens away is one select and one
 // shuffle. The K-th largest key is found by one radix round over all keys
-// (11 bits: exponent and three bits of the fraction; only the first of a
-// warp's run of equal digits, which pooling makes, adds to the histogram);
-// the keys of its bucket, if at most kPoolCand, are then copied to every CTA
-// of the unit, which finishes on them alone, without the cluster. Larger
-// buckets (many equal votes) take further rounds over all keys. Kept tokens go
-// to a list in shared memory, from which the positions are written and the
-// rows gathered.
+// (2048 bins of a 32nd of a binade; only the first of a warp's run of equal
+// digits, which pooling makes, adds to the histogram); the keys of its bucket,
+// if at most kPoolCand, are then copied to every CTA of the unit, which
+// finishes on them alone, without the cluster: up to kPoolRank of them by
+// counting, more by two rounds of 9 bits. Larger buckets (many equal votes)
+// take further rounds over all keys. Kept tokens go to a list in shared memory,
+// from which the positions are written and the rows gathered.
 //
 // Bound: latency (barriers, votes from L2) for few units, HBM of the gather for
-// many. One layer of 32 units, 32736 tokens, 1024 kept, takes 20.5 us; three
-// 11-bit rounds over 8-CTA clusters, every CTA reading all the histograms, and
-// a gather kernel took 41 us, and 256 units of 5991 tokens 98 us against 35.
+// many. One layer of 32 units, 32736 tokens, 1024 kept, takes 16.7 us
+// (17.8 with 8 bins a binade, where more atomics meet in a bin and its keys
+// take two more rounds); three 11-bit rounds over 8-CTA clusters, every CTA
+// reading all the histograms, and a gather kernel took 41 us, and 256 units of
+// 5991 tokens 98 us against 35.
 constexpr int kPoolThreads = 512;
 constexpr int kPoolWarps = kPoolThreads / 32;
 constexpr int kPoolMaxCta = 8;                       // CTAs per unit, at most
 constexpr int kPoolMaxP = kPoolMaxCta * kPoolThreads * 32;
 constexpr int kPoolCand = 2048;
+constexpr int kPoolRank = 192;                       // bucket keys ranked directly
+constexpr int kPoolBin0 = (0x80000000u >> 18) + (72 << 5);  // key >> 18 of 2^-55: bin 0
 
 struct PoolSmem {
   alignas(16) uint32_t hist[2][kBins];  // one per round parity; read 16 bytes at a time
@@ -546,6 +550,7 @@ struct PoolSmem {
   int wsum[2][kPoolWarps];
   int wgt[kPoolWarps], weq[kPoolWarps];
   int digit[2][3];              // per round parity: digit, remaining, bucket keys
+  uint32_t tau[2];              // the threshold of a small bucket and its keys kept
 };
 static_assert(offsetof(PoolSmem, cnt) % 8 == 0 && offsetof(PoolSmem, hist) % 16 == 0 &&
                   sizeof(PoolSmem) % 16 == 0,
@@ -667,25 +672,26 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
     const int live = P - w0 - lane;  // key[i] is a token's if 32 i < live
 
     // ---------------- the K-th largest key
-    // Rounds over the 31 bits below the sign bit, for the keys that have it
-    // (votes >= 0; the others, and zeros, count in the lowest bin of the first
-    // round); if the threshold falls into that bin, the search starts over on
-    // all 32 bits.
+    // First round: 64 binades of 32 bins, 2^-55 up to 2^9 (votes are sums of at
+    // most 256 probabilities); further rounds over the 18 bits below. Keys
+    // beyond (smaller, zero, negative or larger) count in the lowest and the
+    // highest bin; if the threshold falls into one of those, the search starts
+    // over on all 32 bits.
     uint32_t prefix = 0, mask = 0;
     int remaining = K;
     bool full = false;
-    auto shift_of = [&](int level) { return level == 2 ? 0 : (level == 1 ? 9 : 20) + (full ? 1 : 0); };
-    auto dmask_of = [&](int level) { return level < 2 ? 2047u : full ? 1023u : 511u; };
+    auto shift_of = [&](int level) { return level == 2 ? 0 : full ? (level == 0 ? 21 : 10) : 9; };
+    auto dmask_of = [&](int level) { return !full ? 511u : level == 2 ? 1023u : 2047u; };
     __syncthreads();  // the first histogram is clear
     for (int it = 0, level = 0; level < 3; ++it, ++level) {
       uint32_t *hist = s.hist[it & 1];
-      const int shift = shift_of(level);
-      const uint32_t dmask = dmask_of(level);
+      const bool first = level == 0 && !full;
+      const int shift = first ? 18 : shift_of(level), bin0 = first ? kPoolBin0 : 0;
+      const uint32_t dmask = first ? ~0u : dmask_of(level);
 #pragma unroll
       for (int i = 0; i < KPT; ++i) {
         const bool in = 32 * i < live && (key[i] & mask) == prefix;
-        uint32_t d = key[i] >> shift & dmask;
-        if (level == 0 && !full && !(key[i] >> 31)) d = 0;
+        uint32_t d = min(max((int)(key[i] >> shift & dmask) - bin0, 0), kBins - 1);
         // the first lane of a run of equal digits adds the run's length
         if (!in) d = 0xffffffffu;
         const uint32_t up = __shfl_up_sync(0xffffffffu, d, 1);
@@ -716,17 +722,19 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
       if (tid == 0) s.n_cand = 0;
       int digit, bucket;
       find_digit(c, remaining, it & 1, s, digit, bucket);
-      if (level == 0 && !full) {
-        if (digit == 0) {
+      if (first) {
+        if (digit == 0 || digit == kBins - 1) {
           full = true;
           remaining = K;
           level = -1;
           continue;
         }
-        prefix = mask = 0x80000000u;
+        prefix = (uint32_t)(digit + kPoolBin0) << 18;
+        mask = ~0u << 18;
+      } else {
+        prefix |= (uint32_t)digit << shift_of(level);
+        mask |= dmask_of(level) << shift_of(level);
       }
-      prefix |= (uint32_t)digit << shift;
-      mask |= dmask << shift;
       if (level == 2 || bucket > kPoolCand) continue;
       // ---------------- the bucket's keys, to every CTA of the unit
 #pragma unroll
@@ -752,7 +760,28 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
         all = s.all;
       }
       __syncthreads();
-      // the remaining rounds on those keys alone
+      if (bucket <= kPoolRank) {
+        // few: each of them counts the keys above and equal to it, and the one
+        // with remaining - 1 above and at least remaining above or equal is tau
+        if (tid < bucket) {
+          const uint32_t u = all[tid];
+          int above = 0, same = 0;
+          for (int i = 0; i < bucket; ++i) {
+            const uint32_t y = all[i];
+            above += y > u;
+            same += y == u;
+          }
+          if (above < remaining && remaining <= above + same) {
+            s.tau[0] = u;
+            s.tau[1] = (uint32_t)(remaining - above);
+          }
+        }
+        __syncthreads();
+        prefix = s.tau[0];
+        remaining = (int)s.tau[1];
+        break;
+      }
+      // else the remaining rounds on those keys alone
       for (++it, ++level; level < 3; ++it, ++level) {
         uint32_t *h2 = s.hist[it & 1];
         const int sh = shift_of(level);

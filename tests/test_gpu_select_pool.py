@@ -76,3 +76,25 @@ def test_vote_distributions(lib, kind, P):
 def test_budget_edges(lib, budget):
     votes = synth.synthetic_votes(990, 2, 9000, 0)
     _run(lib, votes, budget, 8, "max", 7, range(2))
+
+
+@pytest.mark.parametrize("n", [1, 2, 191, 192, 193, 2048, 2049])
+@pytest.mark.parametrize("base,step", [(1.0, 2.0 ** -18), (1.0, 2.0 ** -22), (2.0 ** -55, 2.0 ** -70),
+                                       (511.0, 2.0 ** -12), (600.0, 2.0 ** -10), (1e30, 1e25),
+                                       (2.0 ** -60, 2.0 ** -75), (-3.0, 2.0 ** -16)])
+def test_threshold_bucket(lib, n, base, step):
+    """n keys, half of them in pairs of equal ones, hold the threshold; the others
+    lie well above or below: bins of the first round of one key up to more than are
+    copied, inside the round's range and on either side of it."""
+    P = 9000
+    r = np.random.default_rng(n)
+    x = np.where(r.random((2, P)) < 0.3, base + abs(base), base - abs(base) / 2).astype(np.float32)
+    keep = []
+    for u in range(2):
+        at = r.choice(P, n, replace=False)
+        i = np.arange(n)
+        x[u, at] = base + step * np.where(i < n // 2, i // 2, i)
+        keep.append(int((x[u] > base + step * n).sum()))
+    for u in range(2):  # the threshold at the first, a middle and the last of them
+        for k in {keep[u] + 1, keep[u] + (n + 1) // 2, keep[u] + n}:
+            _run(lib, torch.from_numpy(x), 8 + k, 8, "none", 1, range(2))
