@@ -50,7 +50,10 @@
 // output rows (a 1/n_ch share) over the unit's partials in item order (the
 // unit's other items are done by then; a bounded wait covers the rest), so
 // the sum is deterministic and no CTA holds up the others with a whole
-// unit's sum.
+// unit's sum. Bound: HBM, which brings the keys twice and the values once (a
+// CTA's item of keys is too large to stay in L2 until its second pass, and
+// smaller items pay a step's fixed cost more often): 64 units of 256 tiles,
+// 1.6 GB, take 297 us with selection, 5.6 TB/s.
 #include <cuda.h>
 #include <math.h>
 
@@ -78,9 +81,9 @@ constexpr int kTilesPerItem = 9;
 constexpr int kTilesPerItem64 = 12;
 // kO: what a step costs on top of its item's tiles, in tiles: the item's
 // partial output, its row-slice sum, the hand-overs and the queries. Fitted to
-// 8 layers of 8 units and 256 tiles (items of 256 / 128 / 64 / 43 / 37 / 32 /
-// 19 tiles, 1 / 1 / 2 / 3 / 3 / 4 / 6 steps: 728 / 428 / 441 / 452 / 411 / 464
-// / 466 us, about 128 us and 2.34 us a tile) and to five other shapes.
+// 64 units of 256 tiles (items of 256 / 128 / 64 / 43 / 37 / 32 / 29 / 19 tiles,
+// 1 / 1 / 2 / 3 / 3 / 4 / 4 / 6 steps: 516 / 302 / 321 / 332 / 297 / 343 / 318
+// / 331 us, about 2.1 us a tile and 11 us a step).
 constexpr int kStepTilesO = 5;
 constexpr int kMaxStages = 8;
 constexpr int kOReduceLag = 2;  // kO: a step's item rows are summed this many steps later
@@ -343,11 +346,14 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 
 // Probabilities of this thread's key for 64 window rows (logit columns
 // c0 * 32 .. c0 * 32 + 63 of a pass-2 tile, x = those columns) and their sum
-// in a fixed order; with kP also as bf16 pairs (rows 2i, 2i + 1 of the 64 in
-// pk[i]), zero for the rows a window key is hidden from (hidden_below: the
-// rows of window position below it; -1 for a prefix key). A key's vote is
-// the sum of its two halves, half 0 + half 1, in every mode.
-template <bool kP>
+// in a fixed order, also as bf16 pairs (rows 2i, 2i + 1 of the 64 in pk[i]);
+// with kMask zero for the rows a window key is hidden from (hidden_below: the
+// rows of window position below it; none for a prefix key). A key's vote is
+// the sum of its two halves, half 0 + half 1, in every mode. Only the tiles of
+// the last keys are masked: one instance for all tiles, with its test at every
+// four columns, kept a thread's exponentials from overlapping (64 units of 256
+// tiles: 318 us, 297 without).
+template <bool kMask>
 __device__ __forceinline__ float half_probs(const uint32_t (&x)[2][32], const float4 *o4, int c0,
                                             float scale2, int hidden_below, int W,
                                             uint32_t (&pk)[32]) {
@@ -370,17 +376,15 @@ __device__ __forceinline__ float half_probs(const uint32_t (&x)[2][32], const fl
                                    s2, make_float2(-o.z, -o.w));
       float2 e0 = make_float2(fast_exp2(y0.x), fast_exp2(y0.y));
       float2 e1 = make_float2(fast_exp2(y1.x), fast_exp2(y1.y));
-      if constexpr (kP) {
-        if (hidden_below >= 0) {
-          const int col = c * 32 + 4 * j4;  // window row of e0.x
-          if ((col + 0) % W < hidden_below) e0.x = 0.f;
-          if ((col + 1) % W < hidden_below) e0.y = 0.f;
-          if ((col + 2) % W < hidden_below) e1.x = 0.f;
-          if ((col + 3) % W < hidden_below) e1.y = 0.f;
-        }
-        pk[(cc * 32 + 4 * j4) >> 1] = pack_bf16x2(e0.x, e0.y);
-        pk[((cc * 32 + 4 * j4) >> 1) + 1] = pack_bf16x2(e1.x, e1.y);
+      if constexpr (kMask) {
+        const int col = c * 32 + 4 * j4;  // window row of e0.x
+        if ((col + 0) % W < hidden_below) e0.x = 0.f;
+        if ((col + 1) % W < hidden_below) e0.y = 0.f;
+        if ((col + 2) % W < hidden_below) e1.x = 0.f;
+        if ((col + 3) % W < hidden_below) e1.y = 0.f;
       }
+      pk[(cc * 32 + 4 * j4) >> 1] = pack_bf16x2(e0.x, e0.y);
+      pk[((cc * 32 + 4 * j4) >> 1) + 1] = pack_bf16x2(e1.x, e1.y);
       sv[(2 * j4) & 3] = __fadd2_rn(sv[(2 * j4) & 3], e0);
       sv[(2 * j4 + 1) & 3] = __fadd2_rn(sv[(2 * j4 + 1) & 3], e1);
     }
@@ -894,8 +898,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               // a window key (or a key past the end) is seen only by the rows
               // at or after it (causal inside the window)
               uint32_t pk[32];
-              half = half_probs<true>(x, reinterpret_cast<const float4 *>(ms->offs[ob]), 2 * wg,
-                                      p.scale2, key >= p.P ? key - p.P : -1, p.W, pk);
+              const float4 *o4 = reinterpret_cast<const float4 *>(ms->offs[ob]);
+              if ((st.b0 + s + 1) * kTile > p.P)
+                half = half_probs<true>(x, o4, 2 * wg, p.scale2, key - p.P, p.W, pk);
+              else
+                half = half_probs<false>(x, o4, 2 * wg, p.scale2, 0, p.W, pk);
               // into the tile once the previous tile's probabilities have
               // been multiplied
               if (ptc > 0) warp_wait(&ms->p_empty, (ptc - 1) & 1, ms, p.status);
