@@ -943,9 +943,10 @@ cudaError_t select_long(const LayerGeom &g, int n_layers, const float *votes, co
 // 8 where they fill the CTA (P <= 4096) or where 16 leave three quarters of
 // the SMs idle, or 32 where there are CTAs for many waves, which saves cluster
 // barriers. Measured with 8 / 16 / 32 keys: one layer of 32 units and 32736
-// tokens 26.6 / 20.5 / 27.1 us, 8 units of 8160 tokens (with scoring) 39.9 /
-// 43.5 / 52.3 us, 256 units of 5991 tokens (with scoring) 143 / 136 / 166 us,
-// 1024 units of 32736 tokens (with scoring) 2872 / 2663 / 2630 us.
+// tokens 21.6 / 16.6 / 23.6 us, 8 units of 8160 tokens (with scoring) 37.1 /
+// 40.0 / 47.0 us, 1024 units of 32736 tokens (with scoring) 2754 / 2573 / 2539
+// us, and, before the first round's finer bins, 256 units of 5991 tokens (with
+// scoring) 143 / 136 / 166 us.
 void pool_shape(int P, int n_units, int *kpt, int *n_cta) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
