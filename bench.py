@@ -602,7 +602,7 @@ def measure_workloads(R, synth, dev, names, reps):
     unit and pass) against the measured sustained bf16 peak, and for decode the
     fp32 FMA fraction (q.k and p.v: 2 * d FMAs per cached row and query head)
     against the peak derived from the SM count, 128 FMA lanes per SM and the
-    maximum SM clock."""
+    maximum SM clock (a measure of the work; bf16 steps do it on the tensor cores)."""
     import torch
     hbm, _ = measured_peaks()
     tensor_peak = measured_peak("bf16_tflops_sustained", 1700.0)
