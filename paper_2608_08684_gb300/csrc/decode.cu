@@ -246,10 +246,24 @@ __device__ __forceinline__ bool wait_init(const DecParams &p, int *abort_flag) {
   }
 }
 
-// Waits until this CTA's producer has seen the init flag.
+// Block-scope acquire load / release store of a flag in shared memory: what the
+// storing thread has itself acquired (another block's writes included) is
+// ordered before what the loading thread does next.
+__device__ __forceinline__ int ld_acquire_cta(const int *p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release_cta(int *p, int v) {
+  asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+
+// Waits until this CTA's producer has seen the init flag. Release and acquire on
+// the shared word hand on what the producer acquired with the flag: CTA 0's
+// zeroing comes before this thread's counting on the counters.
 __device__ __forceinline__ bool wait_seen(const DecParams &p, const int *seen, int *abort_flag) {
   const long long t0 = clock64();
-  while (!*(const volatile int *)seen) {
+  while (!ld_acquire_cta(seen)) {
     if (*(volatile int *)abort_flag) return false;
     if (clock64() - t0 > p.wait_cycles) {
       *(volatile int *)abort_flag = 1;
@@ -257,7 +271,6 @@ __device__ __forceinline__ bool wait_seen(const DecParams &p, const int *seen, i
       return false;
     }
   }
-  __threadfence_block();
   return true;
 }
 
@@ -376,7 +389,7 @@ __device__ __forceinline__ void produce(const DecParams &p, DecSmem<Tin, D, G> &
   // wait for in shared memory: from here on it needs neither.
   auto arrive = [&] {  // lane 0, once, before the first item's end
     if (see_init()) {
-      *(volatile int *)&s.init_seen = 1;
+      st_release_cta(&s.init_seen, 1);
       atomicAdd(&p.ctrl[kCtrlArrived], 1);
     }
   };
