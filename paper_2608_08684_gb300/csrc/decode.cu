@@ -802,17 +802,24 @@ __device__ __forceinline__ void mma_16x8x16(float (&c)[4], uint32_t a0, uint32_t
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t *>(&b);
+// The high halves of two fp32 values: both cut to bf16.
+__device__ __forceinline__ uint32_t high_halves(float x0, float x1) {
+  return __byte_perm(__float_as_uint(x0), __float_as_uint(x1), 0x7632);
 }
-// A pair of fp32 values as the sum of three bf16 pairs: 24 bits of each, so
-// that products with bf16 values lose nothing against fp32.
+// x less its bf16 part, at least 2^-125 (whose half is a normal value still).
+__device__ __forceinline__ float below_bf16(float x) {
+  return fmaxf(x - __uint_as_float(__float_as_uint(x) & 0xffff0000u), 0x1p-125f);
+}
+// A pair of fp32 values >= 0 as h + m + 2 l, bf16 pairs: 24 bits of each, so
+// that products with bf16 values lose nothing against fp32. Each part is cut off,
+// not rounded, and m and l are never 0: no part of a positive probability times
+// an infinite value is a NaN or has the other sign (with rounded parts every
+// output of a column with an infinite value was NaN).
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t &h, uint32_t &m, uint32_t &l) {
-  h = pack_bf16(x0, x1);
-  const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xffff0000u);
-  m = pack_bf16(r0, r1);
-  l = pack_bf16(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xffff0000u));
+  h = high_halves(x0, x1);
+  const float r0 = below_bf16(x0), r1 = below_bf16(x1);
+  m = high_halves(r0, r1);
+  l = high_halves(0.5f * below_bf16(r0), 0.5f * below_bf16(r1));
 }
 
 // The compute warps of a bf16 step. Per 16 cache rows (two blocks of 8 keys):
@@ -822,9 +829,11 @@ __device__ __forceinline__ void split3(float x0, float x1, uint32_t &h, uint32_t
 //   output   O[row][dim] += P . V with the probabilities, as they lie, as the
 //            A operand and V (ldmatrix.trans) as B. A probability is split
 //            into three bf16 parts that fill the operand's 16 rows: 8 heads
-//            take rows 0-7 (high parts), 8-15 (middle) and a second MMA (low);
-//            up to 4 heads repeat in rows 4-7 and take rows 0-3 (high), 4-7
-//            (middle) and 8-11 (low) of one MMA.
+//            take rows 0-7 (high parts), 8-15 (middle) and a second MMA (half
+//            of the low part on all 16); up to 4 heads repeat in rows 4-7 and
+//            take rows 0-3 (high), 4-7 (middle) and 8-15 (half of the low part,
+//            twice) of one MMA. No row of a head holds a 0 for a positive
+//            probability, which an infinite value would turn into a NaN.
 // Matrix instructions cut their sums off rather than round them, so only short
 // chains stay in their accumulators (32 dims of a score, 16 rows of an output)
 // and the rest is added on the fp32 pipes.
@@ -954,7 +963,7 @@ __device__ __forceinline__ void consume_mma(const DecParams &p,
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         a0[i] = kWide || g < 4 ? hi[i] : mi[i];
-        a1[i] = kWide ? mi[i] : (g < 4 ? lo[i] : 0u);
+        a1[i] = kWide ? mi[i] : lo[i];
       }
 #pragma unroll
       for (int b2 = 0; b2 < NB / 2; ++b2) {
@@ -967,7 +976,7 @@ __device__ __forceinline__ void consume_mma(const DecParams &p,
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           float part[4] = {0.f, 0.f, 0.f, 0.f};
-          if (kWide) mma_16x8x16(part, lo[0], 0u, lo[1], 0u, vb[2 * e], vb[2 * e + 1]);
+          if (kWide) mma_16x8x16(part, lo[0], lo[0], lo[1], lo[1], vb[2 * e], vb[2 * e + 1]);
           mma_16x8x16(part, a0[0], a1[0], a0[1], a1[1], vb[2 * e], vb[2 * e + 1]);
           acc[2 * b2 + e] =
               __fadd2_rn(acc[2 * b2 + e], make_float2(part[0] + part[2], part[1] + part[3]));

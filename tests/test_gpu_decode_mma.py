@@ -66,3 +66,46 @@ def test_rows_past_the_cache_never_count(lib, G, d):
     assert int(s.status.item()) == 0
     assert np.isfinite(got[1:]).all()
     _check(wl, lens0, kc, vc, q, kn, vn, got, [1, 2], [(0, 0), (41, 2), (79, 3)])
+
+
+@pytest.mark.parametrize("G,d", [(1, 64), (2, 128), (4, 128), (8, 64), (8, 128)])
+def test_infinite_values_stay_infinite(lib, G, d):
+    # A probability is positive, so a column that holds an infinite value has an
+    # infinite output, whatever parts the probability is split into (1, of one
+    # bf16 part, and the largest of a row included); the other columns stay as
+    # they are.
+    wl = synth.WORKLOADS["tiny"].replace(n_layers=4, batch=1, n_q_heads=2 * G, n_kv_heads=2,
+                                         head_dim=d, dtype="bf16", seed=760 + G + d)
+    lens0 = [1, 40, 300, 5000]
+    kc, vc = zip(*[synth.decode_caches(wl, i, n + 2) for i, n in enumerate(lens0)])
+    for i, n in enumerate(lens0):
+        vc[i][0, 0, 0, 3] = float("inf")
+        vc[i][0, 0, n // 2, d - 1] = -float("inf")
+        vc[i][0, 1, n - 1, d // 2] = float("inf")
+        vc[i][0, 1, : n // 2 + 1, 7] = -float("inf")
+    s, q, kn, vn, got = _step(lib, wl, lens0, kc, vc)
+    assert int(s.status.item()) == 0
+    bad = np.zeros((2, d), np.float64)
+    bad[0, 3], bad[0, d - 1], bad[1, d // 2], bad[1, 7] = np.inf, -np.inf, np.inf, -np.inf
+    for i in range(len(lens0)):
+        for h in range(2):
+            at = np.isinf(bad[h])
+            o = got[i, 0, h * G:(h + 1) * G]
+            assert (o[:, at] == bad[h][at]).all(), (i, h, o[:, at])
+            vc[i][0, h][:, at] = 0.0
+    _check(wl, lens0, kc, vc, q, kn, _zeroed(vn, bad), _zero_cols(got, bad, G),
+           range(len(lens0)), [(0, 0), (0, 1)])
+
+
+def _zeroed(vn, bad):
+    vn = vn.clone()
+    for h in range(2):
+        vn[:, 0, h, np.isinf(bad[h])] = 0.0
+    return vn
+
+
+def _zero_cols(got, bad, G):
+    got = got.copy()
+    for h in range(2):
+        got[:, 0, h * G:(h + 1) * G, np.isinf(bad[h])] = 0.0
+    return got
