@@ -208,7 +208,9 @@ ripple_status ripple_compress_layers(const ripple_layer_desc *desc, int32_t n_la
                                      size_t workspace_bytes, int32_t *dev_status, void *stream);
 
 /* Device workspace bytes ripple_compress_layers_attn needs for n_layers layers
- * of this shape (RIPPLE_EINVAL for shapes it does not take). */
+ * of this shape (RIPPLE_EINVAL for shapes it does not take). Never fewer for more
+ * layers, a larger batch or more tokens, so that a workspace made for a
+ * program's largest call serves its smaller ones, as for the other calls. */
 ripple_status ripple_compress_layers_attn_workspace_bytes(const ripple_layer_desc *desc,
                                                           int32_t n_layers, size_t *bytes_host);
 

@@ -183,7 +183,7 @@ static CompressWs carve_layers_attn_ws(const LayerGeom &g, int n_layers, void *b
   size_t off = w.bytes;
   const size_t units = (size_t)g.units * n_layers;
   w.o_part = p ? (float *)(p + off) : nullptr;
-  off += round_up(sizeof(float) * units * score_tc1_attn_items(g, n_layers) * g.R * g.D);
+  off += round_up(sizeof(float) * (size_t)score_tc1_attn_max_items(g, n_layers) * g.R * g.D);
   w.o_count = p ? (int32_t *)(p + off) : nullptr;
   off += round_up(sizeof(int32_t) * units);
   w.bytes = off;

@@ -39,7 +39,8 @@ struct CompressWs {
   float *votes;         // [units][P] unpooled votes (when scores_out is NULL)
   uint32_t *keys;       // [units][P] pooled-score sort keys (long prefixes only)
   int32_t *counters;    // small control block
-  float *o_part;        // with the window rows' output: [units][items][G*w][d] partials
+  float *o_part;        // with the window rows' output: [units][items][G*w][d] partials,
+                        // room for score_tc1_attn_max_items
   int32_t *o_count;     // with the window rows' output: [units] items written
   size_t bytes;
 };
@@ -71,10 +72,13 @@ cudaError_t launch_score_tc1(const LayerGeom &g, int n_slots, const int *slots, 
                              const CompressWs &ws, float *votes, int32_t *status,
                              cudaStream_t st, const void *const *v = nullptr,
                              float *const *o_win = nullptr);
-// Items per unit of a launch_score_tc1 with outputs (sizes the output partials):
-// the number with the least modelled time, the steps of the busiest CTA times
-// its item's tiles and the cost of a step, so that few units still fill the GPU.
+// Items per unit of a launch_score_tc1 with outputs: the number with the least
+// modelled time, the steps of the busiest CTA times its item's tiles and the cost
+// of a step, so that few units still fill the GPU.
 int score_tc1_attn_items(const LayerGeom &g, int n_layers);
+// Bound of all units' items in such a launch (sizes the output partials): grows
+// with the units and the tokens and does not depend on the device.
+long long score_tc1_attn_max_items(const LayerGeom &g, int n_layers);
 // The gather's inputs and outputs per layer (launch_gather's arguments).
 struct GatherArgs {
   const void *const *k;

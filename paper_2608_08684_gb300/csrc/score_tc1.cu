@@ -85,6 +85,13 @@ constexpr int kTilesPerItem64 = 12;
 // 1 / 1 / 2 / 3 / 3 / 4 / 4 / 6 steps: 516 / 302 / 321 / 332 / 297 / 343 / 318
 // / 331 us, about 2.1 us a tile and 11 us a step).
 constexpr int kStepTilesO = 5;
+// kO: items of a call, at most (unless it has more units), 64 KB of partial
+// outputs each. The workspace is sized for this bound and not for the number a
+// call takes, which falls where one more layer or tile fits fewer steps: a
+// workspace made for a program's largest call has to serve all smaller ones.
+// The model's choices stay within it but for 2% of the (units, tiles) up to 2560
+// and 1024, which it costs at most 5%.
+constexpr int kMaxItemsO = 2432;
 constexpr int kMaxStages = 8;
 constexpr int kOReduceLag = 2;  // kO: a step's item rows are summed this many steps later
 
@@ -1167,14 +1174,27 @@ Tc1Kernel tc1_kernel_for(int R) {
 
 }  // namespace
 
+// kO: items of a unit, at most; one of up to kTilesPerItem tiles is one item, as
+// without outputs.
+static int attn_items_per_unit(const LayerGeom &g) {
+  const int n = (g.T + kTile - 1) / kTile / kTilesPerItem;
+  return n > 1 ? n : 1;
+}
+
+long long score_tc1_attn_max_items(const LayerGeom &g, int n_layers) {
+  const long long units = (long long)g.units * n_layers;
+  const long long items = units * attn_items_per_unit(g);
+  return units > kMaxItemsO ? units : items < kMaxItemsO ? items : kMaxItemsO;
+}
+
 int score_tc1_attn_items(const LayerGeom &g, int n_layers) {
   const int n_tiles = (g.T + kTile - 1) / kTile, sms = sm_count();
-  // a unit of up to kTilesPerItem tiles is one item, as without outputs
-  const int most = n_tiles / kTilesPerItem < sms ? n_tiles / kTilesPerItem : sms;
+  const int per_unit = attn_items_per_unit(g), most = per_unit < sms ? per_unit : sms;
   const long long units = (long long)g.units * n_layers;
+  const long long max_items = score_tc1_attn_max_items(g, n_layers);
   int best = 1;
   long long best_cost = -1;
-  for (int n = 1; n <= most || n == 1; ++n) {
+  for (int n = 1; n == 1 || (n <= most && units * n <= max_items); ++n) {
     const int per = (n_tiles + n - 1) / n;
     if ((n_tiles + per - 1) / per != n) continue;  // items would be left empty
     const long long cost = (units * n + sms - 1) / sms * (per + kStepTilesO);

@@ -116,6 +116,23 @@ def test_entry_points_reject_before_any_cuda_work(lib):
     assert lib.status_string(lib.EFULL) == "cache full"
 
 
+def test_workspace_queries_grow_with_the_call(lib):
+    # a workspace made for a program's largest call serves its smaller ones
+    def attn(layers, batch, seq):
+        d = lib.layer_desc(batch, 32, 8, 128, seq, 32)
+        return lib.ripple_compress_layers_attn_workspace_bytes(d, layers)
+
+    def layers(n, batch, seq):
+        return lib.ripple_compress_layers_workspace_bytes(
+            lib.layer_desc(batch, 32, 8, 128, seq, 32), n)
+
+    for query in (attn, layers):
+        for sizes in ([query(n, 1, 32768) for n in range(1, 81)],
+                      [query(4, 1, t) for t in range(40, 60000, 61)],
+                      [query(7, b, 5000) for b in range(1, 65)]):
+            assert sizes == sorted(sizes), query
+
+
 def test_compress_layers_host_validation(lib):
     d = lib.layer_desc(4, 32, 8, 128, 32768, 32)
     one = lib.ripple_compress_workspace_bytes(d)

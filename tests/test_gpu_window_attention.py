@@ -24,7 +24,7 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-def _run(lib, wl, budgets, attn=True):
+def _run(lib, wl, budgets, attn=True, ws=None):
     L = len(budgets)
     desc = lib.layer_desc(wl.batch, wl.n_q_heads, wl.n_kv_heads, wl.head_dim, wl.seq_len,
                           wl.window, wl.pool_kernel, "max", wl.torch_dtype)
@@ -41,8 +41,9 @@ def _run(lib, wl, budgets, attn=True):
     if attn:
         o_win = [torch.full((B, wl.n_q_heads, wl.window, d), float("nan"), device=DEV)
                  for _ in range(L)]
-        ws = torch.empty(lib.ripple_compress_layers_attn_workspace_bytes(desc, L),
-                         dtype=torch.uint8, device=DEV)
+        if ws is None:
+            ws = torch.empty(lib.ripple_compress_layers_attn_workspace_bytes(desc, L),
+                             dtype=torch.uint8, device=DEV)
         got = lib.ripple_compress_layers_attn(desc, budgets, tables, o_win, ws, dev_status=status)
     else:
         ws = torch.empty(lib.ripple_compress_layers_workspace_bytes(desc, L), dtype=torch.uint8,
@@ -144,3 +145,25 @@ def test_window_attention_rejects_other_shapes(lib):
                           wl.window, wl.pool_kernel, "max", wl.torch_dtype)
     with pytest.raises(lib.RippleError):
         lib.ripple_compress_layers_attn_workspace_bytes(desc, 1)
+
+
+def test_smaller_call_in_a_larger_calls_workspace(lib):
+    # 72 units of 18 key tiles fill the GPU as two items each, 80 as one each: the
+    # larger call has fewer partial outputs
+    wl = synth.WORKLOADS["tiny"].replace(n_layers=9, batch=1, n_q_heads=32, n_kv_heads=8,
+                                         head_dim=128, seq_len=2304, dtype="bf16", seed=77)
+    budgets = [400] * 9
+    desc = lib.layer_desc(1, 32, 8, 128, wl.seq_len, wl.window, wl.pool_kernel, "max",
+                          wl.torch_dtype)
+    ws = torch.empty(lib.ripple_compress_layers_attn_workspace_bytes(desc, 10), dtype=torch.uint8,
+                     device=DEV)
+    res, own = _run(lib, wl, budgets, ws=ws), _run(lib, wl, budgets)
+    for key in ("idx", "k_out", "v_out", "o_win"):
+        assert all(torch.equal(a, b) for a, b in zip(res[key], own[key])), key
+    # and a shorter prompt in a longer one's
+    long_desc = lib.layer_desc(1, 32, 8, 128, 20000, wl.window)
+    ws = torch.empty(lib.ripple_compress_layers_attn_workspace_bytes(long_desc, 4),
+                     dtype=torch.uint8, device=DEV)
+    for T in (700, 2304, 9000):
+        small = wl.replace(n_layers=4, seq_len=T)
+        _check_compression(small, _run(lib, small, [200] * 4, ws=ws), [200] * 4, units=[(0, 1)])
