@@ -285,7 +285,9 @@ typedef struct {
   float scale;        /* logit scale; 0 means 1/sqrt(head_dim) */
 } ripple_decode_desc;
 
-/* Device workspace bytes ripple_decode_attn needs for these layers' capacities. */
+/* Device workspace bytes ripple_decode_attn needs for these layers' capacities
+ * on the current device. Never fewer for more layers, a larger batch or larger
+ * capacities: a workspace made for a program's largest step serves all. */
 ripple_status ripple_decode_workspace_bytes(const ripple_decode_desc *desc,
                                             const int32_t *caps_host, size_t *bytes_host);
 

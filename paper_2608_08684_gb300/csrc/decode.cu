@@ -57,6 +57,7 @@
 // roles leave their loops together.
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <mutex>
@@ -1288,27 +1289,28 @@ int next_epoch() {
   return (int)e;
 }
 
-// Cache rows per work item for these capacities (the workspace holds one
-// partial per item): kMaxItemRows when that already gives at least one item
-// per SM; otherwise (a single layer's step, short caches) items that fit one
-// wave of one CTA per SM, so that no CTA takes two one after the other, cut so
-// that the longest group takes the least modelled time: its item's bytes at
-// kItemBytesPerNs, plus, when the group has several items, their hand-over and
-// combination. Measured on graphs of 32 single-layer steps, 8 groups, 4 heads
+// Work items of these capacities cut into `rows` cache rows each.
+long long items_of(const ripple_decode_desc *d, const int32_t *caps, int rows) {
+  long long n = 0;
+  for (int l = 0; l < d->n_layers; ++l)
+    n += (long long)d->batch * d->n_kv_heads * ((caps[l] + rows - 1) / rows);
+  return n;
+}
+
+// Cache rows per work item for these capacities: kMaxItemRows when that already
+// gives at least one item per SM; otherwise (a single layer's step, short caches)
+// items that fit one wave of one CTA per SM, so that no CTA takes two one after
+// the other, cut so that the longest group takes the least modelled time: its
+// item's bytes at kItemBytesPerNs, plus, when the group has several items, their
+// hand-over and combination. Measured on graphs of 32 single-layer steps, 8 groups, 4 heads
 // of 128 dims, per step: one item 4.75 us + 6.6 ns a row; items of 128 rows
 // 7.5 us for 3 to 7 of them (320 rows: 210 us for the 32 layers as one item, 240
-// as three; 576 rows 264 as one, 239 as five). A step's lengths are at most
-// its capacities, so the plan's item count bounds the kernel's.
+// as three; 576 rows 264 as one, 239 as five).
 int item_rows(const ripple_decode_desc *d, const int32_t *caps) {
   int dev = 0;
   cudaGetDevice(&dev);
   const long long sms = sm_count(dev);
-  auto items = [&](int rows) {
-    long long n = 0;
-    for (int l = 0; l < d->n_layers; ++l)
-      n += (long long)d->batch * d->n_kv_heads * ((caps[l] + rows - 1) / rows);
-    return n;
-  };
+  auto items = [&](int rows) { return items_of(d, caps, rows); };
   if (items(kMaxItemRows) >= sms) return kMaxItemRows;
   // the fewest rows whose items fit one wave: items() only falls as they grow,
   // so bisect the steps
@@ -1344,20 +1346,28 @@ int item_rows(const ripple_decode_desc *d, const int32_t *caps) {
 static size_t round_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Workspace layout for these capacities: control block, partial (max, sum),
-// partial outputs. Returns the total bytes; fills p's pointers if given.
+// partial outputs. Returns the total bytes; fills p's pointers if given. The
+// partials are not counted by the items of item_rows, whose number falls where
+// some more rows are cut differently (caches of 2048 rows take 16 items a group,
+// of 2080 rows 13), but by a bound of them that grows with the layers, the batch
+// and every capacity: a workspace made for a program's largest step has to
+// serve all smaller ones. It bounds the kernel's items, since a step's lengths
+// are at most its capacities.
 size_t plan(const ripple_decode_desc *d, const int32_t *caps, void *ws, DecParams *p) {
   const int G = d->n_q_heads / d->n_kv_heads;
-  const int rows = item_rows(d, caps);
-  size_t items = 0;
-  for (int l = 0; l < d->n_layers; ++l)
-    items += (size_t)d->batch * d->n_kv_heads * ((caps[l] + rows - 1) / rows);
+  int dev = 0;
+  cudaGetDevice(&dev);
+  // item_rows cuts into one wave at most, of items of at least kMinItemRows, or
+  // into items of kMaxItemRows
+  const long long wave = std::min<long long>(items_of(d, caps, kMinItemRows), sm_count(dev));
+  const size_t items = (size_t)std::max<long long>(items_of(d, caps, kMaxItemRows), wave);
   const size_t groups = (size_t)d->n_layers * d->batch * d->n_kv_heads;
   const size_t ctrl = round_up(sizeof(int) * (kCtrlGroup + groups));
   const size_t ml = round_up(sizeof(float2) * items * G);
   const size_t o = round_up(sizeof(float) * items * G * d->head_dim);
   if (p != nullptr) {
     uint8_t *base = (uint8_t *)ws;
-    p->item_rows = rows;
+    p->item_rows = item_rows(d, caps);
     p->ws_items = (long long)items;
     p->n_ctrl = (int)(kCtrlGroup + groups);
     p->ctrl = (int *)base;

@@ -325,3 +325,28 @@ def test_workspace_reallocated_at_the_same_address(lib):
         assert int(b.status.item()) == 0
         np.testing.assert_array_equal(got, want)
     print(f"workspace handed back at the same address in {reused} of 3 steps")
+
+
+def test_smaller_steps_in_a_larger_steps_workspace(lib):
+    # caches of 2048 rows are cut into more items than caches of 2080: the
+    # workspace is sized by a bound that grows with the capacities
+    def need(caps, batch=1, hq=32, hkv=8):
+        return lib.ripple_decode_workspace_bytes(
+            lib.decode_desc(len(caps), batch, hq, hkv, 128, torch.bfloat16), caps)
+
+    for sizes in ([need([c]) for c in range(1, 12000, 7)],
+                  [need([c] * 4, hq=8, hkv=1) for c in range(1, 40000, 97)],
+                  [need([300] * n) for n in range(1, 129)],
+                  [need([3000], batch=b) for b in range(1, 65)]):
+        assert sizes == sorted(sizes)
+    wl = synth.WORKLOADS["tiny"].replace(n_layers=1, batch=1, n_q_heads=32, n_kv_heads=8,
+                                         head_dim=128, dtype="bf16", seed=78)
+    for small, large in ((2048, 2080), (1024, 1030), (4096, 4100)):
+        ws = torch.empty(need([large]), dtype=torch.uint8, device=DEV)
+        kc, vc = synth.decode_caches(wl, 0, small)
+        q, kn, vn = synth.decode_inputs(wl, 0)
+        own = Session(lib, wl, [0], [small], [small - 1], [kc], [vc])
+        shared = Session(lib, wl, [0], [small], [small - 1], [kc], [vc])
+        shared.ws = ws
+        np.testing.assert_array_equal(shared.step(q, kn, vn), own.step(q, kn, vn))
+        assert int(shared.status.item()) == 0
