@@ -209,6 +209,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int NR = C::NR;
   constexpr int kTileBytes = C::TileBytes;
   const TcParams &p = lp.p;
+  // window rows, a constant without padding: with the count from the parameters
+  // the loads of a merge were predicated one by one and overlapped less (5 to 15
+  // us a call of one layer)
+  const int R = kPad ? p.R : C::R;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *ktiles = smem + C::OFF_K;
@@ -306,10 +310,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&ms->q_full, (uint32_t)(p.R * D * 2));
+          mbar_arrive_expect_tx(&ms->q_full, (uint32_t)(R * D * 2));
 #pragma unroll
           for (int half = 0; half < D / 64; ++half)
-            tma_load_2d(qbufs + half * (NR * kHalfBytes), qm, half * 64, local * p.R, &ms->q_full);
+            tma_load_2d(qbufs + half * (NR * kHalfBytes), qm, half * 64, local * R, &ms->q_full);
           ++qcount;
         }
       }
@@ -391,14 +395,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       // One partial per item: the two warpgroups' statistics combined here.
       float2 *mine = p.partial + guard((long long)it.unit * p.n_ch + it.chunk, 1,
                                        (long long)p.units * p.n_ch, p.status) *
-                                     p.R;
+                                     R;
 #pragma unroll
       for (int j = 0; j < RJ; ++j) {
         const int r = lane + 32 * j;
         float2 a = ms->pstat[slot][0][r];
         const float2 b = ms->pstat[slot][1][r];
         combine(a.x, a.y, b.x, b.y);
-        if (r < p.R) mine[r] = a;
+        if (r < R) mine[r] = a;
       }
       __syncwarp();  // all lanes' rows are written (and the slot read) before lane 0 goes on
       int last = 0;
@@ -414,7 +418,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float2 *part =
             p.partial + guard((long long)it.unit * p.n_ch, p.n_ch, (long long)p.units * p.n_ch,
                               p.status) *
-                            p.R;
+                            R;
         float mm[RJ], ll[RJ];
 #pragma unroll
         for (int j = 0; j < RJ; ++j) {
@@ -427,8 +431,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int c = 0; c < CB; ++c)
 #pragma unroll
             for (int j = 0; j < RJ; ++j)
-              q[c][j] = c0 + c < p.n_ch && lane + 32 * j < p.R
-                            ? __ldcg(&part[(size_t)(c0 + c) * p.R + lane + 32 * j])
+              q[c][j] = c0 + c < p.n_ch && lane + 32 * j < R
+                            ? __ldcg(&part[(size_t)(c0 + c) * R + lane + 32 * j])
                             : make_float2(-INFINITY, 0.f);
 #pragma unroll
           for (int c = 0; c < CB; ++c)
@@ -437,8 +441,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
 #pragma unroll
         for (int j = 0; j < RJ; ++j)
-          if (lane + 32 * j < p.R)
-            p.lognorm[guard(it.unit, 1, p.units, p.status) * p.R + lane + 32 * j] =
+          if (lane + 32 * j < R)
+            p.lognorm[guard(it.unit, 1, p.units, p.status) * R + lane + 32 * j] =
                 mm[j] + __log2f(ll[j]);
         __threadfence();
         __syncwarp();
@@ -544,8 +548,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (wtid == 0)
             wait_ready(&p.ctrl[guard(p.units + it.unit, 1, 2LL * p.units, p.status)], ms, p.status);
           named_bar_sync(3 + wg, 128);
-          for (int r = wtid; r < p.R; r += 128)
-            ms->off[wg][r] = __ldcg(&p.lognorm[guard(it.unit, 1, p.units, p.status) * p.R + r]);
+          for (int r = wtid; r < R; r += 128)
+            ms->off[wg][r] = __ldcg(&p.lognorm[guard(it.unit, 1, p.units, p.status) * R + r]);
           named_bar_sync(3 + wg, 128);
         }
         const float4 *off4 = (const float4 *)ms->off[wg];
@@ -587,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float2 e0 = make_float2(fast_exp2(y0.x), fast_exp2(y0.y));
                 float2 e1 = make_float2(fast_exp2(y1.x), fast_exp2(y1.y));
                 if constexpr (decltype(some_padding)::value) {
-                  const int left = p.R - (c4 * 128 + c * 32 + j);  // rows from this column on
+                  const int left = R - (c4 * 128 + c * 32 + j);  // rows from this column on
                   if (left < 1) e0.x = 0.f;
                   if (left < 2) e0.y = 0.f;
                   if (left < 3) e1.x = 0.f;
@@ -600,9 +604,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               const int first = c4 * 128 + c * 32;
-              if (!kPad || first + 32 <= p.R)
+              if (!kPad || first + 32 <= R)
                 columns(c, std::false_type{});
-              else if (first < p.R)
+              else if (first < R)
                 columns(c, std::true_type{});
             }
           }
