@@ -36,6 +36,7 @@
 #include <cuda.h>
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -52,13 +53,24 @@ constexpr int kThreads = 352;
 constexpr int kPubSlots = 2;
 // A unit is cut into items of 8 tiles (up to 64 tiles) or 16, but at most 16
 // items: more partial statistics take the one publisher that merges them too
-// long, and fewer items leave small calls on few SMs. One 8k-token layer of 8
-// units took 161 / 63 / 54 / 49 us with items of 64 / 16 / 12 / 8 tiles, 16
-// layers of 256 tiles 628 / 600 / 641 us with 64 / 16 / 15, 16 layers of 1024
-// tiles 2181 / 2207 / 2267 us with 64 / 57 / 86 (16 / 18 / 12 items).
+// long, and fewer items leave small calls on few SMs. A function of the layer's
+// shape alone, so that one layer's call and a multi-layer call merge the same
+// statistics. Measured with items of 4 / 8 / 16 / 32 / 64 tiles, us a call:
+//   64 tiles, one layer of 8 units     40 /   46 /   63 /   96 /  161
+//   64 tiles, 32 such layers          335 /  312 /  296 /  319 /  316
+//   65 tiles, one layer of 8 units     40 /   48 /   58 /   75 /   97
+//   65 tiles, 32 such layers          386 /  370 /  325 /  343 /  350
+//   128 tiles, one layer of 8 units    54 /   48 /   63 /   96 /  162
+//   128 tiles, 16 such layers         379 /  302 /  288 /  312 /  312
+//   1024 tiles, 16 such layers             3546 / 2188 / 2024 / 2011
+// Smaller items gain a single layer and cost many layers, which decide from 65
+// tiles on.
+// Prompts of more than 1024 tiles take up to an item per 64 tiles where those fill
+// the SMs better in a layer's units (items_per_unit).
 constexpr int kTilesPerItem = 16, kTilesPerItemShort = 8;
 constexpr int kShortTiles = 64;
 constexpr int kMaxItems = 16;
+constexpr int kTilesPerItemLong = 64;
 
 
 // ------------------------------------------------------------ work list
@@ -657,6 +669,27 @@ int sm_count() {
   return n > 0 ? n : 1;
 }
 
+// Items a unit of n_tiles key tiles is cut into, in layers of `units` units: see
+// kTilesPerItem. Between 16 and an item per 64 tiles the number with the least
+// modelled time is taken, the layer's waves of items times an item's tiles (more
+// items by 2% or not): one unit of 4096 tiles 1049 us in 64 items, 1461 in 16; 4
+// units of 1563 tiles 217 us in 25, 281 in 16; 8 of 4096 tiles 1348 us in 19, 1430
+// in 16, 1524 in 64; 16 of 1172 tiles 352 us in 19, 400 in 16. No more items than
+// SMs (the schedule is free of deadlock up to twice as many).
+int items_per_unit(int n_tiles, int units, int sms) {
+  const int per = n_tiles <= kShortTiles ? kTilesPerItemShort : kTilesPerItem;
+  const int items = (n_tiles + per - 1) / per;
+  if (items <= kMaxItems) return std::min(items, sms);
+  const int most = std::min((n_tiles + kTilesPerItemLong - 1) / kTilesPerItemLong, sms);
+  int best = std::min(kMaxItems, sms);
+  auto cost = [&](int n) {
+    return ((long long)units * n + sms - 1) / sms * ((n_tiles + n - 1) / n);
+  };
+  for (int n = best + 1; n <= most; ++n)
+    if (cost(n) * 50 < cost(best) * 49) best = n;
+  return best;
+}
+
 template <int D>
 cudaError_t launch_d(const LayerGeom &g, int n_slots, const int *slots, int n_scored,
                       const void *const *q_win, const void *const *k, const CompressWs &ws,
@@ -695,11 +728,7 @@ cudaError_t launch_d(const LayerGeom &g, int n_slots, const int *slots, int n_sc
   p.R = g.R;
   p.n_tiles1 = (g.T + kTile - 1) / kTile;
   p.n_tiles2 = (g.P + kTile - 1) / kTile;
-  // (and no more items than SMs: deadlock-free schedule, see the header comment)
-  const int per = p.n_tiles1 <= kShortTiles ? kTilesPerItemShort : kTilesPerItem;
-  const int items = (p.n_tiles1 + per - 1) / per;
-  p.n_ch = items < kMaxItems ? items : kMaxItems;
-  p.n_ch = p.n_ch < sms ? p.n_ch : sms;
+  p.n_ch = items_per_unit(p.n_tiles1, g.units, sms);
   p.tpi = (p.n_tiles1 + p.n_ch - 1) / p.n_ch;
   p.n_ch = (p.n_tiles1 + p.tpi - 1) / p.tpi;
   p.total_items = p.units * p.n_ch;

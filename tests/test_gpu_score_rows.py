@@ -20,7 +20,11 @@ SHAPES = [
 ]
 
 
-@pytest.mark.parametrize("G,w,d,T", SHAPES)
+# few units of more than 1024 tiles: items of 64 tiles, more than 16 a unit
+LONG = [(8, 32, 64, 140900)]
+
+
+@pytest.mark.parametrize("G,w,d,T", SHAPES + LONG)
 def test_votes_and_selection_match_oracle(lib, G, w, d, T):
     wl = synth.WORKLOADS["tiny"].replace(
         batch=1, n_q_heads=2 * G, n_kv_heads=2, head_dim=d, seq_len=T, window=w, dtype="bf16",
