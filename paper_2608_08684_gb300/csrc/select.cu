@@ -302,8 +302,8 @@ struct SelTable {
   int n_keep[kCompressMaxLayers];
   int32_t *idx[kCompressMaxLayers];
   int32_t *status;
-  // select_pool_kernel, which also copies each unit's kept rows:
-  int row_bytes;
+  // select_pool_kernel, which also copies each unit's kept rows (with gather):
+  int row_bytes, gather;
   const uint8_t *k[kCompressMaxLayers];
   const uint8_t *v[kCompressMaxLayers];
   uint8_t *k_out[kCompressMaxLayers];
@@ -525,7 +525,8 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kCThreads)
 // finishes on them alone, without the cluster: up to kPoolRank of them by
 // counting, more by two rounds of 9 bits. Larger buckets (many equal votes)
 // take further rounds over all keys. Kept tokens go to a list in shared memory,
-// from which the positions are written and the rows gathered.
+// from which the positions are written and the rows gathered (or the gather kernel
+// copies them, gather_apart).
 //
 // Bound: latency (barriers, votes from L2) for few units, HBM of the gather for
 // many. One layer of 32 units, 32736 tokens, 1024 kept, takes 16.7 us
@@ -868,31 +869,33 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
   const int local = unit % tab.upl;
   int32_t *out = tab.idx[layer] + (size_t)local * n_keep + first;
   for (int i = tid; i < rows; i += kPoolThreads) out[i] = list[i];
-  // row_bytes / 16 consecutive threads copy one row 16 bytes each, four rows a
-  // thread in flight
-  const int rb = tab.row_bytes, lpr = rb >> 4, rpp = kPoolThreads / lpr;
-  const int r_in = tid / lpr, c16 = (tid % lpr) * 16;
-  const uint8_t *kin = tab.k[layer] + (size_t)local * g.T * rb;
-  const uint8_t *vin = tab.v[layer] + (size_t)local * g.T * rb;
-  uint8_t *kout = tab.k_out[layer] + ((size_t)local * tab.cap[layer] + first) * rb;
-  uint8_t *vout = tab.v_out[layer] + ((size_t)local * tab.cap[layer] + first) * rb;
-  for (int r0 = 0; r0 < rows; r0 += 4 * rpp) {
-    uint4 xk[4], xv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = r0 + u * rpp + r_in;
-      if (r < rows) {
-        const long long t = guard(list[r], 1, g.T, tab.status);
-        xk[u] = __ldcs(reinterpret_cast<const uint4 *>(kin + t * rb + c16));
-        xv[u] = __ldcs(reinterpret_cast<const uint4 *>(vin + t * rb + c16));
+  if (tab.gather) {
+    // row_bytes / 16 consecutive threads copy one row 16 bytes each, four rows a
+    // thread in flight
+    const int rb = tab.row_bytes, lpr = rb >> 4, rpp = kPoolThreads / lpr;
+    const int r_in = tid / lpr, c16 = (tid % lpr) * 16;
+    const uint8_t *kin = tab.k[layer] + (size_t)local * g.T * rb;
+    const uint8_t *vin = tab.v[layer] + (size_t)local * g.T * rb;
+    uint8_t *kout = tab.k_out[layer] + ((size_t)local * tab.cap[layer] + first) * rb;
+    uint8_t *vout = tab.v_out[layer] + ((size_t)local * tab.cap[layer] + first) * rb;
+    for (int r0 = 0; r0 < rows; r0 += 4 * rpp) {
+      uint4 xk[4], xv[4];
+  #pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + u * rpp + r_in;
+        if (r < rows) {
+          const long long t = guard(list[r], 1, g.T, tab.status);
+          xk[u] = __ldcs(reinterpret_cast<const uint4 *>(kin + t * rb + c16));
+          xv[u] = __ldcs(reinterpret_cast<const uint4 *>(vin + t * rb + c16));
+        }
       }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = r0 + u * rpp + r_in;
-      if (r < rows) {
-        *reinterpret_cast<uint4 *>(kout + (size_t)r * rb + c16) = xk[u];
-        *reinterpret_cast<uint4 *>(vout + (size_t)r * rb + c16) = xv[u];
+  #pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + u * rpp + r_in;
+        if (r < rows) {
+          *reinterpret_cast<uint4 *>(kout + (size_t)r * rb + c16) = xk[u];
+          *reinterpret_cast<uint4 *>(vout + (size_t)r * rb + c16) = xv[u];
+        }
       }
     }
   }
@@ -964,6 +967,30 @@ void pool_shape(int P, int n_units, int *kpt, int *n_cta) {
   *n_cta = ctas(*kpt);
 }
 
+// Whether the rows are copied by the gather kernel instead of the CTAs that
+// selected them: where few CTAs would copy many rows each. A CTA copies about 64
+// GB/s, and the launch costs 4 us, which pay at 256 KB of keys and values a CTA
+// while few CTAs run; the more CTAs, the nearer they are to HBM's rate by
+// themselves (where every token is kept a CTA does nothing else, and the line lies
+// lower). Measured, rows copied by the selecting CTAs / by the gather kernel
+// (bf16, d 128): 1 CTA of 256 KB 12.4 / 12.7 us, of 512 KB 18.0 / 13.7; 32 of 512
+// KB 18.4 / 13.1 to 20.3 / 17.5; 64 of 512 KB 25.9 / 26.0, of 1 MB 39.9 / 36.7; 128
+// of 1 MB 59.4 / 63.0, of 1.5 MB 144 / 102; 256 of 1 MB 98 / 101, of 2 MB 184 / 177;
+// one unit of 100000 tokens, all kept, 176 / 25, 32 of 8192, all kept, 59.6 / 49.4.
+bool gather_apart(const LayerGeom &g, int n_layers, const int *n_keep, int kpt,
+                  int n_cta) {
+  const int row_bytes = g.D * (g.dtype == RIPPLE_F32 ? 4 : 2);
+  int most = 0;
+  for (int l = 0; l < n_layers; ++l) most = n_keep[l] > most ? n_keep[l] : most;
+  const long long ctas = (long long)g.units * n_layers * n_cta;
+  // of the rows of a unit, the share of a CTA that is full of tokens
+  const int tokens = kPoolThreads * kpt < g.P ? kPoolThreads * kpt : g.P;
+  const long long bytes = g.P > 0 ? 2LL * row_bytes * most * tokens / g.P : 0;
+  const long long most_kb = most == g.T ? 960 : 1536;
+  const long long line_kb = 256 + 8 * ctas < most_kb ? 256 + 8 * ctas : most_kb;
+  return bytes >= line_kb * 1024;
+}
+
 template <int KPT>
 cudaError_t launch_pool(const LayerGeom &g, int n_units, const float *votes, const SelTable &tab,
                         int n_cta, cudaStream_t st) {
@@ -996,6 +1023,7 @@ cudaError_t launch_select(const LayerGeom &g, int n_layers, const float *votes,
                           int32_t *status, cudaStream_t st, const GatherArgs &gather) {
   if (n_layers < 1 || n_layers > kCompressMaxLayers) return cudaErrorInvalidValue;
   const int n_units = g.units * n_layers;
+  cudaError_t e;
   if (g.P <= kPoolMaxP) {
     SelTable tab;
     tab.upl = g.units;
@@ -1012,12 +1040,14 @@ cudaError_t launch_select(const LayerGeom &g, int n_layers, const float *votes,
     }
     int kpt, n_cta;
     pool_shape(g.P, n_units, &kpt, &n_cta);
-    return kpt == 8    ? launch_pool<8>(g, n_units, votes, tab, n_cta, st)
-           : kpt == 16 ? launch_pool<16>(g, n_units, votes, tab, n_cta, st)
-                       : launch_pool<32>(g, n_units, votes, tab, n_cta, st);
+    tab.gather = !gather_apart(g, n_layers, n_keep, kpt, n_cta);
+    e = kpt == 8    ? launch_pool<8>(g, n_units, votes, tab, n_cta, st)
+        : kpt == 16 ? launch_pool<16>(g, n_units, votes, tab, n_cta, st)
+                    : launch_pool<32>(g, n_units, votes, tab, n_cta, st);
+    if (tab.gather) return e;
+  } else {
+    e = select_long(g, n_layers, votes, ws, n_keep, idx, status, st);
   }
-  // Longer prefixes: selection, then the gather of all layers.
-  cudaError_t e = select_long(g, n_layers, votes, ws, n_keep, idx, status, st);
   if (e != cudaSuccess) return e;
   return launch_gather(g, n_layers, gather.k, gather.v, (const int32_t *const *)idx, n_keep,
                        gather.k_out, gather.v_out, gather.cap, status, st);

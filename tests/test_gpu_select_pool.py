@@ -10,6 +10,7 @@ import torch
 
 from oracle import ripple_oracle as O
 from paper_2608_08684_gb300 import synth
+from tests import gpu_common as C
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -98,3 +99,34 @@ def test_threshold_bucket(lib, n, base, step):
     for u in range(2):  # the threshold at the first, a middle and the last of them
         for k in {keep[u] + 1, keep[u] + (n + 1) // 2, keep[u] + n}:
             _run(lib, torch.from_numpy(x), 8 + k, 8, "none", 1, range(2))
+
+
+# many rows a CTA: copied by the gather kernel; around the line between the two
+@pytest.mark.parametrize("units,P,keep", [
+    (1, 3000, 1031), (1, 3000, 1032), (1, 3000, 2999), (2, 9000, 8000), (1, 131072, 131071),
+    (8, 20000, 12000), (3, 70000, 60000), (1, 50000, 50000), (2, 9000, 9000), (8, 700, 700)])
+def test_rows_copied_apart(lib, units, P, keep):
+    votes = synth.synthetic_votes(1100 + P, units, P, 100)
+    _run(lib, votes, 8 + keep, 8, "max", 7, range(units))
+
+
+def test_layers_of_different_size_copied_apart(lib):
+    wl = synth.WORKLOADS["tiny"].replace(n_layers=4, batch=1, n_q_heads=4, n_kv_heads=2,
+                                         head_dim=64, seq_len=6000, dtype="bf16", seed=88)
+    budgets = [6000, 32, 5000, 700]  # every token, the window only, most, some
+    ins = [tuple(t.to(DEV) for t in C.layer_inputs(wl, l, "cpu")) for l in range(4)]
+    refs = [C.run_compress(lib, wl, budgets[l], *ins[l], cap_extra=1) for l in range(4)]
+    desc = lib.layer_desc(1, 4, 2, 64, 6000, wl.window, wl.pool_kernel, "max", torch.bfloat16)
+    k_out = [torch.zeros_like(r["k_out"]) for r in refs]
+    v_out = [torch.zeros_like(r["v_out"]) for r in refs]
+    idx = [torch.full((2 * r["n"],), -1, dtype=torch.int32, device=DEV) for r in refs]
+    tables = lib.CompressTables([x[0] for x in ins], [x[1] for x in ins], [x[2] for x in ins],
+                                k_out, v_out, idx)
+    ws = torch.empty(lib.ripple_compress_layers_workspace_bytes(desc, 4), dtype=torch.uint8,
+                     device=DEV)
+    lib.ripple_compress_layers(desc, budgets, tables, ws)
+    torch.cuda.synchronize()
+    for l, r in enumerate(refs):
+        assert torch.equal(idx[l], r["idx"].reshape(-1)), l
+        assert torch.equal(k_out[l], r["k_out"]) and torch.equal(v_out[l], r["v_out"]), l
+        C.check_compress_unit(wl, r, *ins[l], 0, 1, budgets[l])
