@@ -514,19 +514,18 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kCThreads)
 // Prefixes of up to kPoolMaxP tokens: pooling, selection and gather in one
 // launch, a cluster of C CTAs (1 to 8) per unit.
 //
-// CTA r of a unit takes kPoolThreads * KPT consecutive tokens, warp w of it KPT
-// rows of 32 consecutive tokens, one token of a row per lane, so that votes
-// are loaded coalesced straight into registers (a row more at either end is
-// the pooling halo) and a neighbour d tokens away is one select and one
-// shuffle. The K-th largest key is found by one radix round over all keys
-// (2048 bins of a 32nd of a binade; only the first of a warp's run of equal
-// digits, which pooling makes, adds to the histogram); the keys of its bucket,
-// if at most kPoolCand, are then copied to every CTA of the unit, which
-// finishes on them alone, without the cluster: up to kPoolRank of them by
-// counting, more by two rounds of 9 bits. Larger buckets (many equal votes)
-// take further rounds over all keys. Kept tokens go to a list in shared memory,
-// from which the positions are written and the rows gathered (or the gather kernel
-// copies them, gather_apart).
+// CTA r of a unit takes KPT consecutive tokens a thread, warp w of it KPT rows of
+// 32 consecutive tokens, one token of a row per lane, so that votes are loaded
+// coalesced straight into registers (a row more at either end is the pooling
+// halo) and a neighbour d tokens away is one select and one shuffle. The K-th
+// largest key is found by one radix round over all keys (2048 bins of a 32nd of a
+// binade; only the first of a warp's run of equal digits, which pooling makes,
+// adds to the histogram); the keys of its bucket, if at most kPoolCand, are then
+// copied to every CTA of the unit, which finishes on them alone, without the
+// cluster: up to kPoolRank of them by counting, more by two rounds of 9 bits.
+// Larger buckets (many equal votes) take further rounds over all keys. Kept
+// tokens go to a list in shared memory, from which the positions are written and
+// the rows gathered (or the gather kernel copies them, gather_apart).
 //
 // Bound: latency (barriers, votes from L2) for few units, HBM of the gather for
 // many. One layer of 32 units, 32736 tokens, 1024 kept, takes 16.7 us
@@ -535,7 +534,6 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kCThreads)
 // reading all the histograms, and a gather kernel took 41 us, and 256 units of
 // 5991 tokens 98 us against 35.
 constexpr int kPoolThreads = 512;
-constexpr int kPoolWarps = kPoolThreads / 32;
 constexpr int kPoolMaxCta = 8;                       // CTAs per unit, at most
 constexpr int kPoolMaxP = kPoolMaxCta * kPoolThreads * 32;
 constexpr int kPoolCand = 2048;
@@ -548,8 +546,8 @@ struct PoolSmem {
   uint32_t all[kPoolCand];      // the unit's bucket keys
   int n_cand;                   // this CTA's
   alignas(8) int cnt[2];        // this CTA's kept keys: above tau, equal to tau; read as a pair
-  int wsum[2][kPoolWarps];
-  int wgt[kPoolWarps], weq[kPoolWarps];
+  int wsum[2][32];
+  int wgt[32], weq[32];
   int digit[2][3];              // per round parity: digit, remaining, bucket keys
   uint32_t tau[2];              // the threshold of a small bucket and its keys kept
 };
@@ -557,12 +555,36 @@ static_assert(offsetof(PoolSmem, cnt) % 8 == 0 && offsetof(PoolSmem, hist) % 16 
                   sizeof(PoolSmem) % 16 == 0,
               "vector reads of shared memory");
 
-// The digit of the K-th largest (`remaining`-th) key from 2048 bin counts, four
-// per thread in descending order (c[q]: bin 2047 - 4 tid - q). Two barriers.
-__device__ __forceinline__ void find_digit(const int (&c)[4], int &remaining, int par,
+// kCols bins of a histogram downwards from `top`, in CTA r of the cluster.
+template <int kCols>
+__device__ __forceinline__ void load_bins(const uint32_t *top, uint32_t r, int n_cta,
+                                          int (&c)[kCols]) {
+  const uint32_t *p = top - (kCols - 1);
+  if constexpr (kCols == 4) {
+    const uint4 h = n_cta > 1 ? ld_cluster_v4(cluster_addr(p, r))
+                              : *reinterpret_cast<const uint4 *>(p);
+    c[0] = (int)h.w;
+    c[1] = (int)h.z;
+    c[2] = (int)h.y;
+    c[3] = (int)h.x;
+  } else {
+    static_assert(kCols == 2, "bins per thread");
+    const uint2 h = n_cta > 1 ? ld_cluster_v2(cluster_addr(p, r))
+                              : *reinterpret_cast<const uint2 *>(p);
+    c[0] = (int)h.y;
+    c[1] = (int)h.x;
+  }
+}
+
+// The digit of the K-th largest (`remaining`-th) key from 2048 bin counts, kCols
+// per thread in descending order (c[q]: bin 2047 - kCols tid - q). Two barriers.
+template <int kCols>
+__device__ __forceinline__ void find_digit(const int (&c)[kCols], int &remaining, int par,
                                            PoolSmem &s, int &digit, int &bucket) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int sum = c[0] + c[1] + c[2] + c[3];
+  int sum = 0;
+#pragma unroll
+  for (int q = 0; q < kCols; ++q) sum += c[q];
   int incl = sum;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -576,9 +598,9 @@ __device__ __forceinline__ void find_digit(const int (&c)[4], int &remaining, in
   for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
   int above = before + incl - sum;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < kCols; ++q) {
     if (above < remaining && remaining <= above + c[q]) {
-      s.digit[par][0] = kBins - 1 - 4 * tid - q;
+      s.digit[par][0] = kBins - 1 - kCols * tid - q;
       s.digit[par][1] = remaining - above;
       s.digit[par][2] = c[q];
     }
@@ -599,14 +621,15 @@ __device__ __forceinline__ float behind(float prev, float cur, int d, int lane) 
   return __shfl_sync(0xffffffffu, lane >= 32 - d ? prev : cur, lane - d);
 }
 
-template <int KPT>
-__global__ void __launch_bounds__(kPoolThreads, 2)
+template <int KPT, int kThr>
+__global__ void __launch_bounds__(kThr, 1024 / kThr)
     select_pool_kernel(LayerGeom g, const float *votes, const __grid_constant__ SelTable tab,
                        int n_cta) {
   extern __shared__ __align__(16) uint8_t pool_sm[];
   PoolSmem &s = *reinterpret_cast<PoolSmem *>(pool_sm);
   int *list = reinterpret_cast<int *>(pool_sm + sizeof(PoolSmem));  // kept tokens of this CTA
-  constexpr int kCtaTokens = kPoolThreads * KPT;
+  constexpr int kCols = kBins / kThr;  // histogram bins of a thread
+  constexpr int kCtaTokens = kThr * KPT;
   const int rank = n_cta > 1 ? (int)cluster_rank() : 0;
   const int unit = blockIdx.x / n_cta;  // over all layers of the launch
   const int layer = unit / tab.upl;
@@ -622,7 +645,7 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
     if (K > 0) {
       first = min(t0, P);
       kept = min(P, t0 + kCtaTokens) - first;
-      for (int i = tid; i < kept; i += kPoolThreads) list[i] = first + i;
+      for (int i = tid; i < kept; i += kThr) list[i] = first + i;
     }
   } else {
     // ---------------- pooled keys
@@ -635,7 +658,7 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
       const int j = w0 + (i - 1) * 32 + lane;
       x[i] = j >= 0 && j < P ? __ldcg(v + j) : fill;
     }
-    for (int i = tid; i < kBins; i += kPoolThreads) s.hist[0][i] = 0;
+    for (int i = tid; i < kBins; i += kThr) s.hist[0][i] = 0;
     const int half = g.pool_kernel / 2;
     if (g.pool_type == RIPPLE_POOL_MAX && half > 0) {
       // x[j] = max of the width tokens from j on, width the largest power of
@@ -703,23 +726,21 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
           atomicAdd(&hist[d], (uint32_t)(later ? __ffs(later) : 32 - lane));
         }
       }
-      const int d0 = kBins - 1 - 4 * tid;  // this thread's bins d0 .. d0 - 3
-      int c[4] = {0, 0, 0, 0};
+      const int d0 = kBins - 1 - kCols * tid;  // this thread's bins, down from d0
+      int c[kCols] = {};
       if (n_cta > 1)
         cluster_sync_all();  // every CTA's histogram of this round is complete
       else
         __syncthreads();
       for (int r = 0; r < n_cta; ++r) {
-        const uint4 h = n_cta > 1 ? ld_cluster_v4(cluster_addr(hist + d0 - 3, r))
-                                  : *reinterpret_cast<const uint4 *>(hist + d0 - 3);
-        c[0] += (int)h.w;
-        c[1] += (int)h.z;
-        c[2] += (int)h.y;
-        c[3] += (int)h.x;
+        int h[kCols];
+        load_bins(hist + d0, r, n_cta, h);
+#pragma unroll
+        for (int q = 0; q < kCols; ++q) c[q] += h[q];
       }
       // the other histogram, for the next round (its readers have passed this
       // round's barrier)
-      for (int i = tid; i < kBins; i += kPoolThreads) s.hist[(it & 1) ^ 1][i] = 0;
+      for (int i = tid; i < kBins; i += kThr) s.hist[(it & 1) ^ 1][i] = 0;
       if (tid == 0) s.n_cand = 0;
       int digit, bucket;
       find_digit(c, remaining, it & 1, s, digit, bucket);
@@ -754,7 +775,7 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
         int off = 0;
         for (int r = 0; r < n_cta; ++r) {
           const int n = (int)ld_cluster_u32(cluster_addr(&s.n_cand, r));
-          for (int i = tid; i < n; i += kPoolThreads)
+          for (int i = tid; i < n; i += kThr)
             s.all[off + i] = ld_cluster_u32(cluster_addr(&s.cand[i], r));
           off += n;
         }
@@ -787,14 +808,14 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
         uint32_t *h2 = s.hist[it & 1];
         const int sh = shift_of(level);
         const uint32_t dm = dmask_of(level);
-        for (int i = tid; i < bucket; i += kPoolThreads) {
+        for (int i = tid; i < bucket; i += kThr) {
           const uint32_t u = all[i];
           if ((u & mask) == prefix) atomicAdd(&h2[u >> sh & dm], 1u);
         }
         __syncthreads();
-        const uint4 h = *reinterpret_cast<const uint4 *>(h2 + d0 - 3);
-        const int cc[4] = {(int)h.w, (int)h.z, (int)h.y, (int)h.x};
-        for (int i = tid; i < kBins; i += kPoolThreads) s.hist[(it & 1) ^ 1][i] = 0;
+        int cc[kCols];
+        load_bins(h2 + d0, 0, 1, cc);
+        for (int i = tid; i < kBins; i += kThr) s.hist[(it & 1) ^ 1][i] = 0;
         int n_eq;
         find_digit(cc, remaining, it & 1, s, digit, n_eq);
         prefix |= (uint32_t)digit << sh;
@@ -816,7 +837,7 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
       s.weq[wid] = ceq;
     }
     __syncthreads();
-    int gt = lane < kPoolWarps ? s.wgt[lane] : 0, eq = lane < kPoolWarps ? s.weq[lane] : 0;
+    int gt = lane < kThr / 32 ? s.wgt[lane] : 0, eq = lane < kThr / 32 ? s.weq[lane] : 0;
     int gt_w = lane < wid ? gt : 0, eq_w = lane < wid ? eq : 0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -862,17 +883,17 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
   const int window = rank == n_cta - 1 ? g.W : 0;
   if (window > 0) {
     if (kept == 0) first = max(K, 0);
-    for (int i = tid; i < window; i += kPoolThreads) list[kept + i] = P + i;
+    for (int i = tid; i < window; i += kThr) list[kept + i] = P + i;
   }
   const int rows = kept + window;
   __syncthreads();
   const int local = unit % tab.upl;
   int32_t *out = tab.idx[layer] + (size_t)local * n_keep + first;
-  for (int i = tid; i < rows; i += kPoolThreads) out[i] = list[i];
+  for (int i = tid; i < rows; i += kThr) out[i] = list[i];
   if (tab.gather) {
     // row_bytes / 16 consecutive threads copy one row 16 bytes each, four rows a
     // thread in flight
-    const int rb = tab.row_bytes, lpr = rb >> 4, rpp = kPoolThreads / lpr;
+    const int rb = tab.row_bytes, lpr = rb >> 4, rpp = kThr / lpr;
     const int r_in = tid / lpr, c16 = (tid % lpr) * 16;
     const uint8_t *kin = tab.k[layer] + (size_t)local * g.T * rb;
     const uint8_t *vin = tab.v[layer] + (size_t)local * g.T * rb;
@@ -942,29 +963,58 @@ cudaError_t select_long(const LayerGeom &g, int n_layers, const float *votes, co
   return cudaSuccess;
 }
 
-// Keys per thread (8, 16 or 32; 512 threads a CTA) and CTAs per unit: 16, or
-// 8 where they fill the CTA (P <= 4096) or where 16 leave three quarters of
-// the SMs idle, or 32 where there are CTAs for many waves, which saves cluster
-// barriers. Measured with 8 / 16 / 32 keys: one layer of 32 units and 32736
-// tokens 21.6 / 16.6 / 23.6 us, 8 units of 8160 tokens (with scoring) 37.1 /
-// 40.0 / 47.0 us, 1024 units of 32736 tokens (with scoring) 2754 / 2573 / 2539
-// us, and, before the first round's finer bins, 256 units of 5991 tokens (with
-// scoring) 143 / 136 / 166 us.
-void pool_shape(int P, int n_units, int *kpt, int *n_cta) {
+// The CTAs of a unit: `threads` threads of `keys` keys each.
+struct PoolShape {
+  int keys, threads, n_cta;
+};
+
+// Shapes of the selecting CTAs. While 16 keys a thread make at most one wave of
+// two CTAs per SM: 16, or 8 where they fill the CTA (P <= 4096) or where 16 leave
+// three quarters of the SMs idle (one layer of 32 units and 32736 tokens, 8 / 16 /
+// 32 keys: 21.6 / 16.6 / 23.6 us; 8 units of 8160 tokens, with scoring, 37.1 / 40.0 /
+// 47.0). With more CTAs than that the waves count, and 32 keys a thread, in CTAs
+// of 512 threads or one of 1024, make fewer of them; where many rows are kept,
+// though, their copies count, which more and smaller CTAs overlap better. Keys
+// and values a unit keeps, us with 16 x 512 / 32 x 512 / 32 x 1024 (one layer, bf16,
+// d 128 or 64):
+//   8968 tokens, 256 units    128 KB 35 / 27 / 46, 256 KB 43 / 37 / 60, 512 KB 65 / 69 / 87
+//   16968 tokens, 256 units    64 KB 46 / 46 / 42, 256 KB 57 / 64 / 58, 512 KB 77 / 99 / 88
+//   16968 tokens, 1024 units   64 KB 159 / 162 / 147, 256 KB 204 / 228 / 209
+//   23968 tokens, 256 units   128 KB 50 / 50 / 47, 256 KB 58 / 64 / 62, 512 KB 77 / 92 / 88
+//   32736 tokens, 128 units   256 KB 40 / 32 / 30, 512 KB 49 / 42 / 42
+//   32736 tokens, 256 units   128 KB 60 / 50 / 49, 256 KB 70 / 70 / 68, 512 KB 85 / 91 / 90
+//   32736 tokens, 1024 units (with scoring) 750 KB 2540 / 2491 / 2512
+// Beyond 32768 tokens 32 x 512 is left; beyond 65536, where 16 x 512 are more than 8
+// CTAs, 16 x 1024 while all units' clusters are resident, one CTA an SM: 4 units of
+// 80000 tokens, 20000 kept, 19 us against 29 with 32 x 512 (16 units of 100000,
+// whose 7-CTA clusters no longer fit at once, 34 against 28).
+PoolShape pool_shape(const LayerGeom &g, int n_layers, const int *n_keep) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  auto ctas = [&](int keys) {
-    int n = 1;
-    while (n * kPoolThreads * keys < P) n *= 2;
-    return n;
+  const int P = g.P;
+  auto ctas = [&](int tokens) { return P > tokens ? (P + tokens - 1) / tokens : 1; };
+  auto shape = [&](int keys, int threads) {
+    return PoolShape{keys, threads, ctas(keys * threads)};
   };
-  const long long at16 = (long long)n_units * ctas(16);
-  if (P <= kPoolThreads * 8 || (ctas(8) <= kPoolMaxCta && at16 * 4 <= sms))
-    *kpt = 8;
-  else
-    *kpt = ctas(16) > kPoolMaxCta || (P > kPoolThreads * 16 && at16 >= 8LL * sms) ? 32 : 16;
-  *n_cta = ctas(*kpt);
+  const long long units = (long long)g.units * n_layers;
+  const int c16 = ctas(16 * kPoolThreads);
+  if (P <= 8 * kPoolThreads ||
+      (ctas(8 * kPoolThreads) <= kPoolMaxCta && units * c16 * 4 <= sms))
+    return shape(8, kPoolThreads);
+  if (c16 > kPoolMaxCta)
+    return units * ctas(32 * kPoolThreads) * 3 <= 2LL * sms ? shape(16, 2 * kPoolThreads)
+                                                            : shape(32, kPoolThreads);
+  if (P <= 16 * kPoolThreads || units * c16 <= 2LL * sms) return shape(16, kPoolThreads);
+  long long rows = 0;
+  for (int l = 0; l < n_layers; ++l) rows += n_keep[l];
+  const long long kb =  // keys and values a unit keeps, on average
+      rows * 2 * g.D * (g.dtype == RIPPLE_F32 ? 4 : 2) / n_layers >> 10;
+  if (P > 64 * kPoolThreads) return shape(32, kPoolThreads);
+  if (P <= 32 * kPoolThreads) return shape(kb < 384 ? 32 : 16, kPoolThreads);
+  if (kb < 256 || (units <= sms && P > 48 * kPoolThreads && kb < 2048))
+    return shape(32, 2 * kPoolThreads);
+  return shape(P > 48 * kPoolThreads && (kb < 512 || units >= 512) ? 32 : 16, kPoolThreads);
 }
 
 // Whether the rows are copied by the gather kernel instead of the CTAs that
@@ -977,30 +1027,29 @@ void pool_shape(int P, int n_units, int *kpt, int *n_cta) {
 // KB 18.4 / 13.1 to 20.3 / 17.5; 64 of 512 KB 25.9 / 26.0, of 1 MB 39.9 / 36.7; 128
 // of 1 MB 59.4 / 63.0, of 1.5 MB 144 / 102; 256 of 1 MB 98 / 101, of 2 MB 184 / 177;
 // one unit of 100000 tokens, all kept, 176 / 25, 32 of 8192, all kept, 59.6 / 49.4.
-bool gather_apart(const LayerGeom &g, int n_layers, const int *n_keep, int kpt,
-                  int n_cta) {
+bool gather_apart(const LayerGeom &g, int n_layers, const int *n_keep, const PoolShape &sh) {
   const int row_bytes = g.D * (g.dtype == RIPPLE_F32 ? 4 : 2);
   int most = 0;
   for (int l = 0; l < n_layers; ++l) most = n_keep[l] > most ? n_keep[l] : most;
-  const long long ctas = (long long)g.units * n_layers * n_cta;
+  const long long ctas = (long long)g.units * n_layers * sh.n_cta;
   // of the rows of a unit, the share of a CTA that is full of tokens
-  const int tokens = kPoolThreads * kpt < g.P ? kPoolThreads * kpt : g.P;
+  const int tokens = sh.keys * sh.threads < g.P ? sh.keys * sh.threads : g.P;
   const long long bytes = g.P > 0 ? 2LL * row_bytes * most * tokens / g.P : 0;
   const long long most_kb = most == g.T ? 960 : 1536;
   const long long line_kb = 256 + 8 * ctas < most_kb ? 256 + 8 * ctas : most_kb;
   return bytes >= line_kb * 1024;
 }
 
-template <int KPT>
+template <int KPT, int kThr>
 cudaError_t launch_pool(const LayerGeom &g, int n_units, const float *votes, const SelTable &tab,
                         int n_cta, cudaStream_t st) {
-  const size_t smem = sizeof(PoolSmem) + sizeof(int) * (kPoolThreads * KPT + 64);
-  cudaError_t e = cudaFuncSetAttribute(select_pool_kernel<KPT>,
+  const size_t smem = sizeof(PoolSmem) + sizeof(int) * (kThr * KPT + 64);
+  cudaError_t e = cudaFuncSetAttribute(select_pool_kernel<KPT, kThr>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_units * n_cta);
-  cfg.blockDim = dim3(kPoolThreads);
+  cfg.blockDim = dim3(kThr);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -1011,7 +1060,7 @@ cudaError_t launch_pool(const LayerGeom &g, int n_units, const float *votes, con
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, select_pool_kernel<KPT>, g, votes, tab, n_cta);
+  e = cudaLaunchKernelEx(&cfg, select_pool_kernel<KPT, kThr>, g, votes, tab, n_cta);
   count_launches(1);
   return e;
 }
@@ -1038,12 +1087,15 @@ cudaError_t launch_select(const LayerGeom &g, int n_layers, const float *votes,
       tab.v_out[l] = (uint8_t *)gather.v_out[l];
       tab.cap[l] = gather.cap[l];
     }
-    int kpt, n_cta;
-    pool_shape(g.P, n_units, &kpt, &n_cta);
-    tab.gather = !gather_apart(g, n_layers, n_keep, kpt, n_cta);
-    e = kpt == 8    ? launch_pool<8>(g, n_units, votes, tab, n_cta, st)
-        : kpt == 16 ? launch_pool<16>(g, n_units, votes, tab, n_cta, st)
-                    : launch_pool<32>(g, n_units, votes, tab, n_cta, st);
+    const PoolShape sh = pool_shape(g, n_layers, n_keep);
+    tab.gather = !gather_apart(g, n_layers, n_keep, sh);
+    e = sh.keys == 8    ? launch_pool<8, kPoolThreads>(g, n_units, votes, tab, sh.n_cta, st)
+        : sh.keys == 16 && sh.threads == kPoolThreads
+            ? launch_pool<16, kPoolThreads>(g, n_units, votes, tab, sh.n_cta, st)
+        : sh.keys == 16 ? launch_pool<16, 2 * kPoolThreads>(g, n_units, votes, tab, sh.n_cta, st)
+        : sh.threads == kPoolThreads
+            ? launch_pool<32, kPoolThreads>(g, n_units, votes, tab, sh.n_cta, st)
+            : launch_pool<32, 2 * kPoolThreads>(g, n_units, votes, tab, sh.n_cta, st);
     if (tab.gather) return e;
   } else {
     e = select_long(g, n_layers, votes, ws, n_keep, idx, status, st);

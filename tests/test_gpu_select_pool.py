@@ -101,6 +101,18 @@ def test_threshold_bucket(lib, n, base, step):
             _run(lib, torch.from_numpy(x), 8 + k, 8, "none", 1, range(2))
 
 
+# one 1024-thread CTA a unit; three, five, six and seven CTAs a unit, the last of
+# them nearly empty or full; one wave of CTAs and more
+@pytest.mark.parametrize("units,P,keep", [
+    (160, 16385, 40), (160, 24576, 700), (200, 24577, 30), (153, 32768, 90), (100, 32767, 5000),
+    (3, 24576, 100), (40, 40000, 50), (3, 50000, 77), (20, 61440, 3000), (3, 70000, 100),
+    (2, 98304, 100), (2, 98305, 100), (3, 114688, 2000), (320, 9000, 300), (320, 9000, 4000),
+    (260, 20000, 5000), (300, 32768, 600)])
+def test_cta_shapes(lib, units, P, keep):
+    votes = synth.synthetic_votes(1000 + P, units, P, 100)
+    _run(lib, votes, 8 + keep, 8, "max", 7, [0, units // 2, units - 1])
+
+
 # many rows a CTA: copied by the gather kernel; around the line between the two
 @pytest.mark.parametrize("units,P,keep", [
     (1, 3000, 1031), (1, 3000, 1032), (1, 3000, 2999), (2, 9000, 8000), (1, 131072, 131071),
