@@ -65,8 +65,8 @@ constexpr int kPubSlots = 2;
 //   1024 tiles, 16 such layers             3546 / 2188 / 2024 / 2011
 // Smaller items gain a single layer and cost many layers, which decide from 65
 // tiles on.
-// Prompts of more than 1024 tiles take up to an item per 64 tiles where those fill
-// the SMs better in a layer's units (items_per_unit).
+// Prompts of more than 256 tiles can take other numbers where those fill the SMs
+// better in a layer's units (items_per_unit).
 constexpr int kTilesPerItem = 16, kTilesPerItemShort = 8;
 constexpr int kShortTiles = 64;
 constexpr int kMaxItems = 16;
@@ -670,23 +670,26 @@ int sm_count() {
 }
 
 // Items a unit of n_tiles key tiles is cut into, in layers of `units` units: see
-// kTilesPerItem. Between 16 and an item per 64 tiles the number with the least
-// modelled time is taken, the layer's waves of items times an item's tiles (more
-// items by 2% or not): one unit of 4096 tiles 1049 us in 64 items, 1461 in 16; 4
-// units of 1563 tiles 217 us in 25, 281 in 16; 8 of 4096 tiles 1348 us in 19, 1430
-// in 16, 1524 in 64; 16 of 1172 tiles 352 us in 19, 400 in 16. No more items than
-// SMs (the schedule is free of deadlock up to twice as many).
+// kTilesPerItem. Of more than 256 tiles 16, or another number from an item per 64
+// tiles on that takes less modelled time, the layer's waves of items times an
+// item's tiles (4% less, or 12% for fewer items, as the waves of many layers even
+// out): one unit of 4096 tiles 1049 us in 64 items, 1461
+// in 16; 4 units of 1563 tiles 217 us in 25, 281 in 16; 8 of 4096 tiles 1348 us in
+// 19, 1430 in 16, 1524 in 64; 16 of 1172 tiles 352 us in 19, 400 in 16; 32 of 547
+// tiles 314 us in 9, 360 in 16. No more items than SMs (the schedule is free of
+// deadlock up to twice as many).
 int items_per_unit(int n_tiles, int units, int sms) {
   const int per = n_tiles <= kShortTiles ? kTilesPerItemShort : kTilesPerItem;
   const int items = (n_tiles + per - 1) / per;
   if (items <= kMaxItems) return std::min(items, sms);
-  const int most = std::min((n_tiles + kTilesPerItemLong - 1) / kTilesPerItemLong, sms);
+  const int per_long = (n_tiles + kTilesPerItemLong - 1) / kTilesPerItemLong;
+  const int most = std::min(std::max(per_long, kMaxItems), sms);
   int best = std::min(kMaxItems, sms);
   auto cost = [&](int n) {
     return ((long long)units * n + sms - 1) / sms * ((n_tiles + n - 1) / n);
   };
-  for (int n = best + 1; n <= most; ++n)
-    if (cost(n) * 50 < cost(best) * 49) best = n;
+  for (int n = std::min(per_long, best); n <= most; ++n)
+    if (cost(n) * 100 < cost(best) * (n < kMaxItems && best == kMaxItems ? 88 : 96)) best = n;
   return best;
 }
 
