@@ -85,7 +85,7 @@ constexpr int kMiscBytes = 4096;              // barriers, work list, merge stat
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxComb = 16;                  // partials of a group combined at a time, at most
 constexpr int kPlanPerLane = RIPPLE_MAX_LAYERS / 32;  // layers per lane of the work list
-constexpr long long kSuspendCycles = 1000000;  // wait bounds from here on suspend
+constexpr uint32_t kSuspendNs = 1000000;      // of a poll of an mbarrier, at most
 
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
 constexpr int cmin(int a, int b) { return a < b ? a : b; }
@@ -210,17 +210,30 @@ __device__ __forceinline__ ItemInfo item_info(const DecParams &p, const S &s, in
   return f;
 }
 
+// Whether the phase has completed, after suspending the thread for at most about
+// `ns` nanoseconds until it does.
+__device__ __forceinline__ bool mbar_try_wait_for(uint64_t *bar, uint32_t parity, uint32_t ns) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n"
+      " mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait on an mbarrier phase. Gives up when another role of the CTA
 // has given up, or after p.wait_cycles (then raises the CTA's abort flag and
-// reports RIPPLE_ETIMEOUT). A try_wait may suspend the thread until the phase
-// completes, past a short bound, so short bounds poll instead.
+// reports RIPPLE_ETIMEOUT). A poll suspends the thread for p.suspend_ns at most,
+// which is within the bound, so that short bounds are kept by the same path.
 __device__ __forceinline__ bool wait_bar(uint64_t *bar, uint32_t parity, int *abort_flag,
                                          const DecParams &p) {
-  const bool suspend = p.wait_cycles >= kSuspendCycles;
-  if (suspend && mbar_try_wait(bar, parity)) return true;
+  if (mbar_try_wait_for(bar, parity, p.suspend_ns)) return true;
   const long long t0 = clock64();
   for (;;) {
-    if (suspend ? mbar_try_wait(bar, parity) : mbar_test_wait(bar, parity)) return true;
+    if (mbar_try_wait_for(bar, parity, p.suspend_ns)) return true;
     if (*(volatile int *)abort_flag) return false;
     if (clock64() - t0 > p.wait_cycles) {
       *(volatile int *)abort_flag = 1;
@@ -1439,6 +1452,8 @@ ripple_status prepare(const ripple_decode_desc *desc, const void *q, const void 
 ripple_status run(const ripple_decode_desc *desc, DecParams &p, void *stream) {
   p.epoch = next_epoch();
   p.wait_cycles = wait_limit_cycles();
+  // a quarter of the bound's cycles, at 2 GHz half of its time
+  p.suspend_ns = (uint32_t)std::min<long long>(p.wait_cycles / 4, kSuspendNs);
   cudaStream_t st = (cudaStream_t)stream;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return RIPPLE_ECUDA;

@@ -22,6 +22,7 @@ struct DecParams {
   int epoch;        // nonzero tag of this call: the init flag's value once the
                     // counters are zeroed
   long long wait_cycles;  // bound of the in-kernel waits
+  uint32_t suspend_ns;    // of one poll of an mbarrier, at most
   int item_rows;          // cache rows per work item
   long long ws_items;     // work items the partials (ws_o, ws_ml) have room for
   int n_ctrl;             // words of the control block

@@ -6,11 +6,14 @@ its tensor memory); the call must come back within seconds with
 RIPPLE_ETIMEOUT in the device status, and the next call at the default limit
 must match the oracle again.
 
-A wait gives up only after a poll of its mbarrier has come back empty; one
-poll may suspend the thread until the phase completes or a hardware time
-limit passes, so waits on a bulk copy that lands within that limit never give
-up. The calls tested here also wait on flags other thread blocks raise (the
-decode's counter initialisation, the scoring's row statistics), which do."""
+A wait gives up only after a poll of its mbarrier has come back empty. The
+decode's polls suspend the thread for half the bound at most, whatever the
+bound is, so that these tests run the path that ships; the scoring's may suspend
+it until the phase completes or a hardware time limit passes, so that waits on a
+copy that lands within that limit never give up. The scoring waits on flags that
+other thread blocks raise (its row statistics) as well, which do. The gather
+kernel (its own copies) and the window divergence wait on mbarriers alone, in the
+second way: their giving up is not run."""
 import time
 
 import numpy as np
@@ -56,8 +59,7 @@ def test_wait_limit_setter_round_trips(lib):
 
 def test_compress_layers_times_out_then_recovers(lib):
     # two layers of the 32k workload's shape: the tensor-core scoring (waits
-    # on its TMA ring, TMEM accumulators and other blocks' row statistics) and
-    # the gather (waits on its bulk copies)
+    # on its TMA ring, TMEM accumulators and other blocks' row statistics)
     wl = synth.WORKLOADS["llama8b-32k"].replace(n_layers=2)
     L, B, H, d = wl.n_layers, wl.batch, wl.n_kv_heads, wl.head_dim
     budgets = [1500, 700]
@@ -122,9 +124,8 @@ def test_decode_times_out_then_recovers(lib):
         return status, out, kc, vc
 
     torch.cuda.synchronize()
-    # Whether a wait outlasts the bound depends on timing (an mbarrier wait is
-    # suspended in hardware and may return only when its phase completes), so
-    # the short-bound call is repeated until one of its waits gives up.
+    # Whether a wait outlasts the bound depends on timing, so the short-bound
+    # call is repeated until one of its waits gives up.
     seen = []
     for _ in range(5):
         with _ShortWaits(lib):
