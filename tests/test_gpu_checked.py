@@ -4,9 +4,11 @@ extent and would report RIPPLE_EBOUNDS in the status word instead of going
 out of bounds. It stands in for a memory checker, which is not available on
 these GPUs. Both builds are loaded side by side (a second instance of the
 binding over the checked library). On shapes that exercise every scoring path
-(tensor cores with 128 and 256 window rows, fp32 on the CUDA cores), the
-three selection kernels, the gather, split and single decode items in both
-dtypes, the no-allocation decode and the window divergence with ragged
+(tensor cores with 128 and 256 window rows and with rows padded to 32, 64, 128 and
+256, d 64 and 128, the fused outputs; fp32 on the CUDA cores), the three selection
+kernels (select_pool_kernel in its five shapes, with and without the gather),
+the gather kernel, split and single decode items in both dtypes up to 8 heads a
+group, the no-allocation decode and the window divergence with ragged
 slices and empty shares, the checked build reports no violation and its
 outputs equal the normal build's bit for bit (the guards change no
 arithmetic when an access is in bounds)."""
@@ -46,12 +48,25 @@ def chk():
 
 
 COMPRESS = [
-    # 128 window rows: tcgen05 scoring, cluster selection (few units)
+    # 128 window rows: tcgen05 scoring
     ("tc-128", dict(batch=2, n_q_heads=8, n_kv_heads=2, head_dim=128, seq_len=1000, dtype="bf16",
                     kv_dist="scaled_sinks", seed=61), [31, 200, 968, 10**6]),
     # 256 window rows: the other tcgen05 kernel
     ("tc-256", dict(batch=1, n_q_heads=16, n_kv_heads=2, head_dim=128, seq_len=700, dtype="bf16",
                     seed=62), [50, 300]),
+    # rows padded to 32, 64, 128 and 256, several items a unit, d 64 and 128
+    ("tc-24-d64", dict(batch=1, n_q_heads=6, n_kv_heads=2, head_dim=64, seq_len=3300, window=8,
+                       dtype="bf16", seed=71), [200]),
+    ("tc-33", dict(batch=1, n_q_heads=2, n_kv_heads=2, head_dim=128, seq_len=1300, window=33,
+                   dtype="bf16", seed=72), [200]),
+    ("tc-64-d64", dict(batch=1, n_q_heads=8, n_kv_heads=2, head_dim=64, seq_len=1700, window=16,
+                       dtype="bf16", seed=73), [300]),
+    ("tc-96-d64", dict(batch=1, n_q_heads=6, n_kv_heads=2, head_dim=64, seq_len=1601, window=32,
+                       dtype="bf16", seed=74), [300]),
+    ("tc-160", dict(batch=1, n_q_heads=10, n_kv_heads=2, head_dim=128, seq_len=1100, window=32,
+                    dtype="bf16", seed=75), [300]),
+    ("tc-256-d64", dict(batch=1, n_q_heads=16, n_kv_heads=2, head_dim=64, seq_len=2500,
+                        window=32, dtype="bf16", seed=76), [300]),
     # fp32, d = 64: scoring on the CUDA cores
     ("simt-f32", dict(batch=1, n_q_heads=4, n_kv_heads=2, head_dim=64, seq_len=389, dtype="f32",
                       seed=63), [10, 128]),
@@ -70,8 +85,36 @@ def test_compress_layer_checked(lib, chk, name, over, budgets):
             assert torch.equal(a[key], b[key]), (name, budget, key)
 
 
+# (units, prefix, kept): select_pool_kernel with 8, 16 and 32 keys a thread and 512
+# threads, 16 and 32 keys and 1024, the rows copied by it or by the gather kernel; the
+# cluster kernel; the kernel with its keys in the workspace
+@pytest.mark.parametrize("units,P,keep", [
+    (2, 9000, 300), (2, 9000, 9000), (40, 40000, 90), (320, 9000, 50), (22, 66000, 100),
+    (2, 70000, 300), (3, 66000, 40000), (160, 17000, 60), (2, 131073, 500), (2, 212993, 700)])
+def test_select_layer_checked(lib, chk, units, P, keep):
+    w = 8
+    votes = synth.synthetic_votes(1200 + P, units, P, 100).to(DEV)
+    g = torch.Generator(device=DEV).manual_seed(P)
+    k = torch.randn(1, units, P + w, 64, dtype=torch.bfloat16, device=DEV, generator=g)
+    runs = []
+    for m in (lib, chk):
+        desc = m.layer_desc(1, units, units, 64, P + w, w, 7, "max", torch.bfloat16)
+        n = m.ripple_keep_count(keep + w, P + w, w)
+        k_out = torch.zeros(1, units, n + 1, 64, dtype=torch.bfloat16, device=DEV)
+        v_out = torch.zeros_like(k_out)
+        idx = torch.full((units * n,), -1, dtype=torch.int32, device=DEV)
+        ws = torch.empty(m.ripple_compress_workspace_bytes(desc), dtype=torch.uint8, device=DEV)
+        status = torch.zeros(1, dtype=torch.int32, device=DEV)
+        m.ripple_select_layer(desc, keep + w, votes, k, k, k_out, v_out, idx, ws,
+                              dev_status=status)
+        torch.cuda.synchronize()
+        runs.append((int(status.item()), idx, k_out, v_out))
+    assert runs[1][0] == 0
+    assert all(torch.equal(x, y) for x, y in zip(runs[0][1:], runs[1][1:]))
+
+
 def test_compress_layers_checked(lib, chk):
-    # 32 layers x 8 units: one 1024-thread selection CTA per unit
+    # 32 layers x 8 units in one call
     wl = synth.WORKLOADS["tiny"].replace(n_layers=32, batch=1, n_q_heads=32, n_kv_heads=8,
                                          head_dim=128, seq_len=640, dtype="bf16", seed=64)
     budgets = [32 + 19 * l for l in range(wl.n_layers)]
@@ -105,6 +148,13 @@ DECODE = [
                       seed=65), [2047, 4097, 8300]),
     ("G8-f32", dict(n_layers=2, batch=2, n_q_heads=16, n_kv_heads=2, head_dim=64, dtype="f32",
                     seed=66), [0, 513]),
+    # 8 heads of 128 dims (two MMAs a block, merge buffers shared by the warps)
+    ("split-G8", dict(n_layers=2, batch=1, n_q_heads=16, n_kv_heads=2, head_dim=128, dtype="bf16",
+                      seed=69), [5000, 700]),
+    ("single-G8", dict(n_layers=3, batch=20, n_q_heads=32, n_kv_heads=4, head_dim=128,
+                       dtype="bf16", seed=70), [40, 0, 129]),
+    ("split-G2-d64", dict(n_layers=1, batch=1, n_q_heads=4, n_kv_heads=2, head_dim=64,
+                          dtype="bf16", seed=71), [3000]),
     ("G1-single-layer", dict(n_layers=1, batch=2, n_q_heads=2, n_kv_heads=2, head_dim=128,
                              dtype="bf16", seed=67), [3000]),
 ]
