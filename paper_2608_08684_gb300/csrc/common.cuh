@@ -1,5 +1,5 @@
-// Shared device helpers of libripple: element loads, warp reductions, status
-// reporting, and the inline-PTX wrappers (mbarrier, bulk async copies).
+// Shared device helpers of libripple: element loads, status reporting, and the
+// inline-PTX wrappers (mbarrier, bulk async copies).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -42,18 +42,7 @@ __device__ __forceinline__ void load8(const float *p, float (&out)[8]) {
   out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
 }
 
-// ---------------------------------------------------------------- reductions
-
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+// ---------------------------------------------------------------- arithmetic
 
 // exp2 on the special-function unit (ex2.approx.ftz.f32: rel. error ~2^-22).
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -121,12 +110,6 @@ __device__ __forceinline__ void fence_mbar_init() {
 
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-// Orders this thread's earlier (generic) observations of global memory before
-// its later async-proxy (bulk copy) reads of global memory.
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
@@ -197,9 +180,6 @@ __device__ __forceinline__ void bulk_commit() {
 }
 __device__ __forceinline__ void bulk_wait_all() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_wait_read_all() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 // Programmatic dependent launches. A kernel that may be followed by a dependent

@@ -190,13 +190,9 @@ __device__ __forceinline__ void advance(const Tc1Params &p, ItemAt &it) {
     ++it.unit;
     ++it.local;
   }
-  if (it.local >= p.upl) {  // d_local < upl: once, or once more by the carry
+  if (it.local >= p.upl) {  // once: d_local < upl, so local is at most 2 upl - 1 here
     it.local -= p.upl;
     ++it.layer;
-    if (it.local >= p.upl) {
-      it.local -= p.upl;
-      ++it.layer;
-    }
   }
 }
 
