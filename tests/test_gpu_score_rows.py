@@ -3,9 +3,11 @@ inside the kernel to 32, 64, 128 or 256 rows) and head dims (64, 128): votes and
 selection against the oracle at row counts on, below and above each padding
 step, prompts that end on, before and after a key tile, and units of one and
 several work items; the multi-layer call against the per-layer calls."""
+import numpy as np
 import pytest
 import torch
 
+from oracle import ripple_oracle as O
 from paper_2608_08684_gb300 import synth
 from tests import gpu_common as C
 
@@ -64,3 +66,25 @@ def test_layers_call_equals_per_layer_calls(lib, G, w, d, T):
     for l, r in enumerate(refs):
         assert torch.equal(idx[l], r["idx"].reshape(-1)), l
         assert torch.equal(k_out[l], r["k_out"]) and torch.equal(v_out[l], r["v_out"]), l
+
+
+# Votes against 64 bits. A logit is a sum of d exact products in fp32, off by at
+# most d 2^-24 sum |q_c k_c| (1e-4 in log2 units for these inputs, a few 1e-6 in
+# fact, as the terms' errors average out); an exponential adds 2^-22, a normaliser
+# the errors of its largest terms, and a vote's rows average again. So no vote is
+# off by more than 1e-5 of it (3e-6 seen) and all of them by more than 2e-6 in the
+# 2-norm (3e-7 seen, as with fp32 multiply-adds and exp2f in place of the tensor
+# cores and ex2).
+@pytest.mark.parametrize("G,w,d,T", [SHAPES[i] for i in (1, 2, 4, 5, 7, 9, 11, 12, 13)] + LONG)
+def test_votes_to_fp32_precision(lib, G, w, d, T):
+    wl = synth.WORKLOADS["tiny"].replace(
+        batch=1, n_q_heads=2 * G, n_kv_heads=2, head_dim=d, seq_len=T, window=w, dtype="bf16",
+        kv_dist="scaled_sinks", seed=520 + G + w + T)
+    q, k, v = (t.to(DEV) for t in C.layer_inputs(wl, 0, "cpu"))
+    out = C.run_compress(lib, wl, max(w + 1, T // 5), q, k, v)
+    for h in range(2):
+        q64, k64, _ = C.unit_f64(wl, q, k, v, 0, h)
+        ref = O.window_votes(q64, k64, 1.0 / np.sqrt(d))[0][:T - w]
+        err = np.abs(out["scores"][0, h].cpu().numpy().astype(np.float64) - ref)
+        assert np.linalg.norm(err) <= 2e-6 * np.linalg.norm(ref)
+        assert (err <= 1e-5 * ref).all(), (err / ref).max()
