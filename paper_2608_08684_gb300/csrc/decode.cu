@@ -1170,8 +1170,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
   const int n_ctrl = (kCtrlGroup - kCtrlItem) + p.L * units;
   if (blockIdx.x == 0)
     for (int i = tid; i < n_ctrl; i += kThreads) p.ctrl[kCtrlItem + i] = 0;
-  // Work list of this step from the current lengths (read once, before any
-  // CTA can advance them: that happens after every CTA has exited).
+  // Work list of this step from the current lengths (read once, before the last
+  // block can advance them: that happens once every CTA has counted itself as
+  // arrived, which it does after this).
   if (warp == 0) {
     const LayerPlan w = plan_layers(p, lane);
 #pragma unroll

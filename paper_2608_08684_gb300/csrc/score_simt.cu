@@ -12,11 +12,12 @@
 //
 // Keys and window rows lie in shared memory dim by dim, and a thread has 4 rows
 // x 8 keys of a 64 x 128 block in registers: three 16-byte shared loads for 16
-// packed FMAs, so that the FMA pipe is the bound: 16 layers of 8 units, 1192
-// tokens, 128 rows of d = 128 take 332 us with selection (60 TFLOP/s over the
-// two passes). One row x 16 keys a thread with a scalar load per FMA, three
-// launches a layer, took 1610 us. Few CTAs, as in a 512-token prompt, are bound
-// by latency: four layers 28.7 us, against 148 us with three launches each.
+// packed FMAs. Bound: shared memory (83% of its rate, the FMA pipe 45%): 16 layers
+// of 8 units, 1192 tokens, 128 rows of d = 128 take 323 us with selection, 31
+// TFLOP/s over the two passes; 32 layers of 8 units and 8192 tokens 38. One row x
+// 16 keys a thread with a scalar load per FMA, three launches a layer, took the
+// first 1610 us. Few CTAs, as in a 512-token prompt, are bound by latency: four
+// layers 24.6 us with selection, against 152 us with three launches each.
 #include <math.h>
 
 #include "common.cuh"

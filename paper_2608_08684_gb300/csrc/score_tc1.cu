@@ -3,13 +3,16 @@
 // the 5th-generation tensor cores. Row counts other than 32, 64 and 128 are
 // padded to the next of them with zero rows that no sum counts.
 //
-// Bound: board power for 128 rows of d = 128 in large calls (32 layers of 32
-// units, 32768 keys: 1370 W, the SM clock down to 1970 MHz, 70 us a layer), so
-// that schedules with the same reads, MMAs and exponentials take the same
-// time; else the epilogue's arithmetic (about 1350 cycles for 128 logits a
-// thread, two warps to an SM partition, the exponential unit 75% busy) and, for
-// few rows or d = 64, the MMA warp's issue of about 900 cycles a tile. Before
-// these kernels took every bf16 shape, 16 layers of 16 units, 6007 keys, d = 64
+// Bound, 128 rows of d = 128 in large calls (32 units a layer, 32768 keys: 70 us a
+// layer): the lock step of the two passes. All CTAs read a pass-1 item from DRAM
+// and then a pass-2 item from L2 together, a pattern whose bare stream takes 63 to
+// 68 us a layer, and no unit is saturated (DRAM 53% busy, tensor pipe 40%,
+// exponentials 41%, issue 39%). Board power, which such calls reach when they run
+// for long, costs 3%: 78.9 us a layer with selection at 1942 MHz and 1390 W, 76.7
+// in bursts at 2070 MHz. Else the epilogue's arithmetic (about 1350 cycles for 128
+// logits a thread, two warps to an SM partition) and, for few rows or d = 64, the
+// MMA warp's issue of about 900 cycles a tile. Before these kernels took every bf16
+// shape, 16 layers of 16 units, 6007 keys, d = 64
 // and 64 rows took 1917 us on the fp32 pipes; 105 us now, with selection.
 //
 // One persistent CTA per SM, item i on CTA i mod grid; in its step k a CTA
@@ -53,7 +56,7 @@
 // unit's sum. Bound: HBM, which brings the keys twice and the values once (a
 // CTA's item of keys is too large to stay in L2 until its second pass, and
 // smaller items pay a step's fixed cost more often): 64 units of 256 tiles,
-// 1.6 GB, take 297 us with selection, 5.6 TB/s.
+// 1.61 GB, take 298 us with selection, 5.4 TB/s.
 #include <cuda.h>
 #include <math.h>
 
@@ -473,10 +476,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int kTileBytes = C::TileBytes;
   // 128 rows: both epilogue warpgroups take every pass-2 tile, each for 64 of
   // its rows, whose normalisers a thread keeps in registers for the item. With a
-  // tile to a warpgroup every tile reads all of them from shared memory; at the
-  // power limit, where the 32k workload runs, those reads cost 2% (2624 -> 2570
-  // us). Not with padding rows, which would leave one warpgroup short of work
-  // (96 rows: 112 -> 115 us).
+  // tile to a warpgroup every tile reads all of them from shared memory, which cost
+  // 2% (32 layers of 32 units and 32768 keys 2624 -> 2570 us). Not with padding
+  // rows, which would leave one warpgroup short of work (96 rows: 112 -> 115 us).
   constexpr bool kSplit = RP == 128 && !kPad;
   const Tc1Params &p = lp.p;
   const int R = kPad ? p.R : RP;  // window rows
@@ -499,8 +501,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(&ms->q_empty, 1);
     for (int i = 0; i < C::NA; ++i) {
       mbar_init(&ms->acc_full[i], 1);
-      // kO: pass-2 tiles are released by all eight epilogue warps, pass-1
-      // tiles by the four of their warpgroup with two arrivals each
+      // kSplit (and kO): pass-2 tiles are released by all eight epilogue warps,
+      // pass-1 tiles by the four of their warpgroup with two arrivals each
       mbar_init(&ms->acc_empty[i], kSplit ? 8 : 4);
     }
     mbar_init(&ms->qs_full, 1);
@@ -1044,9 +1046,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (kO && st.n2 > 0) {
         // ---------------- kO: item k - kLag's partial O (both warpgroups:
-        // this thread's row, warpgroup wg's 64 dims), and the unit's output
-        // from its items' partials, summed in item order by the item that
-        // completes the unit
+        // this thread's row, warpgroup wg's 64 dims)
         const ItemAt &it = st.i2;
         const size_t prow = ((size_t)it.unit * p.n_ch + it.chunk) * 128 + r;
         if (warp_wait(&ms->o_full, oc & 1, ms, p.status)) {
