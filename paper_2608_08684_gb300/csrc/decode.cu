@@ -504,10 +504,11 @@ __device__ __forceinline__ void finish_item(const DecParams &p, DecSmem<Tin, D, 
     float M = -INFINITY;
 #pragma unroll
     for (int w = 0; w < C::RED; ++w) M = fmaxf(M, s.red_m[w][g]);
+    const float M_sub = M == -INFINITY ? 0.f : M;  // -infinity: scores of that alone
     float num = 0.f, den = 0.f;
 #pragma unroll
     for (int w = 0; w < C::RED; ++w) {
-      const float wgt = fast_exp2(s.red_m[w][g] - M);  // M is finite: some warp had a row
+      const float wgt = fast_exp2(s.red_m[w][g] - M_sub);
       num += wgt * s.red_o[w][g * C::RED_PITCH + e % D];
       den += wgt * s.red_l[w][g];
     }
@@ -552,13 +553,14 @@ __device__ __forceinline__ void finish_item(const DecParams &p, DecSmem<Tin, D, 
             float Mn = M;
 #pragma unroll
             for (int c = 0; c < kComb; ++c) Mn = fmaxf(Mn, ml[c].x);
-            const float a = fast_exp2(M - Mn);  // Mn is finite: every item has rows
+            const float M_sub = Mn == -INFINITY ? 0.f : Mn;
+            const float a = fast_exp2(M - M_sub);
             num *= a;
             den *= a;
             M = Mn;
 #pragma unroll
             for (int c = 0; c < kComb; ++c) {
-              const float wgt = fast_exp2(ml[c].x - M);
+              const float wgt = fast_exp2(ml[c].x - M_sub);
               den += wgt * ml[c].y;
               num += wgt * o[c];
             }
@@ -651,7 +653,8 @@ __device__ __forceinline__ void consume(const DecParams &p, DecSmem<Tin, D, G> &
     float m_run = -INFINITY, l_run = 0.f;  // of head hq over this row group's rows
 
     // One sub-chunk of this warp's rows; kMask: some rows are past nrows
-    // (their index is clamped to a valid row and their probability is 0).
+    // (their index is clamped to a valid row; they count for nothing by their
+    // place, not by that row's score).
     auto rows_step = [&](const Tin *ks, const Tin *vs, int nrows, auto mask_tag) {
       constexpr bool kMask = decltype(mask_tag)::value;
       float2 d2[NIT][G];
@@ -710,12 +713,13 @@ __device__ __forceinline__ void consume(const DecParams &p, DecSmem<Tin, D, G> &
           for (int e = 0; e < DL / 2; ++e) acc[g][e] = __fmul2_rn(acc[g][e], make_float2(ag[g], ag[g]));
         m_run = mn;
       }
+      const float m_sub = m_run == -INFINITY ? 0.f : m_run;  // scores of -infinity alone
 #pragma unroll
       for (int t = 0; t < NIT; ++t) {
         const int row = rw0 + t * R + rg;
         const int rr = kMask ? min(row, nrows - 1) : row;
-        const float pt =
-            (!kMask || sc[t] > -INFINITY) ? fast_exp2(sc[t] - m_run) : 0.f;  // m_run is finite
+        const bool live = !kMask || row < nrows;
+        const float pt = live ? fast_exp2(sc[t] - m_sub) : 0.f;
         l_run += pt;
         float pg[G];
         all_gather<S, G>(pt, pg);
@@ -820,20 +824,21 @@ __device__ __forceinline__ void mma_16x8x16(float (&c)[4], uint32_t a0, uint32_t
 __device__ __forceinline__ uint32_t high_halves(float x0, float x1) {
   return __byte_perm(__float_as_uint(x0), __float_as_uint(x1), 0x7632);
 }
-// x less its bf16 part, at least 2^-125 (whose half is a normal value still).
-__device__ __forceinline__ float below_bf16(float x) {
-  return fmaxf(x - __uint_as_float(__float_as_uint(x) & 0xffff0000u), 0x1p-125f);
+// x less its bf16 part, at least `least`.
+__device__ __forceinline__ float below_bf16(float x, float least) {
+  return fmaxf(x - __uint_as_float(__float_as_uint(x) & 0xffff0000u), least);
 }
 // A pair of fp32 values >= 0 as h + m + 2 l, bf16 pairs: 24 bits of each, so
 // that products with bf16 values lose nothing against fp32. Each part is cut off,
-// not rounded, and m and l are never 0: no part of a positive probability times
-// an infinite value is a NaN or has the other sign (with rounded parts every
-// output of a column with an infinite value was NaN).
+// not rounded, and m and l are at least the smallest bf16 value, 2^-133: no part
+// of a positive probability times an infinite value is a NaN or has the other
+// sign (with rounded parts every output of a column with an infinite value was
+// NaN), and a finite value v comes out at most 2^-131 |v| too large.
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t &h, uint32_t &m, uint32_t &l) {
   h = high_halves(x0, x1);
-  const float r0 = below_bf16(x0), r1 = below_bf16(x1);
+  const float r0 = below_bf16(x0, 0x1p-133f), r1 = below_bf16(x1, 0x1p-133f);
   m = high_halves(r0, r1);
-  l = high_halves(0.5f * below_bf16(r0), 0.5f * below_bf16(r1));
+  l = high_halves(0.5f * below_bf16(r0, 0x1p-132f), 0.5f * below_bf16(r1, 0x1p-132f));
 }
 
 // The compute warps of a bf16 step. Per 16 cache rows (two blocks of 8 keys):
@@ -935,17 +940,16 @@ __device__ __forceinline__ void consume_mma(const DecParams &p,
       }
       // this lane's keys: chunk 2t + e, row r + i
       float x[2][2];
+      bool live[2][2];
       uint32_t vmask[2];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         vmask[i] = 0xffffffffu;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          x[i][e] = sc[i][e] * p.scale2;
-          if (kMask && (2 * t + e) * C::CHUNK_ROWS + r + i >= nrows) {
-            x[i][e] = -INFINITY;
-            vmask[i] &= e ? 0x0000ffffu : 0xffff0000u;
-          }
+          live[i][e] = !kMask || (2 * t + e) * C::CHUNK_ROWS + r + i < nrows;
+          x[i][e] = live[i][e] ? sc[i][e] * p.scale2 : -INFINITY;
+          if (!live[i][e]) vmask[i] &= e ? 0x0000ffffu : 0xffff0000u;
         }
       }
       const float mb = fmaxf(fmaxf(x[0][0], x[0][1]), fmaxf(x[1][0], x[1][1]));
@@ -961,14 +965,21 @@ __device__ __forceinline__ void consume_mma(const DecParams &p,
         }
         __syncwarp();
       }
+      // a row past the cached ones counts for nothing by its place, not by its
+      // score, so that a NaN score of a cached row reaches the output; scores of
+      // -infinity alone leave no finite maximum; and the fused multiply-add, which
+      // leaves out the rounding of the score, must not meet a maximum whose own
+      // rounding is a large part of 1
+      const float m_sub = m_run == -INFINITY ? 0.f : m_run;
+      const bool rounded = fabsf(m_sub) >= 65536.f;
       uint32_t hi[2], mi[2], lo[2];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         float pt[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          pt[e] = (!kMask || x[i][e] > -INFINITY)
-                      ? fast_exp2(fmaf(sc[i][e], p.scale2, -m_run)) : 0.f;
+          const float y = rounded ? x[i][e] - m_sub : fmaf(sc[i][e], p.scale2, -m_sub);
+          pt[e] = live[i][e] ? fast_exp2(y) : 0.f;
           l_run += pt[e];
         }
         split3(pt[0], pt[1], hi[i], mi[i], lo[i]);

@@ -1,7 +1,8 @@
 """bf16 decode on mma.sync: cache lengths around the edges of a 16-row warp step,
 of a 4 KB chunk, of a sub-chunk and of a work item, for every group size and
 head dim, against the oracle to the decode precision bound; rows past the
-cached ones never count, whatever shared memory holds there."""
+cached ones never count, whatever shared memory holds there. Scores and values
+that are not finite, on fp32 caches as well."""
 import numpy as np
 import pytest
 import torch
@@ -109,3 +110,41 @@ def _zero_cols(got, bad, G):
     for h in range(2):
         got[:, 0, h * G:(h + 1) * G, np.isinf(bad[h])] = 0.0
     return got
+
+
+@pytest.mark.parametrize("G,d,dtype", [(1, 64, "bf16"), (4, 128, "bf16"), (8, 64, "bf16"),
+                                       (8, 128, "bf16"), (2, 64, "f32"), (8, 128, "f32")])
+def test_scores_that_are_not_finite_or_huge(lib, G, d, dtype):
+    # Three groups, in caches of which most end inside a sub-chunk: a NaN in a key
+    # makes the group's outputs NaN (a row counts for nothing by its place past the
+    # cached ones, not by its score); keys whose score is -infinity, a first row and
+    # a whole run of them, count for nothing; a score so large that its rounding
+    # alone is many powers of two takes all the weight.
+    wl = synth.WORKLOADS["tiny"].replace(n_layers=5, batch=1, n_q_heads=3 * G, n_kv_heads=3,
+                                         head_dim=d, dtype=dtype, seed=790 + G + d)
+    lens0 = [2, 40, 256, 700, 5000]
+    kc, vc = zip(*[synth.decode_caches(wl, i, n + 2) for i, n in enumerate(lens0)])
+    s0 = Session(lib, wl, range(5), [t.shape[2] for t in kc], lens0, kc, vc)
+    q, kn, vn = synth.decode_inputs(wl, 0)
+    q[:, :, G:2 * G, 5] = q[:, :, G:2 * G, 5].abs() + 1
+    q[:, :, 2 * G:, 9] = 2.0
+    kept = [list(range(n)) for n in lens0]
+    for i, n in enumerate(lens0):
+        kc[i][0, 0, n - 1, 3] = float("nan")
+        gone = range(0, 1) if n == 2 else range(0, n // 2)
+        kc[i][0, 1, list(gone), 5] = -float("inf")
+        kept[i] = [r for r in range(n) if r not in gone]
+        kc[i][0, 2, n // 2, 9] = 1e30
+    s0.k = [t.to(DEV) for t in kc]
+    s0.tables = lib.DecodeTables(s0.k, s0.v)
+    got = s0.step(q, kn, vn)
+    assert int(s0.status.item()) == 0
+    for i, n in enumerate(lens0):
+        assert np.isnan(got[i, 0, :G]).all(), i
+        rows = kept[i]
+        rk = np.vstack([synth.to_f64(kc[i][0, 1, rows]), synth.to_f64(kn[i, 0, 1])[None]])
+        rv = np.vstack([synth.to_f64(vc[i][0, 1, rows]), synth.to_f64(vn[i, 0, 1])[None]])
+        ref = O.decode_attention(synth.to_f64(q[i, 0, G:2 * G]), rk, rv, 1.0 / np.sqrt(d))
+        C.assert_decode_close(got[i, 0, G:2 * G], ref)
+        np.testing.assert_array_equal(
+            got[i, 0, 2 * G:], np.tile(vc[i][0, 2, n // 2].float().numpy(), (G, 1)))
