@@ -548,7 +548,10 @@ __device__ __forceinline__ void finish_item(const DecParams &p, DecSmem<Tin, D, 
               const size_t i = ib + min(c0 + c, f.nch - 1);
               ml[c] = __ldcg(&p.ws_ml[i * G + g]);
               o[c] = __ldcg(&p.ws_o[i * G * D + e]);
-              if (c0 + c >= f.nch) ml[c] = make_float2(-INFINITY, 0.f);
+              if (c0 + c >= f.nch) {  // no partial: nothing for its weight of 0 to scale
+                ml[c] = make_float2(-INFINITY, 0.f);
+                o[c] = 0.f;
+              }
             }
             float Mn = M;
 #pragma unroll
@@ -727,6 +730,10 @@ __device__ __forceinline__ void consume(const DecParams &p, DecSmem<Tin, D, G> &
         for (int k = 0; k < PPL; ++k) {
           float2 vp[PE / 2];
           load_pairs<PE / 2>(vs + (size_t)rr * D + (sl + k * S) * PE, vp);
+          if (!live) {  // 0 times an infinite value of the row in its place is NaN
+#pragma unroll
+            for (int e = 0; e < PE / 2; ++e) vp[e] = make_float2(0.f, 0.f);
+          }
 #pragma unroll
           for (int g = 0; g < G; ++g)
 #pragma unroll

@@ -69,14 +69,16 @@ def test_rows_past_the_cache_never_count(lib, G, d):
     _check(wl, lens0, kc, vc, q, kn, vn, got, [1, 2], [(0, 0), (41, 2), (79, 3)])
 
 
-@pytest.mark.parametrize("G,d", [(1, 64), (2, 128), (4, 128), (8, 64), (8, 128)])
-def test_infinite_values_stay_infinite(lib, G, d):
+@pytest.mark.parametrize("G,d,dtype", [(1, 64, "bf16"), (2, 128, "bf16"), (4, 128, "bf16"),
+                                       (8, 64, "bf16"), (8, 128, "bf16"), (1, 64, "f32"),
+                                       (4, 128, "f32"), (8, 64, "f32")])
+def test_infinite_values_stay_infinite(lib, G, d, dtype):
     # A probability is positive, so a column that holds an infinite value has an
     # infinite output, whatever parts the probability is split into (1, of one
     # bf16 part, and the largest of a row included); the other columns stay as
     # they are.
     wl = synth.WORKLOADS["tiny"].replace(n_layers=4, batch=1, n_q_heads=2 * G, n_kv_heads=2,
-                                         head_dim=d, dtype="bf16", seed=760 + G + d)
+                                         head_dim=d, dtype=dtype, seed=760 + G + d)
     lens0 = [1, 40, 300, 5000]
     kc, vc = zip(*[synth.decode_caches(wl, i, n + 2) for i, n in enumerate(lens0)])
     for i, n in enumerate(lens0):
